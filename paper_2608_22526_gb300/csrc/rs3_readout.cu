@@ -319,137 +319,6 @@ __global__ void __launch_bounds__(PLAN_THREADS) k_plan(ReadoutArgs a)
 }
 
 // ---------------------------------------------------------------------------
-// k_readout_simt: CUDA-core flash readout (fp32 path; any dtype)
-// ---------------------------------------------------------------------------
-// One CTA per work item of BM = 32 query rows.  A row is owned by TPR = d/16
-// threads, each holding 16 dimensions of q~ and of the output accumulator.
-// Keys are staged 32 at a time in shared memory as fp32.
-constexpr int SIMT_BM = 32;
-constexpr int SIMT_BN = 32;
-
-template <typename T>
-__global__ void __launch_bounds__(512) k_readout_simt(ReadoutArgs a)
-{
-    pdl_wait();
-    extern __shared__ __align__(16) float sm[];
-    const int d = a.d;
-    const int TPR = d / 16;
-    float *sK = sm;                      // [SIMT_BN][d]
-    float *sV = sm + SIMT_BN * d;        // [SIMT_BN][d]
-    const int it_end = a.cta_items[2 * blockIdx.x + 1];
-    for (int it = a.cta_items[2 * blockIdx.x]; it < it_end; ++it) {
-        const WorkItem w = a.items[it];
-        const RangeSet rs = a.ranges[w.u];
-        const int r = threadIdx.x / TPR;
-        const int part = threadIdx.x % TPR;
-        const int j = w.qt * SIMT_BM + r;
-        const bool valid = j < rs.cnt;
-        const int g = a.unit_group[w.u];
-        if (g < 0 || g >= a.G) {                 // uniform over the CTA
-            if (threadIdx.x == 0) latch_status(a.status, RS3_EINVAL);
-            continue;
-        }
-        int cell = 0;
-        if (valid) cell = a.idx[(int64_t)w.u * a.k_max + j];
-        if (cell < 0 || cell >= a.mn) cell = 0;
-        const int c0 = w.h * d + part * 16;
-        float qv[16];
-        {
-            const T *qr = static_cast<const T *>(a.q) + ((int64_t)g * a.mn + cell) * a.D + c0;
-            load16(qr, qv);
-            if (a.rope) {
-                const float *f = a.rope + ((int64_t)cell * (d / 2) + part * 8) * 2;
-#pragma unroll
-                for (int p = 0; p < 8; ++p) {
-                    const float cs = f[2 * p], sn = f[2 * p + 1];
-                    const float x0 = qv[2 * p], x1 = qv[2 * p + 1];
-                    qv[2 * p] = x0 * cs - x1 * sn;
-                    qv[2 * p + 1] = x0 * sn + x1 * cs;
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < 16; ++k) qv[k] *= a.scale_log2;
-        }
-        float o[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) o[k] = 0.f;
-        float mrun = -INFINITY, lrun = 0.f;
-        const T *Kb = static_cast<const T *>(a.k_store) + (int64_t)w.u * a.rows_per_unit * a.D;
-        const T *Vb = static_cast<const T *>(a.v_store) + (int64_t)w.u * a.rows_per_unit * a.D;
-        for (int t = w.tile_begin; t < w.tile_end; ++t) {
-            int64_t row0;
-            int nvalid;
-            tile_rows(rs, t, SIMT_BN, row0, nvalid);
-            if (nvalid <= 0) continue;           // uniform over the CTA
-            __syncthreads();
-            // stage keys / values of this head as fp32
-            const int vec_per_row = d / 4;
-            for (int e = threadIdx.x; e < SIMT_BN * vec_per_row; e += blockDim.x) {
-                const int kk = e / vec_per_row, c4 = (e % vec_per_row) * 4;
-                float4 kv = make_float4(0.f, 0.f, 0.f, 0.f), vv = kv;
-                if (kk < nvalid) {
-                    kv = load4(Kb + (row0 + kk) * a.D + w.h * d + c4);
-                    vv = load4(Vb + (row0 + kk) * a.D + w.h * d + c4);
-                }
-                *reinterpret_cast<float4 *>(sK + kk * d + c4) = kv;
-                *reinterpret_cast<float4 *>(sV + kk * d + c4) = vv;
-            }
-            __syncthreads();
-            float s[SIMT_BN];
-#pragma unroll
-            for (int kk = 0; kk < SIMT_BN; ++kk) {
-                const float *kr = sK + kk * d + part * 16;
-                float acc = 0.f;
-#pragma unroll
-                for (int k = 0; k < 16; ++k) acc = fmaf(qv[k], kr[k], acc);
-                s[kk] = acc;
-            }
-            for (int off = TPR >> 1; off >= 1; off >>= 1) {
-#pragma unroll
-                for (int kk = 0; kk < SIMT_BN; ++kk) s[kk] += __shfl_xor_sync(0xffffffffu, s[kk], off);
-            }
-            float mt = -INFINITY;
-#pragma unroll
-            for (int kk = 0; kk < SIMT_BN; ++kk) {
-                if (kk >= nvalid) s[kk] = -INFINITY;
-                mt = fmaxf(mt, s[kk]);
-            }
-            const float mnew = fmaxf(mrun, mt);
-            const float alpha = exp2f(mrun - mnew);
-            lrun *= alpha;
-#pragma unroll
-            for (int k = 0; k < 16; ++k) o[k] *= alpha;
-#pragma unroll
-            for (int kk = 0; kk < SIMT_BN; ++kk) {
-                const float p = exp2f(s[kk] - mnew);
-                lrun += p;
-                const float *vr = sV + kk * d + part * 16;
-#pragma unroll
-                for (int k = 0; k < 16; ++k) o[k] = fmaf(p, vr[k], o[k]);
-            }
-            mrun = mnew;
-        }
-        if (valid) {
-            if (w.slot < 0) {
-                const float inv = lrun > 0.f ? 1.f / lrun : 0.f;
-#pragma unroll
-                for (int k = 0; k < 16; ++k) o[k] *= inv;
-                store_out16<T>(a, w.u, cell, c0, o);
-            } else {
-                float *po = a.part_o + ((int64_t)w.slot * a.BM + r) * d + part * 16;
-#pragma unroll
-                for (int k = 0; k < 16; k += 4)
-                    *reinterpret_cast<float4 *>(po + k) = make_float4(o[k], o[k + 1], o[k + 2], o[k + 3]);
-                if (part == 0) {
-                    float2 *pm = reinterpret_cast<float2 *>(a.part_ml) + (int64_t)w.slot * a.BM + r;
-                    *pm = make_float2(mrun, lrun);
-                }
-            }
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
 // k_combine: log-sum-exp merge of split-KV partials, then the scatter
 // ---------------------------------------------------------------------------
 // A warp takes one output row: the row's splits' (m, l) pairs give M = max m
@@ -460,45 +329,14 @@ __global__ void __launch_bounds__(512) k_readout_simt(ReadoutArgs a)
 // otherwise one warp does the whole row (lanes striding the columns four at a
 // time), so the loads of the row's entry, cell and (m, l) pairs are not
 // repeated per chunk.
-template <typename T, int E>
-__device__ __forceinline__ void store_out_e(const ReadoutArgs &a, int u, int cell, int c, const float *o);
-
-template <>
-__device__ __forceinline__ void store_out_e<float, 1>(const ReadoutArgs &a, int u, int cell, int c, const float *o)
+__device__ __forceinline__ void store_out1(const float *res, float *out, int64_t off, float o)
 {
-    const int64_t off = ((int64_t)u * a.mn + cell) * a.D + c;
-    const float r = a.residual ? static_cast<const float *>(a.residual)[off] : 0.f;
-    static_cast<float *>(a.out)[off] = r + o[0];
+    out[off] = (res ? res[off] : 0.f) + o;
 }
 
-template <>
-__device__ __forceinline__ void store_out_e<float, 2>(const ReadoutArgs &a, int u, int cell, int c, const float *o)
+__device__ __forceinline__ void store_out1(const uint16_t *res, uint16_t *out, int64_t off, float o)
 {
-    const int64_t off = ((int64_t)u * a.mn + cell) * a.D + c;
-    float2 r = make_float2(0.f, 0.f);
-    if (a.residual) r = *reinterpret_cast<const float2 *>(static_cast<const float *>(a.residual) + off);
-    *reinterpret_cast<float2 *>(static_cast<float *>(a.out) + off) = make_float2(r.x + o[0], r.y + o[1]);
-}
-
-template <>
-__device__ __forceinline__ void store_out_e<uint16_t, 1>(const ReadoutArgs &a, int u, int cell, int c, const float *o)
-{
-    const int64_t off = ((int64_t)u * a.mn + cell) * a.D + c;
-    const float r = a.residual ? bf16_bits_to_float(static_cast<const uint16_t *>(a.residual)[off]) : 0.f;
-    static_cast<uint16_t *>(a.out)[off] = float_to_bf16_bits(r + o[0]);
-}
-
-template <>
-__device__ __forceinline__ void store_out_e<uint16_t, 2>(const ReadoutArgs &a, int u, int cell, int c, const float *o)
-{
-    const int64_t off = ((int64_t)u * a.mn + cell) * a.D + c;
-    float r0 = 0.f, r1 = 0.f;
-    if (a.residual) {
-        const uint32_t x = *reinterpret_cast<const uint32_t *>(static_cast<const uint16_t *>(a.residual) + off);
-        r0 = __uint_as_float(x << 16);
-        r1 = __uint_as_float(x & 0xffff0000u);
-    }
-    *reinterpret_cast<uint32_t *>(static_cast<uint16_t *>(a.out) + off) = pack_bf16x2(r0 + o[0], r1 + o[1]);
+    out[off] = float_to_bf16_bits((res ? bf16_bits_to_float(res[off]) : 0.f) + o);
 }
 
 template <typename T, int E>
@@ -630,7 +468,11 @@ __global__ void __launch_bounds__(256) k_combine(ReadoutArgs a)
 #undef SLOT_REL
 #pragma unroll
         for (int e = 0; e < E; ++e) acc[e] *= inv;
-        store_out_e<T, E>(a, c.u, cell, c.h * d + col, acc);
+        if constexpr (E == 2)
+            store_out2<T>(a, c.u, cell, c.h * d + col, acc);
+        else
+            store_out1(static_cast<const T *>(a.residual), static_cast<T *>(a.out),
+                       ((int64_t)c.u * a.mn + cell) * a.D + c.h * d + col, acc[0]);
     }
 }
 
@@ -690,10 +532,10 @@ ReadoutPath choose_readout_path(rs3_dtype dtype, int d)
         p.BN = rs3_tc_block_n(d);
         p.grid = n_sm;                 // one persistent CTA per SM
     } else {
+        int ctas;
         p.kind = 0;
-        p.BM = SIMT_BM;
-        p.BN = SIMT_BN;
-        p.grid = 4 * n_sm;
+        rs3_simt_tile(d, p.BM, p.BN, ctas);
+        p.grid = ctas * n_sm;
     }
     return p;
 }
@@ -756,10 +598,12 @@ rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, in
     a->BM = p.BM;
     a->BN = p.BN;
     a->n_sm = rs3_sm_count();
-    a->min_chunk = p.kind == 1 ? 2 : 4;
+    a->min_chunk = 2;
     // start-up cost of a piece in tile slots: on the tensor-core path a
-    // sweep of 4..32 over the 1- and 8-object sequences was best at 8..16
-    a->plan_ov = p.kind == 1 ? 12 : 1;
+    // sweep of 4..32 over the 1- and 8-object sequences was best at 8..16; the
+    // CUDA-core path is flat over 1..4.  A slice of at least two slots: four
+    // left a 32 x 32 fp32 frame on half the CTAs (68 us against 61)
+    a->plan_ov = p.kind == 1 ? 12 : 2;
     a->max_slots = L.max_slots;
     a->max_items = L.max_items;
     a->grid_ctas = p.grid;
@@ -804,17 +648,7 @@ rs3_status launch_plan(const ReadoutArgs &a, cudaStream_t st, rs3_dtype dtype)
 rs3_status launch_run(const ReadoutArgs &a, const ReadoutPath &p, rs3_dtype dtype, cudaStream_t st)
 {
     if (p.kind == 1) return rs3_launch_tc_readout(a, st);
-    const size_t smem = (size_t)2 * SIMT_BN * a.d * sizeof(float);
-    const int threads = 2 * a.d;
-    const int64_t blocks = a.grid_ctas;
-    if (rs3_kernel_smem(dtype == RS3_BF16 ? (const void *)k_readout_simt<uint16_t>
-                                          : (const void *)k_readout_simt<float>, smem) != RS3_OK)
-        return RS3_ECUDA;
-    if (dtype == RS3_BF16)
-        launch_pdl(k_readout_simt<uint16_t>, dim3((unsigned)blocks), dim3(threads), smem, st, a);
-    else
-        launch_pdl(k_readout_simt<float>, dim3((unsigned)blocks), dim3(threads), smem, st, a);
-    return cudaGetLastError() == cudaSuccess ? RS3_OK : RS3_ECUDA;
+    return rs3_launch_simt_readout(a, dtype, st);
 }
 
 // merge of the split-KV partials and their scatter

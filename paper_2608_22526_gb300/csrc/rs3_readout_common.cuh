@@ -48,6 +48,9 @@ ReadoutPath choose_readout_path(rs3_dtype dtype, int d);
 bool rs3_tc_supported(int d);
 int rs3_tc_block_n(int d);
 rs3_status rs3_launch_tc_readout(const ReadoutArgs &a, cudaStream_t st);
+// CUDA-core path: rows and keys of a tile and resident CTAs per SM, for a head width
+void rs3_simt_tile(int d, int &bm, int &bn, int &ctas_per_sm);
+rs3_status rs3_launch_simt_readout(const ReadoutArgs &a, rs3_dtype dtype, cudaStream_t st);
 rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, int H, int d,
                                const int32_t *unit_group, const int32_t *idx, const int32_t *count,
                                int k_max, const rs3_bank *bank, const float *rope,
@@ -102,28 +105,6 @@ __device__ __forceinline__ float4 load4(const uint16_t *p)
                        __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
 }
 
-__device__ __forceinline__ void load16(const float *p, float *o)
-{
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(p) + k);
-        o[4 * k] = v.x; o[4 * k + 1] = v.y; o[4 * k + 2] = v.z; o[4 * k + 3] = v.w;
-    }
-}
-__device__ __forceinline__ void load16(const uint16_t *p, float *o)
-{
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p) + k);
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            o[8 * k + 2 * e] = __uint_as_float(w[e] << 16);
-            o[8 * k + 2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
-        }
-    }
-}
-
 // Two fp32 values to a bf16 pair (round to nearest even), `lo` in the low half;
 // one cvt instruction (the per-value conversions cost about three times more).
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
@@ -133,44 +114,31 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
     return r;
 }
 
-// out[u][cell][c0 .. c0+15] = residual[...] + o (one rounding to T)
+// out[u][cell][c .. c+1] (store_out2) or [c .. c+3] (store_out4) =
+// residual[...] + o, rounded once to T
 template <typename T>
-__device__ __forceinline__ void store_out16(const ReadoutArgs &a, int u, int cell, int c0, const float *o);
+__device__ __forceinline__ void store_out2(const ReadoutArgs &a, int u, int cell, int c, const float *o);
 
 template <>
-__device__ __forceinline__ void store_out16<float>(const ReadoutArgs &a, int u, int cell, int c0, const float *o)
+__device__ __forceinline__ void store_out2<float>(const ReadoutArgs &a, int u, int cell, int c, const float *o)
 {
-    const int64_t off = ((int64_t)u * a.mn + cell) * a.D + c0;
-    float r[16];
-    if (a.residual) load16(static_cast<const float *>(a.residual) + off, r);
-    else {
-#pragma unroll
-        for (int k = 0; k < 16; ++k) r[k] = 0.f;
-    }
-    float4 *dst = reinterpret_cast<float4 *>(static_cast<float *>(a.out) + off);
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-        dst[k] = make_float4(r[4 * k] + o[4 * k], r[4 * k + 1] + o[4 * k + 1], r[4 * k + 2] + o[4 * k + 2],
-                             r[4 * k + 3] + o[4 * k + 3]);
+    const int64_t off = ((int64_t)u * a.mn + cell) * a.D + c;
+    float2 r = make_float2(0.f, 0.f);
+    if (a.residual) r = *reinterpret_cast<const float2 *>(static_cast<const float *>(a.residual) + off);
+    *reinterpret_cast<float2 *>(static_cast<float *>(a.out) + off) = make_float2(r.x + o[0], r.y + o[1]);
 }
 
 template <>
-__device__ __forceinline__ void store_out16<uint16_t>(const ReadoutArgs &a, int u, int cell, int c0, const float *o)
+__device__ __forceinline__ void store_out2<uint16_t>(const ReadoutArgs &a, int u, int cell, int c, const float *o)
 {
-    const int64_t off = ((int64_t)u * a.mn + cell) * a.D + c0;
-    float r[16];
-    if (a.residual) load16(static_cast<const uint16_t *>(a.residual) + off, r);
-    else {
-#pragma unroll
-        for (int k = 0; k < 16; ++k) r[k] = 0.f;
+    const int64_t off = ((int64_t)u * a.mn + cell) * a.D + c;
+    float r0 = 0.f, r1 = 0.f;
+    if (a.residual) {
+        const uint32_t x = *reinterpret_cast<const uint32_t *>(static_cast<const uint16_t *>(a.residual) + off);
+        r0 = __uint_as_float(x << 16);
+        r1 = __uint_as_float(x & 0xffff0000u);
     }
-    uint4 *dst = reinterpret_cast<uint4 *>(static_cast<uint16_t *>(a.out) + off);
-#pragma unroll
-    for (int k = 0; k < 2; ++k)
-        dst[k] = make_uint4(pack_bf16x2(r[8 * k] + o[8 * k], r[8 * k + 1] + o[8 * k + 1]),
-                            pack_bf16x2(r[8 * k + 2] + o[8 * k + 2], r[8 * k + 3] + o[8 * k + 3]),
-                            pack_bf16x2(r[8 * k + 4] + o[8 * k + 4], r[8 * k + 5] + o[8 * k + 5]),
-                            pack_bf16x2(r[8 * k + 6] + o[8 * k + 6], r[8 * k + 7] + o[8 * k + 7]));
+    *reinterpret_cast<uint32_t *>(static_cast<uint16_t *>(a.out) + off) = pack_bf16x2(r0 + o[0], r1 + o[1]);
 }
 
 template <typename T>

@@ -319,6 +319,13 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
     return d;
 }
 
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 // Named barrier `id` over `nthreads` threads (a multiple of 32) that also
 // ANDs a predicate across them: every participant gets the same answer.
 __device__ __forceinline__ bool bar_and(uint32_t id, uint32_t nthreads, bool pred)

@@ -1,0 +1,123 @@
+"""The readout at the edges of its tiles: kept counts and bank lengths around
+the query and key tiles of each kernel (CUDA cores: 32 keys, 64 or 128 rows;
+tensor cores: 64 or 128 keys, 128 rows or pairs of that), every head width,
+ring pieces and pointer rows that leave partial tiles, against the fp64 oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as orc
+from paper_2608_22526_gb300 import rs3, synth
+from tests._harness import F32_REL, bf16_ulp, to_dev, to_host, widen
+
+pytestmark = pytest.mark.gpu
+
+
+def _draw(rng, dtype, shape, scale=1.0):
+    x = rng.standard_normal(shape, dtype=np.float32) * np.float32(scale)
+    return synth.f32_to_bf16_bits(x) if dtype == "bf16" else x
+
+
+def _check(dtype, got, exact, vmax, rope, what):
+    """bf16: half a step of the result for its one rounding, plus 2^-9 of the
+    greatest value for the probabilities' rounding (sum p |v| / l <= max |v|) and
+    as much again for the sums; with RoPE the rotated queries are rounded too,
+    which moves a score of the size drawn here by about 2^-9, and p by as much.
+    fp32: the relative bound of the other parity tests."""
+    err = np.abs(widen(got, dtype) - exact)
+    if not err.size:
+        return
+    if dtype == "bf16":
+        excess = float(np.max(err - 0.5 * bf16_ulp(exact)))
+        assert excess <= (2.0 if rope else 1.0) * 2.0 ** -8 * vmax, f"{what}: {excess} beyond one rounding"
+    else:
+        assert float(err.max()) <= F32_REL * max(float(np.abs(exact).max()), 1e-30), f"{what}: {err.max()}"
+
+
+def _case(dtype, H, d, counts, rows, n_ptr=0, rope=False, sharp=1.0, ramp=0.0, seed=0):
+    """One group, a unit per (count, rows) pair: `rows` bank rows in two ring
+    frames, then n_ptr pointer rows.  ramp > 0 makes later keys score higher,
+    so that a row's softmax reference has to move."""
+    rng = np.random.default_rng([seed, d, len(counts)])
+    U, m, n = len(counts), 24, 25
+    mn, D = m * n, H * d
+    k_max = max(counts)
+    bank = rs3.Bank(U, H, d, dtype, mn, 0, 2, 2 * mn, 2, n_ptr)
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    q = _draw(rng, dtype, (1, mn, D), sharp)
+    K, V = [[] for _ in range(U)], [[] for _ in range(U)]
+    for f in range(2):
+        k, v = _draw(rng, dtype, (U, mn, D)), _draw(rng, dtype, (U, mn, D))
+        if ramp:
+            x = widen(k, dtype) + ramp * (f * mn + np.arange(mn))[None, :, None] * widen(q, dtype)[:, :1] / mn
+            k = synth.f32_to_bf16_bits(x.astype(np.float32)) if dtype == "bf16" else x.astype(np.float32)
+        mask = np.zeros((U, mn), np.uint8)
+        for u in range(U):
+            r = rows[u] // 2 + (rows[u] % 2 if f == 0 else 0)
+            mask[u, np.sort(rng.permutation(mn)[:r])] = 1
+            K[u].append(k[u][mask[u] == 1])
+            V[u].append(v[u][mask[u] == 1])
+        rs3.rs3_bank_commit(bank, to_dev(k), to_dev(v), to_dev(mask), 0, st)
+    if n_ptr:
+        kp, vp = _draw(rng, dtype, (U, n_ptr, D)), _draw(rng, dtype, (U, n_ptr, D))
+        rs3.rs3_bank_set_pointers(bank, to_dev(kp), to_dev(vp), st)
+        for u in range(U):
+            K[u].append(kp[u])
+            V[u].append(vp[u])
+    idx = np.zeros((U, k_max), np.int32)
+    for u, c in enumerate(counts):
+        idx[u, :c] = np.sort(rng.permutation(mn)[:c])
+    res = _draw(rng, dtype, (U, mn, D))
+    tab = rng.uniform(0, 6.28, (mn, d // 2)) if rope else None
+    table = np.ascontiguousarray(np.stack([np.cos(tab), np.sin(tab)], -1).astype(np.float32)) if rope else None
+    ws = torch.empty(rs3.rs3_readout_workspace_bytes(U, H, d, k_max, dtype), dtype=torch.uint8, device="cuda")
+    ug = torch.zeros(U, dtype=torch.int32, device="cuda")
+    cnt = torch.tensor(counts, dtype=torch.int32, device="cuda")
+    out = to_dev(res)
+    attn = torch.empty_like(out)
+    dev = to_dev(q), to_dev(idx), None if table is None else to_dev(table)
+
+    def call(r, o):
+        rs3.rs3_memory_readout(dev[0], dtype, 1, mn, H, d, ug, dev[1], cnt, k_max, bank, dev[2], r, o, 0.0, ws, st)
+
+    call(None, attn)
+    call(out, out)
+    attn, out = to_host(attn), to_host(out)
+    for u, c in enumerate(counts):
+        cells = idx[u, :c]
+        vmax, A = 1.0, np.zeros((c, D))
+        if c and rows[u] + n_ptr:
+            Ku, Vu = np.concatenate(K[u]), np.concatenate(V[u])
+            vmax = float(np.abs(widen(Vu, dtype)).max())
+            A = orc.readout(q[0], dtype, H, d, cells, Ku, Vu, dtype, rope=table)
+        what = f"unit {u}: {c} queries, {rows[u]} rows"
+        _check(dtype, attn[u][cells], A, vmax, rope, what)
+        _check(dtype, out[u][cells], widen(res[u][cells], dtype) + A, vmax, rope, what)
+        other = np.setdiff1d(np.arange(mn), cells)
+        assert np.all(widen(attn[u][other], dtype) == 0.0)
+        assert np.array_equal(out[u][other], res[u][other])
+    assert int(st.item()) == 0
+
+
+COUNTS = [1, 31, 33, 64, 65, 127, 128, 129, 255, 257, 513, 0]
+ROWS = [1, 2, 63, 64, 65, 31, 129, 255, 257, 513, 1100, 300]
+
+
+@pytest.mark.parametrize("dtype,H,d", [("f32", 1, 16), ("f32", 3, 32), ("f32", 2, 64), ("f32", 1, 128), ("f32", 1, 256),
+                                       ("bf16", 4, 16), ("bf16", 2, 32), ("bf16", 2, 64), ("bf16", 1, 128), ("bf16", 1, 256)])
+@pytest.mark.parametrize("rope,n_ptr", [(False, 0), (True, 7)])
+def test_tile_edges(dtype, H, d, rope, n_ptr):
+    _case(dtype, H, d, COUNTS, ROWS, n_ptr=n_ptr, rope=rope)
+
+
+@pytest.mark.parametrize("dtype,H,d", [("f32", 2, 64), ("f32", 1, 256), ("bf16", 2, 64), ("bf16", 1, 128), ("bf16", 1, 256)])
+def test_one_group_cut_over_every_slice(dtype, H, d):
+    """One unit with few queries: its keys are spread over all CTAs and merged."""
+    _case(dtype, H, d, [37], [1200])
+
+
+@pytest.mark.parametrize("dtype,H,d", [("f32", 1, 64), ("f32", 1, 128), ("bf16", 1, 64), ("bf16", 1, 128), ("bf16", 1, 256)])
+def test_rising_scores_move_the_reference(dtype, H, d):
+    """Scores that grow along the bank by far more than 2^8 between tiles: the
+    running reference moves and what is accumulated is rescaled."""
+    _case(dtype, H, d, [200, 3, 129, 64], [1200, 900, 700, 1000], ramp=3.0)
