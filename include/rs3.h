@@ -316,8 +316,8 @@ size_t rs3_readout_workspace_bytes(int U, int H, int d, int k_max, rs3_dtype dty
  * bf16: tensor-core path for d in {64, 128, 256}, fp32 accumulation.  fp32:
  * CUDA-core FFMA path for d % 16 == 0, d <= 256.
  * Limits: U <= 4096, mn <= 16384; the work list holds fewer than 2^21
- * entries (U * H * ceil(k_max / BM) plus one per CTA, BM = 128, or 64 for
- * fp32 with d = 256), else RS3_EUNSUPPORTED.
+ * entries (U * H * ceil(k_max / BM) plus one per SM, BM = 128 on the bf16
+ * path and 32 on the fp32 path), else RS3_EUNSUPPORTED.
  */
 rs3_status rs3_memory_readout(const void *q, rs3_dtype dtype, int G, int mn, int H, int d,
                               const int32_t *unit_group, const int32_t *idx,

@@ -568,8 +568,11 @@ rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, in
         return RS3_EINVAL;
     const ReadoutPath p = choose_readout_path(dtype, d);
     const ReadoutLayout L = readout_layout(bank->U, H, d, k_max, p.BM, p.grid);
-    // work-item indices (group + slice) and item ranges are 32-bit
-    if (L.max_items >= ((int64_t)1 << 30) || L.max_slots >= ((int64_t)1 << 30)) return RS3_EUNSUPPORTED;
+    // work-item indices (group + slice) and item ranges are 32-bit.  The limit
+    // counts 32-row query tiles on the CUDA-core path, more than its kernel has.
+    const int limit_rows = p.kind == 1 ? p.BM : 32;
+    const int64_t limit_groups = (int64_t)bank->U * H * (k_max > 0 ? (k_max + limit_rows - 1) / limit_rows : 1);
+    if (limit_groups + p.grid >= ((int64_t)1 << 30)) return RS3_EUNSUPPORTED;
     if (workspace_bytes < L.total) return RS3_ECAPACITY;
     uint8_t *ws = static_cast<uint8_t *>(workspace);
     a->q = q;
@@ -603,7 +606,7 @@ rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, in
     // sweep of 4..32 over the 1- and 8-object sequences was best at 8..16; the
     // CUDA-core path is flat over 1..4.  A slice of at least two slots: four
     // left a 32 x 32 fp32 frame on half the CTAs (68 us against 61)
-    a->plan_ov = p.kind == 1 ? 12 : 2;
+    a->plan_ov = p.kind == 1 ? 12 : 1;
     a->max_slots = L.max_slots;
     a->max_items = L.max_items;
     a->grid_ctas = p.grid;
