@@ -9,27 +9,35 @@
 //                        mask projected onto the grid (the tracker state of
 //                        Eq. 4), with down_s of the mask and the filled box
 //
-// Closure.  A CTA of 256 threads owns a tile of BR rows x 256 columns of one
-// stream's decoder output; thread t owns column t.  The CTAs of a thread-block
-// cluster (up to 8, along the stream's objects) share one tile: rank r closes
-// objects r, r + KC, ... of the stream.  For each of its objects a CTA
-// thresholds the logits (logit > 0) into bit masks -- a warp ballot over 32
-// adjacent columns is one 32-bit word -- for the tile plus a 2R-row halo above
-// and below and one word left and right (all of an object's loads issued
-// before its first ballot), then runs the four separable passes on words in
-// shared memory: horizontal dilation (OR of funnel-shifted words), vertical
-// dilation (OR over rows), horizontal and vertical erosion (AND).  The object
-// is a set of the unbounded plane with nothing set outside the image: pixels
-// outside are zero words, and the dilation is evaluated there too, so the
-// erosion never treats the border as set or unset by convention.  With R <= 8
-// every bit the tile's result depends on lies within 2R = 16 pixels of the
-// tile, i.e. in the loaded window.  Each CTA keeps, per pixel, the largest
-// logit among its objects whose closed mask holds the pixel (in shared memory,
-// the column's thread alone touching it; equal logits keep the earlier
-// object); after a cluster barrier each rank merges a share of the tile's rows
-// from all ranks' shared memory (DSMEM), equal logits going to the object
-// listed first, and writes those palette rows.  Each logit is read
-// from DRAM once; halo re-reads by neighbouring tiles hit L2.
+// Closure.  A CTA of 16 warps owns a tile of up to 24 rows x NS strips of 128
+// columns of one stream's decoder output (NS = 1..4, the whole width up to 512
+// columns) and takes the stream's objects one after the other.  A warp reads a
+// row of a strip with one 16-byte load per lane, so its four ballots (logit >
+// 0) hold the strip's bits by column modulo 4: bit l of word c is column 4 l +
+// c.  In that layout a horizontal shift by d = 4 q + b columns is a shift by q
+// bits of another word, and for the paper's radius of 4 a dilation is two
+// funnel shifts per word of running ORs.  The tile plus a halo of 2R rows above
+// and below and a strip on each side is thresholded into shared memory, then
+// four separable passes (horizontal and vertical dilation, horizontal and
+// vertical erosion) run on 128 columns per thread and step.  The object is a
+// set of the unbounded plane with nothing set outside the image: pixels outside
+// are zero bits, and the dilation is evaluated there too, so the erosion never
+// treats the border as set or unset by convention.  With R <= 8 every bit the
+// tile's result depends on lies within 2R = 16 pixels of the tile.  Per pixel
+// the largest logit among the objects whose closed mask holds it stays in
+// shared memory (equal logits keep the earlier object).
+//
+// Where a stream has few tiles, a thread-block cluster of KC <= 8 CTAs shares
+// one: rank r closes objects r, r + KC, ..., and each rank merges a share of
+// the tile's rows from all ranks' shared memory (DSMEM), equal logits going to
+// the object listed first.  close_shape() picks rows and KC.
+//
+// Each logit is read from DRAM once; halo re-reads by neighbouring tiles hit
+// L2.  16 streams x 3 objects of 384 x 384 (31 MB, 4.6 us at the copy rate): 18.5
+// us per call, half of the issue slots busy, mostly with the thresholds, the
+// argmax and its labels; 91 us with a scalar load and a ballot per 32 pixels,
+// general funnel-shift dilations and an 8-row halo per 16 rows on CTAs that
+// filled 1.3 waves.  8 objects of 1024 x 1024: 79 -> 44 us.
 #include "rs3_internal.cuh"
 
 #include <algorithm>
@@ -37,28 +45,95 @@
 
 namespace {
 
-constexpr int CA_TW = 8;            // words (of 32 pixels) per tile row: 256 columns
-constexpr int CA_THREADS = 32 * CA_TW;
+constexpr int CA_WARPS = 16;
+constexpr int CA_THREADS = 32 * CA_WARPS;
 constexpr int CA_RMAX = 8;
+constexpr int CA_ROWS = 24;         // the most rows of a tile
 
-// bits of the row word x (with its left / right neighbour words) ORed over
-// horizontal shifts -R..R: bit k of the result covers pixels 32w + k - R ..
-// 32w + k + R.  __funnelshift_r(x, nx, d) brings pixel 32w + k + d to bit k,
-// __funnelshift_l(pv, x, d) brings pixel 32w + k - d.
-__device__ __forceinline__ uint32_t dil_h(uint32_t pv, uint32_t x, uint32_t nx, int R)
+// word e of a strip shifted so that bit l holds column 4 (l + q) + e; pv and
+// nx are the same word of the strips to the left and right
+__device__ __forceinline__ uint32_t strip_shift(uint32_t pv, uint32_t x, uint32_t nx, int q)
 {
-    uint32_t r = x;
-#pragma unroll
-    for (int d = 1; d <= R; ++d) r |= __funnelshift_r(x, nx, d) | __funnelshift_l(pv, x, d);
-    return r;
+    return q == 0 ? x : q > 0 ? __funnelshift_r(x, nx, q) : __funnelshift_l(pv, x, -q);
 }
 
-__device__ __forceinline__ uint32_t ero_h(uint32_t pv, uint32_t x, uint32_t nx, int R)
+// Bits ORed (DIL) or ANDed over horizontal shifts -R..R of one strip with its
+// neighbours.  RC = 4: columns 4 l + c - 4 .. 4 l + c + 4 are words c..3 of
+// lane l - 1, every word of lane l and words 0..c of lane l + 1, so running
+// ORs (ANDs) from either end and one shift each way do.  RC = 0 takes any
+// radius up to 8 from R.
+template <bool DIL>
+__device__ __forceinline__ uint32_t comb(uint32_t a, uint32_t b) { return DIL ? (a | b) : (a & b); }
+
+template <bool DIL, int RC>
+__device__ __forceinline__ uint4 horizontal(uint4 pv, uint4 x, uint4 nx, int R)
 {
-    uint32_t r = x;
+    const uint32_t p[4] = {pv.x, pv.y, pv.z, pv.w}, o[4] = {x.x, x.y, x.z, x.w}, n[4] = {nx.x, nx.y, nx.z, nx.w};
+    uint32_t r[4];
+    if (RC == 4) {
+        uint32_t lo[4], lon[4], hi[4], hip[4];       // words 0..c and c..3
+        lo[0] = o[0]; lon[0] = n[0]; hi[3] = o[3]; hip[3] = p[3];
 #pragma unroll
-    for (int d = 1; d <= R; ++d) r &= __funnelshift_r(x, nx, d) & __funnelshift_l(pv, x, d);
-    return r;
+        for (int c = 1; c < 4; ++c) {
+            lo[c] = comb<DIL>(lo[c - 1], o[c]);
+            lon[c] = comb<DIL>(lon[c - 1], n[c]);
+            hi[3 - c] = comb<DIL>(hi[4 - c], o[3 - c]);
+            hip[3 - c] = comb<DIL>(hip[4 - c], p[3 - c]);
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            r[c] = comb<DIL>(lo[3], comb<DIL>(__funnelshift_l(hip[c], hi[c], 1), __funnelshift_r(lo[c], lon[c], 1)));
+    } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) r[c] = o[c];
+#pragma unroll
+        for (int q = -2; q <= 2; ++q)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const uint32_t w = strip_shift(p[e], o[e], n[e], q);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const int d = 4 * q + e - c;
+                    if ((d < 0 ? -d : d) <= R) r[c] = comb<DIL>(r[c], w);
+                }
+            }
+    }
+    return make_uint4(r[0], r[1], r[2], r[3]);
+}
+
+template <bool DIL>
+__device__ __forceinline__ uint4 comb4(uint4 a, uint4 b)
+{
+    return make_uint4(comb<DIL>(a.x, b.x), comb<DIL>(a.y, b.y), comb<DIL>(a.z, b.z), comb<DIL>(a.w, b.w));
+}
+
+// four adjacent logits of a row; VEC: the logits start on a 16-byte boundary
+// (every row then does: w is a multiple of 32)
+template <bool VEC>
+__device__ __forceinline__ float4 load_logits(const float *p)
+{
+    if (VEC) return __ldg(reinterpret_cast<const float4 *>(p));
+    return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+}
+
+// four adjacent bytes; VEC: the array starts on a 4-byte boundary
+template <bool VEC>
+__device__ __forceinline__ void store_bytes(uint8_t *p, uint32_t v)
+{
+    if (VEC) {
+        *reinterpret_cast<uint32_t *>(p) = v;
+    } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) p[c] = (uint8_t)(v >> 8 * c);
+    }
+}
+
+// a strip's row -> its four words (lane 0 stores)
+__device__ __forceinline__ void store_bits(uint4 *dst, float4 v, int lane)
+{
+    const uint32_t b0 = __ballot_sync(0xffffffffu, v.x > 0.f), b1 = __ballot_sync(0xffffffffu, v.y > 0.f);
+    const uint32_t b2 = __ballot_sync(0xffffffffu, v.z > 0.f), b3 = __ballot_sync(0xffffffffu, v.w > 0.f);
+    if (lane == 0) *dst = make_uint4(b0, b1, b2, b3);
 }
 
 __device__ __forceinline__ uint32_t cluster_rank()
@@ -85,106 +160,58 @@ __device__ __forceinline__ uint32_t dsmem_addr(const void *p, uint32_t rank)
     return r;
 }
 
-__device__ __forceinline__ float dsmem_ld_f32(uint32_t a)
+__device__ __forceinline__ float4 dsmem_ld_f32x4(uint32_t a)
 {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
     return v;
 }
 
-__device__ __forceinline__ uint32_t dsmem_ld_u8(uint32_t a)
+__device__ __forceinline__ uint32_t dsmem_ld_u32(uint32_t a)
 {
     uint32_t v;
-    asm volatile("ld.shared::cluster.u8 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
     return v;
 }
 
-constexpr int CA_HB = 16;           // halo rows per load batch
-constexpr int CA_SB = 8;            // side-word ballots per warp per load batch
+// Shared memory of a CTA, in 16-byte words: bits of window rows x (NS + 2)
+// strips (thresholded, dilated along rows, dilated), of the erosion along rows,
+// the closure; the best logits and labels (a byte each, 0 = none) per pixel.
+template <int NS, int RM>
+struct CloseSmem {
+    static constexpr int NR = CA_ROWS + 4 * RM, SW = NS + 2;
+    static constexpr int A = 0, H = A + NR * SW, D = H + NR * SW, E = D + NR * SW;
+    static constexpr int C = E + (CA_ROWS + 2 * RM) * NS;
+    static constexpr int BV = C + CA_ROWS * NS;                    // float4 [rows NS][32]
+    static constexpr int BL = BV + CA_ROWS * NS * 32;              // uint32 [rows NS][32]
+    static constexpr int BYTES = 16 * (BL + CA_ROWS * NS * 8);
+};
 
-// halo rows j0 .. j0 + CA_HB - 1 of the 4R (the first 2R above the tile, the
-// rest below it), column x; rows outside the image read as 0
-__device__ __forceinline__ void load_halo_rows(float (&hv)[CA_HB], const float *L, int j0, int R, int BR, int r0,
-                                               int h, int w, int x, bool colin)
-{
-#pragma unroll
-    for (int q = 0; q < CA_HB; ++q) {
-        const int j = j0 + q;
-        const int lr = j < 2 * R ? j : BR + j;           // window row
-        const int row = r0 - 2 * R + lr;
-        hv[q] = (j < 4 * R && colin && row >= 0 && row < h) ? __ldg(L + (size_t)row * w + x) : 0.f;
-    }
-}
-
-template <int NW>
-__device__ __forceinline__ void store_halo_rows(uint32_t (*sA)[NW], const float (&hv)[CA_HB], int j0, int R,
-                                                int BR, int lane, int warp)
-{
-#pragma unroll
-    for (int q = 0; q < CA_HB; ++q) {
-        const int j = j0 + q;
-        const uint32_t b = __ballot_sync(0xffffffffu, hv[q] > 0.f);
-        if (lane == 0 && j < 4 * R) sA[j < 2 * R ? j : BR + j][1 + warp] = b;
-    }
-}
-
-// side words: pair p = warp + CA_TW * i (i = i0 .. i0 + CA_SB - 1) is window
-// row p / 2, the word left of the tile (p even) or right of it (p odd)
-__device__ __forceinline__ void load_side_words(float (&hw)[CA_SB], const float *L, int i0, int nwin, int r0,
-                                                int R, int h, int w, int w0, int WW, int warp, int lane)
-{
-#pragma unroll
-    for (int q = 0; q < CA_SB; ++q) {
-        const int p = warp + CA_TW * (i0 + q);
-        const int row = r0 - 2 * R + (p >> 1);
-        const int gw = (p & 1) ? w0 + CA_TW : w0 - 1;
-        hw[q] = (p < 2 * nwin && row >= 0 && row < h && gw >= 0 && gw < WW)
-                    ? __ldg(L + (size_t)row * w + 32 * gw + lane)
-                    : 0.f;
-    }
-}
-
-template <int NW>
-__device__ __forceinline__ void store_side_words(uint32_t (*sA)[NW], const float (&hw)[CA_SB], int i0, int nwin,
-                                                 int warp, int lane)
-{
-#pragma unroll
-    for (int q = 0; q < CA_SB; ++q) {
-        const int p = warp + CA_TW * (i0 + q);
-        const uint32_t b = __ballot_sync(0xffffffffu, hw[q] > 0.f);
-        if (lane == 0 && p < 2 * nwin) sA[p >> 1][(p & 1) ? CA_TW + 1 : 0] = b;
-    }
-}
-
-// RC > 0 fixes the radius at compile time (the paper's 9 x 9 element is
-// RC = 4), so the shift and row loops unroll; RC = 0 takes it from R_rt.
-template <int BR, int RC>
-__global__ void __launch_bounds__(CA_THREADS, 2)
+// One tile of `rows` rows x NS strips.  KC > 1: the CTAs of a cluster share the
+// stream's objects.  RC = 4 fixes the radius at compile time (the paper's 9 x 9
+// element), RC = 0 takes it from R_rt.  VEC: aligned arrays.
+template <int NS, int RC, bool VEC>
+__global__ void __launch_bounds__(CA_THREADS, RC > 0 ? 2 : 1)
 k_close_argmax(const float *__restrict__ logits, const int32_t *__restrict__ gstart, int U, int h,
-               int w, int R_rt, int s, int KC, uint8_t *__restrict__ palette, uint8_t *__restrict__ closed,
+               int w, int R_rt, int s, int rows, int KC, uint8_t *__restrict__ palette, uint8_t *__restrict__ closed,
                uint8_t *__restrict__ grid, int32_t *status)
 {
     const int R = RC > 0 ? RC : R_rt;
-    constexpr int NR = BR + 4 * CA_RMAX;    // window rows [r0 - 2R, r0 + BR + 2R)
-    constexpr int NW = CA_TW + 2;           // window words [w0 - 1, w0 + TW + 1)
-    __shared__ uint32_t sA[NR][NW];         // thresholded logits
-    __shared__ uint32_t sH[NR][NW];         // horizontal dilation
-    __shared__ uint32_t sD[NR][NW];         // dilation
-    __shared__ uint32_t sE[NR][CA_TW];      // dilation, then horizontal erosion
-    __shared__ uint32_t sC[BR][CA_TW];      // closure of the tile's rows
-    __shared__ float sV[BR][CA_THREADS];    // the current object's logits of the tile
-    __shared__ float sBV[BR][CA_THREADS];   // this CTA's best logit per pixel
-    __shared__ uint8_t sBL[BR][CA_THREADS]; // ... and its label (0 = none)
-    // (thread t alone touches column t of sV, sBV and sBL until the merge)
+    constexpr int RM = RC > 0 ? RC : CA_RMAX;
+    using M = CloseSmem<NS, RM>;
+    constexpr int SW = M::SW;                              // window strips [s0 - 1, s0 + NS + 1)
+    constexpr int NT = (CA_ROWS * NS + CA_WARPS - 1) / CA_WARPS;   // tile rows x strips of a warp, at most
+    constexpr int NH = (4 * RM * NS + CA_WARPS - 1) / CA_WARPS;    // halo rows x strips of a warp
+    extern __shared__ uint4 ca_smem[];
+    uint4 *sA = ca_smem + M::A, *sH = ca_smem + M::H, *sD = ca_smem + M::D, *sE = ca_smem + M::E, *sC = ca_smem + M::C;
+    float4 *sBV = reinterpret_cast<float4 *>(ca_smem + M::BV);
+    uint32_t *sBL = reinterpret_cast<uint32_t *>(ca_smem + M::BL);
     pdl_wait();
     const uint32_t rank = KC > 1 ? cluster_rank() : 0u;
     const int g = blockIdx.z / KC;
-    const int r0 = blockIdx.y * BR, w0 = blockIdx.x * CA_TW;
-    const int WW = w >> 5;
+    const int r0 = blockIdx.y * rows, x0 = blockIdx.x * NS * 128;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int brv = min(BR, h - r0);                 // tile rows inside the image
-    const bool colin = w0 + warp < WW;               // warp-uniform: the warp's word is inside
-    const int x = 32 * w0 + t;                       // this thread's column
     const int u0 = gstart[g], u1 = gstart[g + 1];
     // the same values reach every CTA of the cluster, so all of them leave
     // here together, before any cluster barrier
@@ -192,133 +219,185 @@ k_close_argmax(const float *__restrict__ logits, const int32_t *__restrict__ gst
         if (t == 0 && rank == 0) latch_status(status, RS3_EINVAL);
         return;
     }
-    const int nwin = BR + 4 * R;                     // window rows in use
-    const int m = h / s, n = w / s;
-    // down_s without divisions in the pixel loop: the tile rows that are grid
-    // rows (a bit per row) and the first one's grid row; this column's grid
-    // column, or -1
-    const int gi0 = (r0 + s - 1) / s;
-    uint32_t growmask = 0u;
-    for (int i = gi0; i * s < r0 + brv; ++i) growmask |= 1u << (i * s - r0);
-    const int gx = (x % s == 0) ? x / s : -1;
+    const int brv = min(rows, h - r0);                     // tile rows inside the image
+    const int nwin = rows + 4 * R;                         // window rows [r0 - 2R, r0 + rows + 2R)
+    const bool sides = x0 > 0 || x0 + NS * 128 < w;        // columns beside the tile lie in the image
+    if (!sides)
+        for (int p = t; p < 2 * nwin; p += CA_THREADS) sA[(p >> 1) * SW + (p & 1) * (NS + 1)] = make_uint4(0u, 0u, 0u, 0u);
+    // where this lane's pixels lie in an object's image (-1: outside): the
+    // tile's rows, and the halo rows (the first 2R above the tile, the rest
+    // below); and, for s >= 4, their grid cell (4 cell + which of the four
+    // columns it takes)
+    int off[NT], hoff[NH], goff[NT];
+    const int gm = h / s, gn = w / s;
+    const int gi0 = (r0 + s - 1) / s;                      // first grid row of the tile
+    uint32_t grows = 0u;                                   // which of its rows are grid rows
+    if (grid && s >= 4)
+        for (int k = gi0 * s - r0; k < brv; k += s) grows |= 1u << k;
+    constexpr int NX = NS == 3 ? 3 : 1;                    // a warp's tasks lie in one strip, unless NS = 3
+    int gx4[NX];
 #pragma unroll
-    for (int k = 0; k < BR; ++k) {
-        sBV[k][t] = 0.f;
-        sBL[k][t] = 0;
+    for (int k = 0; k < NX; ++k) {
+        const int x = x0 + (NX == 1 ? warp % NS : k) * 128 + 4 * lane, gx = (x + s - 1) / s, c = gx * s - x;
+        gx4[k] = c < 4 ? 4 * gx + c : -1;
     }
+#pragma unroll
+    for (int i = 0; i < NT; ++i) {
+        const int p = warp + CA_WARPS * i, k = p / NS, x = x0 + (p % NS) * 128 + 4 * lane;
+        off[i] = p < brv * NS && x < w ? (r0 + k) * w + x : -1;
+        const int gx = NX == 1 ? gx4[0] : p % NS == 0 ? gx4[0] : p % NS == 1 ? gx4[1 % NX] : gx4[2 % NX];
+        goff[i] = off[i] >= 0 && gx >= 0 && (grows >> k & 1u) ? 4 * (gi0 + __popc(grows & ((1u << k) - 1u))) * gn + gx : -1;
+    }
+#pragma unroll
+    for (int i = 0; i < NH; ++i) {
+        const int p = warp + CA_WARPS * i, j = p / NS, x = x0 + (p % NS) * 128 + 4 * lane;
+        const int row = r0 - 2 * R + (j < 2 * R ? j : rows + j);
+        hoff[i] = j < 4 * R && row >= 0 && row < h && x < w ? row * w + x : -1;
+    }
+    const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+    const uint32_t lane_bit = 1u << lane;
     for (int u = u0 + (int)rank; u < u1; u += KC) {
         const float *L = logits + (size_t)u * h * w;
-        // 1. the object's loads: the tile's rows (thread t reads column x),
-        //    the 4R halo rows, and the words left and right of the tile on
-        //    every window row (one ballot per (row, side); warp j takes pairs
-        //    j, j + 8, ...).  The first batch -- all of it for R <= 4 -- is
-        //    issued before its first ballot; larger radii take more batches.
-        float v[BR], hv[CA_HB], hw[CA_SB];
+        uint8_t *gu = grid + (size_t)u * gm * gn;
+        // 1. all of the object's loads, then its ballots: the tile, the halo
+        //    and, in images wider than the tile, the 16 columns on either side
+        float4 v[NT], hv[NH];
 #pragma unroll
-        for (int k = 0; k < BR; ++k) v[k] = (k < brv && colin) ? __ldg(L + (size_t)(r0 + k) * w + x) : 0.f;
-        load_halo_rows(hv, L, 0, R, BR, r0, h, w, x, colin);
-        load_side_words(hw, L, 0, nwin, r0, R, h, w, w0, WW, warp, lane);
-        // the ballot of warp j over row k is word w0 + j of that row
+        for (int i = 0; i < NT; ++i) v[i] = off[i] >= 0 ? load_logits<VEC>(L + off[i]) : none;
 #pragma unroll
-        for (int k = 0; k < BR; ++k) {
-            const uint32_t b = __ballot_sync(0xffffffffu, v[k] > 0.f);
-            if (lane == 0) sA[2 * R + k][1 + warp] = b;
-            sV[k][t] = v[k];
+        for (int i = 0; i < NH; ++i) hv[i] = hoff[i] >= 0 ? load_logits<VEC>(L + hoff[i]) : none;
+#pragma unroll
+        for (int i = 0; i < NT; ++i) {
+            const int p = warp + CA_WARPS * i;
+            if (p < rows * NS) store_bits(&sA[(2 * R + p / NS) * SW + 1 + p % NS], v[i], lane);
         }
-        store_halo_rows<NW>(sA, hv, 0, R, BR, lane, warp);
-        store_side_words<NW>(sA, hw, 0, nwin, warp, lane);
-        for (int j0 = CA_HB; j0 < 4 * R; j0 += CA_HB) {
-            load_halo_rows(hv, L, j0, R, BR, r0, h, w, x, colin);
-            store_halo_rows<NW>(sA, hv, j0, R, BR, lane, warp);
+#pragma unroll
+        for (int i = 0; i < NH; ++i) {
+            const int p = warp + CA_WARPS * i, j = p / NS;
+            if (j < 4 * R) store_bits(&sA[(j < 2 * R ? j : rows + j) * SW + 1 + p % NS], hv[i], lane);
         }
-        for (int i0 = CA_SB; warp + CA_TW * i0 < 2 * nwin; i0 += CA_SB) {
-            load_side_words(hw, L, i0, nwin, r0, R, h, w, w0, WW, warp, lane);
-            store_side_words<NW>(sA, hw, i0, nwin, warp, lane);
+        if (sides) {
+            // lanes 28..31 read the strip to the left, lanes 0..3 the one to the right
+            for (int lr = warp; lr < nwin; lr += CA_WARPS) {
+                const int row = r0 - 2 * R + lr, x = lane >= 28 ? x0 - 128 + 4 * lane : x0 + NS * 128 + 4 * lane;
+                const bool in = (lane < 4 || lane >= 28) && row >= 0 && row < h && x >= 0 && x < w;
+                const float4 sv = in ? load_logits<VEC>(L + (size_t)row * w + x) : none;
+                const uint32_t b0 = __ballot_sync(0xffffffffu, sv.x > 0.f), b1 = __ballot_sync(0xffffffffu, sv.y > 0.f);
+                const uint32_t b2 = __ballot_sync(0xffffffffu, sv.z > 0.f), b3 = __ballot_sync(0xffffffffu, sv.w > 0.f);
+                if (lane < 2) {
+                    const uint32_t k = lane ? 0xfu : 0xf0000000u;
+                    sA[lr * SW + lane * (NS + 1)] = make_uint4(b0 & k, b1 & k, b2 & k, b3 & k);
+                }
+            }
         }
         __syncthreads();
-        // 2. horizontal dilation on every window word (the outermost words'
+        // 2. horizontal dilation on every window strip (the outermost strips'
         //    missing neighbours are read as zero: only their bits next to the
         //    tile are used below, and those do not depend on them)
-        for (int p = t; p < nwin * NW; p += CA_THREADS) {
-            const int lr = p / NW, lw = p - lr * NW;
-            const uint32_t pv = lw > 0 ? sA[lr][lw - 1] : 0u;
-            const uint32_t nx = lw < NW - 1 ? sA[lr][lw + 1] : 0u;
-            sH[lr][lw] = dil_h(pv, sA[lr][lw], nx, R);
+        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+        for (int p = t; p < nwin * SW; p += CA_THREADS) {
+            const int ls = p % SW;
+            sH[p] = horizontal<true, RC>(ls > 0 ? sA[p - 1] : zero, sA[p], ls < SW - 1 ? sA[p + 1] : zero, R);
         }
         __syncthreads();
-        // 3. vertical dilation, window rows [R, BR + 3R)
-        for (int p = t; p < (BR + 2 * R) * NW; p += CA_THREADS) {
-            const int lr = R + p / NW, lw = p % NW;
-            uint32_t r = 0u;
+        // 3. vertical dilation, window rows [R, rows + 3R)
+        for (int p = R * SW + t; p < (rows + 3 * R) * SW; p += CA_THREADS) {
+            uint4 r = sH[p];
 #pragma unroll
-            for (int d = -R; d <= R; ++d) r |= sH[lr + d][lw];
-            sD[lr][lw] = r;
+            for (int d = 1; d <= R; ++d) r = comb4<true>(r, comb4<true>(sH[p - d * SW], sH[p + d * SW]));
+            sD[p] = r;
         }
         __syncthreads();
-        // 4. horizontal erosion of the tile's words, window rows [R, BR + 3R)
-        for (int p = t; p < (BR + 2 * R) * CA_TW; p += CA_THREADS) {
-            const int lr = R + p / CA_TW, k = p % CA_TW;
-            sE[lr][k] = ero_h(sD[lr][k], sD[lr][k + 1], sD[lr][k + 2], R);
+        // 4. horizontal erosion of the tile's strips, window rows [R, rows + 3R)
+        for (int p = t; p < (rows + 2 * R) * NS; p += CA_THREADS) {
+            const uint4 *d = sD + (R + p / NS) * SW + p % NS;
+            sE[p] = horizontal<false, RC>(d[0], d[1], d[2], R);
         }
         __syncthreads();
         // 5. vertical erosion: the closure of the tile's rows
-        for (int p = t; p < BR * CA_TW; p += CA_THREADS) {
-            const int k = p / CA_TW, wd = p % CA_TW;
-            uint32_t r = 0xffffffffu;
+        for (int p = t; p < rows * NS; p += CA_THREADS) {
+            uint4 r = sE[p + R * NS];
 #pragma unroll
-            for (int d = -R; d <= R; ++d) r &= sE[2 * R + k + d][wd];
-            sC[k][wd] = r;
+            for (int d = 1; d <= R; ++d) r = comb4<false>(r, comb4<false>(sE[p + (R - d) * NS], sE[p + (R + d) * NS]));
+            sC[p] = r;
         }
         __syncthreads();
         // 6. argmax update, closed mask and its down_s onto the grid
-        const uint32_t label = (uint32_t)(u - u0 + 1);
+        const uint32_t lab = (uint32_t)(u - u0 + 1);
+        const bool first = u == u0 + (int)rank;
 #pragma unroll
-        for (int k = 0; k < BR; ++k) {
-            if (k < brv && colin) {
-                const uint32_t bit = (sC[k][warp] >> lane) & 1u;
-                const float vk = sV[k][t];
-                if (bit && (sBL[k][t] == 0 || vk > sBV[k][t])) {
-                    sBV[k][t] = vk;
-                    sBL[k][t] = (uint8_t)label;
+        for (int i = 0; i < NT; ++i) {
+            const int p = warp + CA_WARPS * i;
+            if (p >= rows * NS) continue;
+            const uint4 cw = sC[p];
+            const bool bit[4] = {(cw.x & lane_bit) != 0, (cw.y & lane_bit) != 0, (cw.z & lane_bit) != 0,
+                                 (cw.w & lane_bit) != 0};
+            const float vv[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+            float bv[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+            uint32_t bl = 0u;
+            if (!first) {
+                const float4 b = sBV[p * 32 + lane];
+                bv[0] = b.x; bv[1] = b.y; bv[2] = b.z; bv[3] = b.w;
+                bl = sBL[p * 32 + lane];
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (bit[c] && vv[c] > bv[c]) {
+                    bv[c] = vv[c];
+                    bl = __byte_perm(bl, lab, c == 0 ? 0x3214 : c == 1 ? 0x3240 : c == 2 ? 0x3410 : 0x4210);
                 }
-                if (closed) closed[((size_t)u * h + r0 + k) * w + x] = (uint8_t)bit;
-                if (grid && gx >= 0 && ((growmask >> k) & 1u))
-                    grid[((size_t)u * m + gi0 + __popc(growmask & ((1u << k) - 1u))) * n + gx] = (uint8_t)bit;
+            sBV[p * 32 + lane] = make_float4(bv[0], bv[1], bv[2], bv[3]);
+            sBL[p * 32 + lane] = bl;
+            const uint32_t bytes = (uint32_t)bit[0] | (uint32_t)bit[1] << 8 | (uint32_t)bit[2] << 16 | (uint32_t)bit[3] << 24;
+            if (closed && off[i] >= 0) store_bytes<VEC>(closed + (size_t)u * h * w + off[i], bytes);
+            if (goff[i] >= 0) gu[goff[i] >> 2] = (uint8_t)(bytes >> 8 * (goff[i] & 3) & 1u);
+            if (grid && s < 4 && off[i] >= 0) {            // several cells in the lane's four columns
+                const int row = r0 + p / NS, x = x0 + (p % NS) * 128 + 4 * lane;
+                if (row % s == 0)
+                    for (int gx = (x + s - 1) / s; gx * s < x + 4; ++gx)
+                        gu[row / s * gn + gx] = (uint8_t)(bytes >> 8 * (gx * s - x) & 1u);
             }
         }
     }
+    if (u0 + (int)rank >= u1)                              // no object: nothing written above
+        for (int p = warp; p < rows * NS; p += CA_WARPS) sBL[p * 32 + lane] = 0u;
     if (KC > 1) {
-        // 7. the ranks' bests are in their shared memory; rank r merges tile rows
-        //    r, r + KC, ...: the larger logit, the lower label on equal logits
-        //    (each rank's best already holds its lowest label among equal
-        //    logits), and writes those palette rows
+        // 7. rank r merges rows (of a strip) r, r + KC, ... of the tile: the
+        //    larger logit, the lower label on equal logits (each rank's best
+        //    already holds its lowest label among equal logits)
         cluster_barrier();
-        for (int k = (int)rank; k < BR; k += KC) {
-            float v2[8];
+        for (int p = warp * KC + (int)rank; p < rows * NS; p += CA_WARPS * KC) {
+            float b[4] = {0.f, 0.f, 0.f, 0.f};
+            uint32_t bl = 0u;
+            float4 v2[8];
             uint32_t l2[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
+            for (int q = 0; q < 8; ++q)
                 if (q < KC) {
-                    v2[q] = dsmem_ld_f32(dsmem_addr(&sBV[k][t], (uint32_t)q));
-                    l2[q] = dsmem_ld_u8(dsmem_addr(&sBL[k][t], (uint32_t)q));
+                    v2[q] = dsmem_ld_f32x4(dsmem_addr(sBV + p * 32 + lane, (uint32_t)q));
+                    l2[q] = dsmem_ld_u32(dsmem_addr(sBL + p * 32 + lane, (uint32_t)q));
                 }
-            }
-            float b = 0.f;
-            uint32_t l = 0u;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                if (q < KC && l2[q] != 0u && (l == 0u || v2[q] > b || (v2[q] == b && l2[q] < l))) {
-                    b = v2[q];
-                    l = l2[q];
+            for (int q = 0; q < 8; ++q)
+                if (q < KC) {
+                    const float vq[4] = {v2[q].x, v2[q].y, v2[q].z, v2[q].w};
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const uint32_t ln = l2[q] >> 8 * c & 255u, lo = bl >> 8 * c & 255u;
+                        if (ln != 0u && (lo == 0u || vq[c] > b[c] || (vq[c] == b[c] && ln < lo))) {
+                            b[c] = vq[c];
+                            bl = (bl & ~(255u << 8 * c)) | ln << 8 * c;
+                        }
+                    }
                 }
-            }
-            if (palette && k < brv && colin) palette[((size_t)g * h + r0 + k) * w + x] = (uint8_t)l;
+            const int row = r0 + p / NS, x = x0 + (p % NS) * 128 + 4 * lane;
+            if (palette && row < h && x < w) store_bytes<VEC>(palette + ((size_t)g * h + row) * w + x, bl);
         }
         cluster_barrier();       // no CTA leaves while another reads its shared memory
     } else if (palette) {
 #pragma unroll
-        for (int k = 0; k < BR; ++k)
-            if (k < brv && colin) palette[((size_t)g * h + r0 + k) * w + x] = sBL[k][t];
+        for (int i = 0; i < NT; ++i)
+            if (off[i] >= 0) store_bytes<VEC>(palette + (size_t)g * h * w + off[i], sBL[(warp + CA_WARPS * i) * 32 + lane]);
     }
 }
 
@@ -403,15 +482,50 @@ __global__ void __launch_bounds__(256) k_seed_finish(const uint8_t *__restrict__
 
 }  // namespace
 
-template <int BR, int RC>
-static cudaError_t launch_close(int tiles_x, int h, int G, int KC, cudaStream_t st, const float *logits,
+struct CloseShape {
+    int ns, rows, KC, tiles_x;
+};
+
+// Rows per tile and CTAs per cluster: the least waves x objects per CTA x cost
+// of an object, where the cost counts the strip rows read (halo and all) and a
+// fixed part for the passes' latency, worth about 40 of them.  Two CTAs are
+// resident per SM; the rows tried are those that just fill one wave, 16 and 24.
+static CloseShape close_shape(int G, int objects, int h, int w)
+{
+    CloseShape best = {};
+    best.ns = std::min(4, (w + 127) / 128);
+    best.tiles_x = (w + 128 * best.ns - 1) / (128 * best.ns);
+    const int slots = 2 * rs3_sm_count();
+    double least = 0.0;
+    for (int KC = 1; KC <= objects; ++KC) {
+        const long long columns = (long long)best.tiles_x * G * KC;     // CTAs per row of tiles
+        const int tiles = (int)std::max(1ll, slots / columns);
+        const int fit = std::min(CA_ROWS, std::max(4, (h + tiles - 1) / tiles));
+        for (const int rows : {fit, 16, CA_ROWS}) {
+            const long long ctas = columns * ((h + rows - 1) / rows);
+            const double cost = (double)((ctas + slots - 1) / slots) * ((objects + KC - 1) / KC) *
+                                    (40.0 + (double)(rows + 16) * best.ns) + (KC > 1 ? 20.0 : 0.0);
+            if (best.KC == 0 || cost < least) {
+                least = cost;
+                best.rows = rows;
+                best.KC = KC;
+            }
+        }
+    }
+    return best;
+}
+
+template <int NS, int RC, bool VEC>
+static cudaError_t launch_close(const CloseShape &c, int h, int G, cudaStream_t st, const float *logits,
                                 const int32_t *gstart, int U, int w, int R, int s, uint8_t *palette,
                                 uint8_t *closed, uint8_t *grid, int32_t *status)
 {
+    constexpr int smem = CloseSmem<NS, (RC > 0 ? RC : CA_RMAX)>::BYTES;
+    if (rs3_kernel_smem((const void *)k_close_argmax<NS, RC, VEC>, smem) != RS3_OK) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(tiles_x, (h + BR - 1) / BR, G * KC);
+    cfg.gridDim = dim3(c.tiles_x, (h + c.rows - 1) / c.rows, G * c.KC);
     cfg.blockDim = dim3(CA_THREADS);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -419,11 +533,22 @@ static cudaError_t launch_close(int tiles_x, int h, int G, int KC, cudaStream_t 
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = 1;
     attr[1].val.clusterDim.y = 1;
-    attr[1].val.clusterDim.z = KC;
+    attr[1].val.clusterDim.z = c.KC;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, k_close_argmax<BR, RC>, logits, gstart, U, h, w, R, s, KC, palette, closed,
-                              grid, status);
+    return cudaLaunchKernelEx(&cfg, k_close_argmax<NS, RC, VEC>, logits, gstart, U, h, w, R, s, c.rows, c.KC, palette,
+                              closed, grid, status);
+}
+
+template <int RC, bool VEC, typename... Args>
+static cudaError_t launch_close_strips(const CloseShape &c, Args... args)
+{
+    switch (c.ns) {
+    case 1: return launch_close<1, RC, VEC>(c, args...);
+    case 2: return launch_close<2, RC, VEC>(c, args...);
+    case 3: return launch_close<3, RC, VEC>(c, args...);
+    default: return launch_close<4, RC, VEC>(c, args...);
+    }
 }
 
 extern "C" rs3_status rs3_close_argmax(const float *logits, const int32_t *group_start, int G, int U, int h,
@@ -436,26 +561,24 @@ extern "C" rs3_status rs3_close_argmax(const float *logits, const int32_t *group
     if (grid_masks && (h % s != 0 || w % s != 0)) return RS3_EINVAL;
     if ((long long)h * w > (1ll << 31)) return RS3_EUNSUPPORTED;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    // cluster size: the mean number of objects per stream, at most 8 (the
-    // portable cluster size); ranks past a stream's object count idle
-    const int KC = std::min(8, std::max(1, (U + G - 1) / G));
-    if ((long long)G * KC > 65535) return RS3_EUNSUPPORTED;
-    const int tiles_x = (w / 32 + CA_TW - 1) / CA_TW;
-    // the taller tile (fewer halo rows per tile row) when it still gives two
-    // CTAs per SM
-    const long long ctas16 = (long long)tiles_x * ((h + 15) / 16) * G * KC;
-    const bool tall = ctas16 >= 2ll * rs3_sm_count();
+    // objects of a stream on average, at most 8 (the portable cluster size);
+    // ranks past a stream's object count idle
+    const int objects = std::min(8, std::max(1, (U + G - 1) / G));
+    if ((long long)G * objects > 65535) return RS3_EUNSUPPORTED;
+    const CloseShape c = close_shape(G, objects, h, w);
+    // 16-byte loads and 4-byte stores where the arrays allow them
+    const auto low = [](const void *p) { return reinterpret_cast<uintptr_t>(p); };
+    const bool vec = rs3_aligned16(logits) && ((low(palette) | low(closed)) & 3u) == 0;
     cudaError_t e;
-    if (radius == 4)        // the paper's 9 x 9 element, unrolled
-        e = tall ? launch_close<16, 4>(tiles_x, h, G, KC, st, logits, group_start, U, w, radius, s, palette,
-                                       closed, grid_masks, status)
-                 : launch_close<8, 4>(tiles_x, h, G, KC, st, logits, group_start, U, w, radius, s, palette,
-                                      closed, grid_masks, status);
+    if (!vec)
+        e = launch_close_strips<0, false>(c, h, G, st, logits, group_start, U, w, radius, s, palette,
+                                          closed, grid_masks, status);
+    else if (radius == 4)                    // the paper's 9 x 9 element
+        e = launch_close_strips<4, true>(c, h, G, st, logits, group_start, U, w, radius, s, palette,
+                                         closed, grid_masks, status);
     else
-        e = tall ? launch_close<16, 0>(tiles_x, h, G, KC, st, logits, group_start, U, w, radius, s, palette,
-                                       closed, grid_masks, status)
-                 : launch_close<8, 0>(tiles_x, h, G, KC, st, logits, group_start, U, w, radius, s, palette,
-                                      closed, grid_masks, status);
+        e = launch_close_strips<0, true>(c, h, G, st, logits, group_start, U, w, radius, s, palette,
+                                         closed, grid_masks, status);
     return e == cudaSuccess ? RS3_OK : RS3_ECUDA;
 }
 
