@@ -36,7 +36,7 @@ sys.path.insert(0, ROOT)
 
 METRIC = "pruned readout frames/s & TFLOP/s vs dense (1 GB300); bank-commit HBM GB/s"
 WORKLOAD = "sam2_8obj"
-KERNELS_PER_READOUT_FRAME = 7     # prior, energy, select, plan, readout, combine, commit
+KERNELS_PER_READOUT_FRAME = 5     # select, plan, readout, combine, commit
 STEP_TARGET_S = 0.05              # a step replays the sequence about this long
 DECODER_STRIDE = 4                # decoder masks at 4x the token grid (SAM2: 256^2 masks, 64^2 tokens)
 CLOSE_RADIUS = 4                  # the 9 x 9 closure of Sec. 3.3
@@ -710,7 +710,7 @@ RUN_KERNEL = "k_readout_tc (tcgen05 attention kernel; bf16 workloads)"
 def launches_per_pass(w):
     """Library kernels one benchmark pass launches: the bank reset, the
     conditioning commit (and the pointer rows), and per readout frame the
-    selection (prior, energy, select), the readout (plan, attention, merge)
+    selection, the readout (plan, attention, merge)
     and the commit."""
     return (1 + w.prefill_frames + (2 if w.n_ptr > 0 else 1)
             + (w.frames - (1 if w.n_cond > 0 else 0)) * KERNELS_PER_READOUT_FRAME)

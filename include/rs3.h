@@ -112,8 +112,8 @@ int rs3_version(void);
 /* Read side: keep-set selection (Sec. 3.1; Eq. 1, 2, 4, 5)                 */
 /* ------------------------------------------------------------------------ */
 
-/* Bytes of device workspace rs3_select_queries needs (a group "needed-cell"
- * bitmap, per-unit priors and group energies). */
+/* Bytes of device workspace rs3_select_queries is to be given (a group
+ * "needed-cell" bitmap, per-unit priors and group energies). */
 size_t rs3_select_workspace_bytes(int G, int U, int m, int n);
 
 /*
@@ -157,23 +157,12 @@ rs3_status rs3_select_queries(const void *z, rs3_dtype dtype, int G, int m, int 
  * Some callers have no allocator to ask for the workspace (code running while
  * a stream is captured in the global capture mode, serving loops that must not
  * allocate after start-up, hosts that pass only input and output buffers
- * through a plugin interface); this call instead uses scratch memory compiled
- * into the library: an 8 MiB device array that every GPU loading the library
- * holds until the process exits.  Arguments and results are those of
+ * through a plugin interface).  Arguments and results are those of
  * rs3_select_queries without the workspace pair.
  *   - Sizes whose workspace (rs3_select_workspace_bytes(G, U, m, n)) exceeds
  *     8 MiB are rejected with RS3_ECAPACITY; nothing is launched.
  *   - The call allocates nothing (no cudaMalloc / cudaFree, no allocating
- *     library routine).
- *   - The first call on a device looks up the array's device address with
- *     that device current and caches it; make that first call before any
- *     stream capture.  The cache remembers the context the address belongs
- *     to: after a device reset the next call looks the address up again, so
- *     make that call before any capture too.
- *   - All calls on a device share the one array, and it keeps the previous
- *     call's contents (the call clears what must start at zero itself), so
- *     calls whose executions overlap on the GPU (different streams without
- *     ordering between them) race and must not be issued.
+ *     library routine) and shares no memory between calls.
  */
 rs3_status rs3_select_queries_noalloc(const void *z, rs3_dtype dtype, int G, int m, int n, int C,
                                       const uint8_t *prev_masks, const int32_t *unit_group, int U,
