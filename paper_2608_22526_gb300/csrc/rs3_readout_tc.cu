@@ -7,14 +7,14 @@
 // (unit, head, 128-query tile, range of BN-key tiles).  Warps:
 //   warp 0      K producer: TMA of the key tile (d/64 boxes of BN rows x 64)
 //   warp 2      V producer: TMA of the value tile
-//   warp 1      TMEM allocation; lane 0 issues S_j = Q K_j^T (M 128, N BN,
+//   warp 1      TMEM allocation; issues S_j = Q K_j^T (M 128, N BN,
 //               K d; A = Q in TMEM, B = K tile, K-major) into one of two TMEM
 //               buffers as soon as the softmax has read the one before
-//   warp 3      lane 0 issues O += P_j V_j (M 128, N d, K BN; A = P_j in
+//   warp 3      issues O += P_j V_j (M 128, N d, K BN; A = P_j in
 //               shared memory, B = V tile, MN-major) once P_j is written.  The
 //               two issuers share no operand, so each one's waits overlap the
 //               other's MMAs.
-//   warp 3      lanes 1..31: L2 prefetch of the query rows of later items
+//   warp 2      lanes 1..31: L2 prefetch of the query rows of later items
 //   warps 4..   2 x 4 softmax warps; warps w and w + 4 own the same TMEM lane
 //               quarter (rows 32 (w % 4) + lane) and split the columns.  Per
 //               item each thread loads its slice of the kept query row,
@@ -26,6 +26,10 @@
 //               buffers).  The slices of a row exchange their maxima through
 //               shared memory at a named barrier that also ANDs their wait
 //               results.  Epilogue: O / l + residual, or split-KV partials.
+// Both issuers are whole warps in uniform code that elect the issuing thread:
+// 8 objects on a 64 x 64 grid, d = 256 (57 GFLOP), 68 us per call, 76 with
+// the issue behind a branch on the lane (16 S instructions then took 1 200 clk
+// to issue, 512 to run).
 // TMEM (512 columns): O in [0, d), S_0 / S_1 from S_COL, Q at Q_COL.
 // Shapes: d = 256 and d = 128 use 64-key tiles, d = 64 128-key tiles; K and V
 // rings fill what shared memory leaves after the three P buffers.
@@ -34,9 +38,8 @@
 // raises an abort flag, drains its copies and MMAs, frees TMEM and the launch
 // latches RS3_ETIMEOUT.
 #include "rs3_readout_common.cuh"
+#include "rs3_tc_host.cuh"
 #include "rs3_tc_ptx.cuh"
-
-#include <cudaTypedefs.h>
 
 namespace tc {
 
@@ -85,49 +88,6 @@ struct Cfg {
 };
 static_assert(Cfg<256>::SMEM <= 232448 && Cfg<128>::SMEM <= 232448 && Cfg<64>::SMEM <= 232448,
               "shared memory budget");
-
-// Softmax pieces of one row's S tile (raw scores as fp32 bits).
-template <int N>
-__device__ __forceinline__ float row_max(const uint32_t (&sr)[N], int nv, bool full)
-{
-    float m0 = -INFINITY, m1 = -INFINITY;
-#pragma unroll
-    for (int c = 0; c < N; c += 2) {
-        m0 = fmaxf(m0, (full || c < nv) ? __uint_as_float(sr[c]) : -INFINITY);
-        m1 = fmaxf(m1, (full || c + 1 < nv) ? __uint_as_float(sr[c + 1]) : -INFINITY);
-    }
-    return fmaxf(m0, m1);
-}
-
-// p = 2^(s * sc - ref) of one slice's scores (raw fp32 bits), as bf16 pairs;
-// returns the sum of the p.  The scale-and-shift and the sums run on packed
-// fp32 pairs (f32x2), the exps on the SFU; four partial sums keep the adds
-// independent.  Columns at or past nv (invalid keys) give p = 0.
-template <int N>
-__device__ __forceinline__ float row_exp(const uint32_t (&sr)[N], uint32_t (&pk)[N / 2], float sc, float ref,
-                                         int nv, bool full)
-{
-    const uint64_t sc2 = f2pack(sc, sc), nref2 = f2pack(-ref, -ref);
-    uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
-#pragma unroll
-    for (int c = 0; c < N / 2; ++c) {
-        float x0, x1;
-        f2unpack(fma2(f2pack(__uint_as_float(sr[2 * c]), __uint_as_float(sr[2 * c + 1])), sc2, nref2), x0, x1);
-        float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
-        if (!full) {
-            p0 = 2 * c < nv ? p0 : 0.f;
-            p1 = 2 * c + 1 < nv ? p1 : 0.f;
-        }
-        acc[c & 3] = add2(acc[c & 3], f2pack(p0, p1));
-        pk[c] = pack_bf16x2(p0, p1);
-    }
-    float a0, a1, a2, a3, a4, a5, a6, a7;
-    f2unpack(acc[0], a0, a1);
-    f2unpack(acc[1], a2, a3);
-    f2unpack(acc[2], a4, a5);
-    f2unpack(acc[3], a6, a7);
-    return ((a0 + a1) + (a2 + a3)) + ((a4 + a5) + (a6 + a7));
-}
 
 // NW consecutive bf16 pairs of one thread's kept query row -> its TMEM lane,
 // columns [tq, tq + NW) (element 2i in the low half).  With a RoPE table,
@@ -253,79 +213,97 @@ k_readout_tc(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk,
         // let every copy this thread issued land before the CTA can exit
         for (uint32_t k = (cnt > nst ? cnt - nst : 0); k < cnt; ++k)
             mbar_drain(BAR(b_full + k % nst), (k / nst) & 1u);
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         // ------------------------------------------------------------------
-        // S issuer: S_t = Q K_t^T into TMEM buffer t & 1, once the softmax
-        // has read S_{t-2}; runs up to two tiles ahead of the softmax
+        // S issuer (the whole warp walks, one thread issues): S_t = Q K_t^T into
+        // TMEM buffer t & 1, once the softmax has read S_{t-2}; runs up to two
+        // tiles ahead of the softmax
         // ------------------------------------------------------------------
         constexpr uint32_t ID_S = idesc_bf16(BM, BN, false);
+        const uint32_t tm = (uint32_t)uniform((int)tmem);
         // descriptors built once; a k-step only adds its byte offset / 16 to the
         // start-address field (every address stays below 256 KB, so the 14-bit
         // field cannot carry)
-        const uint64_t dk0 = desc_sw128(sK, 16, 1024);
+        const uint64_t dk0 = desc_sw128((uint32_t)uniform((int)sK), 16, 1024);
         constexpr uint32_t STAGE16 = C::KVBYTES >> 4;
-        uint32_t tcnt = 0, icnt = 0;
+        uint32_t b = 0, sph = 1, ks = 0, kph = 0, qph = 0;   // S buffer and K stage, their phases; Q's phase
         bool ok = true;
-        for (int it = it_begin; it < it_end && ok; ++it) {
+        const int itb = uniform(it_begin), ite = uniform(it_end);
+        for (int it = itb; it < ite && ok; ++it) {
             const WorkItem w = a.items[it];
-            const int n = w.tile_end - w.tile_begin;
+            const int n = uniform(w.tile_end - w.tile_begin);
             if (n <= 0) continue;
-            if (!mbar_wait(BAR(C::B_QFULL), icnt & 1u, abort_flag, wait_ns)) { ok = false; break; }
-            ++icnt;
-            for (int j = 0; j < n; ++j) {
-                const uint32_t t = tcnt + (uint32_t)j, st = t % KSTK, b = t & 1u;
-                if (!mbar_wait(BAR(C::B_SFREE + b), ((t >> 1) & 1u) ^ 1u, abort_flag, wait_ns)) { ok = false; break; }
-                if (!mbar_wait(BAR(C::B_KFULL + st), (t / KSTK) & 1u, abort_flag, wait_ns)) { ok = false; break; }
+            ok = mbar_wait_warp(BAR(C::B_QFULL), qph, abort_flag, wait_ns);
+            qph ^= 1u;
+            for (int j = 0; j < n && ok; ++j) {
+                ok = mbar_wait_warp(BAR(C::B_SFREE + b), sph, abort_flag, wait_ns) &&
+                     mbar_wait_warp(BAR(C::B_KFULL + ks), kph, abort_flag, wait_ns);
+                if (!ok) break;
                 tc_fence_after();
-                const uint64_t dks = dk0 + st * STAGE16;
-                const uint32_t dst = tmem + C::S_COL + (uint32_t)BN * b;
+                if (elect_one()) {
+                    const uint64_t dks = dk0 + ks * STAGE16;
+                    const uint32_t dst = tm + C::S_COL + (uint32_t)BN * b;
 #pragma unroll
-                for (int kk = 0; kk < DH / 16; ++kk) {
-                    const uint32_t offk = (uint32_t)((kk >> 2) * (BN * 128) + (kk & 3) * 32);
-                    tc_mma_ts(dst, tmem + C::Q_COL + 8u * kk, dks + (offk >> 4), ID_S, kk > 0 ? 1u : 0u);
+                    for (int kk = 0; kk < DH / 16; ++kk) {
+                        const uint32_t offk = (uint32_t)((kk >> 2) * (BN * 128) + (kk & 3) * 32);
+                        tc_mma_ts(dst, tm + C::Q_COL + 8u * kk, dks + (offk >> 4), ID_S, kk > 0 ? 1u : 0u);
+                    }
+                    tc_commit(BAR(C::B_SFULL + b));
+                    tc_commit(BAR(C::B_KEMPTY + ks));
                 }
-                tc_commit(BAR(C::B_SFULL + b));
-                tc_commit(BAR(C::B_KEMPTY + st));
+                __syncwarp();
+                b ^= 1u;
+                if (b == 0u) sph ^= 1u;
+                if (++ks == KSTK) { ks = 0; kph ^= 1u; }
             }
-            tcnt += (uint32_t)n;
         }
         // every MMA issued by this thread completes before TMEM is released
-        tc_commit(BAR(C::B_DRAIN));
-        mbar_drain(BAR(C::B_DRAIN), 0);
-    } else if (warp == 3 && lane == 0) {
+        if (elect_one()) {
+            tc_commit(BAR(C::B_DRAIN));
+            mbar_drain(BAR(C::B_DRAIN), 0);
+        }
+    } else if (warp == 3) {
         // ------------------------------------------------------------------
         // PV issuer: O += P_t V_t once the softmax has written P_t; its own
-        // thread, so its waits overlap the S issue and the other way round
+        // warp, so its waits overlap the S issue and the other way round
         // ------------------------------------------------------------------
         constexpr uint32_t ID_PV = idesc_bf16(BM, DH, true);
-        const uint64_t dv0 = desc_sw128(sV, BN * 128, 1024), dp0 = desc_sw128(sP, 16, 1024);
+        const uint32_t tm = (uint32_t)uniform((int)tmem);
+        const uint64_t dv0 = desc_sw128((uint32_t)uniform((int)sV), BN * 128, 1024);
+        const uint64_t dp0 = desc_sw128((uint32_t)uniform((int)sP), 16, 1024);
         constexpr uint32_t STAGE16 = C::KVBYTES >> 4, PBUF16 = C::PBYTES >> 4;
-        uint32_t tcnt = 0;
+        uint32_t pb = 0, pph = 0, vs = 0, vph = 0;           // P buffer and V stage, their phases
         bool ok = true;
-        for (int it = it_begin; it < it_end && ok; ++it) {
+        const int itb = uniform(it_begin), ite = uniform(it_end);
+        for (int it = itb; it < ite && ok; ++it) {
             const WorkItem w = a.items[it];
-            const int n = w.tile_end - w.tile_begin;
-            if (n <= 0) continue;
-            for (int j = 0; j < n; ++j) {
-                const uint32_t tj = tcnt + (uint32_t)j, pb = tj % C::NPB, st = tj % KSTV;
-                if (!mbar_wait(BAR(C::B_PFULL + pb), (tj / C::NPB) & 1u, abort_flag, wait_ns)) { ok = false; break; }
-                if (!mbar_wait(BAR(C::B_VFULL + st), (tj / KSTV) & 1u, abort_flag, wait_ns)) { ok = false; break; }
+            const int n = uniform(w.tile_end - w.tile_begin);
+            for (int j = 0; j < n && ok; ++j) {
+                ok = mbar_wait_warp(BAR(C::B_VFULL + vs), vph, abort_flag, wait_ns) &&
+                     mbar_wait_warp(BAR(C::B_PFULL + pb), pph, abort_flag, wait_ns);
+                if (!ok) break;
                 tc_fence_after();
-                const uint64_t dvs = dv0 + st * STAGE16, dps = dp0 + pb * PBUF16;
+                if (elect_one()) {
+                    const uint64_t dvs = dv0 + vs * STAGE16, dps = dp0 + pb * PBUF16;
 #pragma unroll
-                for (int kk = 0; kk < BN / 16; ++kk) {
-                    const uint32_t offp = (uint32_t)((kk >> 2) * (BM * 128) + (kk & 3) * 32);
-                    tc_mma(tmem, dps + (offp >> 4), dvs + (uint32_t)((kk * 2048) >> 4), ID_PV,
-                           (j > 0 || kk > 0) ? 1u : 0u);
+                    for (int kk = 0; kk < BN / 16; ++kk) {
+                        const uint32_t offp = (uint32_t)((kk >> 2) * (BM * 128) + (kk & 3) * 32);
+                        tc_mma(tm, dps + (offp >> 4), dvs + (uint32_t)((kk * 2048) >> 4), ID_PV,
+                               j > 0 || kk > 0 ? 1u : 0u);
+                    }
+                    tc_commit(BAR(C::B_PVDONE + pb));
+                    tc_commit(BAR(C::B_VEMPTY + vs));
                 }
-                tc_commit(BAR(C::B_PVDONE + pb));
-                tc_commit(BAR(C::B_VEMPTY + st));
+                __syncwarp();
+                if (++pb == C::NPB) { pb = 0; pph ^= 1u; }
+                if (++vs == KSTV) { vs = 0; vph ^= 1u; }
             }
-            tcnt += (uint32_t)n;
         }
-        tc_commit(BAR(C::B_DRAIN));
-        mbar_drain(BAR(C::B_DRAIN), 0);
-    } else if (warp == 3) {
+        if (elect_one()) {
+            tc_commit(BAR(C::B_DRAIN));
+            mbar_drain(BAR(C::B_DRAIN), 0);
+        }
+    } else if (warp == 2) {
         // ------------------------------------------------------------------
         // lanes 1..31: L2 prefetch of the kept query rows (and their RoPE
         // rows) of this CTA's later items, so their loads do not wait on DRAM
@@ -412,7 +390,6 @@ k_readout_tc(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk,
                     }
                 }
                 const int nv = nvt - h * SCOLS;       // valid columns of this slice (may be <= 0)
-                const bool full = nv >= SCOLS;
                 const uint32_t scol = tl + C::S_COL + (uint32_t)BN * b;
                 const float sc = a.scale_log2;
                 uint32_t sr[SCOLS], pk[PCOLS];
@@ -425,6 +402,7 @@ k_readout_tc(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk,
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(BAR(C::B_SFREE + b));
+                    if (nv < SCOLS) mask_cols(sr, nv);
                 }
                 float *redt = red + (b * NSPLIT) * BM;
                 float m_new = m_run;
@@ -432,13 +410,13 @@ k_readout_tc(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk,
                     // the first tile of an item sets the reference: the row max
                     // over the slices (the scale is positive, so it is applied
                     // to the max of the raw scores)
-                    redt[h * BM + r] = okw ? row_max<SCOLS>(sr, nv, full) : -INFINITY;
+                    redt[h * BM + r] = okw ? row_max(sr) : -INFINITY;
                     if (!bar_and(bar_id, bar_n, okw)) { ok = false; break; }
                     float mrow = redt[r];
 #pragma unroll
                     for (int q = 1; q < NSPLIT; ++q) mrow = fmaxf(mrow, redt[q * BM + r]);
                     m_new = mrow * sc;
-                    rowsum = row_exp<SCOLS>(sr, pk, sc, m_new, nv, full);
+                    rowsum = row_exp(sr, pk, sc, m_new);
                 } else {
                     // Later tiles take their exps against the running reference.
                     // It moves only if the row max grows past it by more than
@@ -446,17 +424,17 @@ k_readout_tc(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk,
                     // none, so only rows above that (or a timeout) take the slow
                     // path, together with their quarter: exact maxima exchanged,
                     // exps redone against a moved reference, O rescaled.
-                    if (okw) rowsum = row_exp<SCOLS>(sr, pk, sc, m_run, nv, full);
+                    if (okw) rowsum = row_exp(sr, pk, sc, m_run);
                     const bool slow = !(rowsum <= 256.0f);
                     if (bar_or(bar_id, bar_n, slow || !okw)) {
-                        redt[h * BM + r] = okw ? row_max<SCOLS>(sr, nv, full) : -INFINITY;
+                        redt[h * BM + r] = okw ? row_max(sr) : -INFINITY;
                         if (!bar_and(bar_id, bar_n, okw)) { ok = false; break; }
                         float mrow = redt[r];
 #pragma unroll
                         for (int q = 1; q < NSPLIT; ++q) mrow = fmaxf(mrow, redt[q * BM + r]);
                         if (mrow * sc > m_run + 8.0f) {
                             m_new = mrow * sc;
-                            rowsum = row_exp<SCOLS>(sr, pk, sc, m_new, nv, full);
+                            rowsum = row_exp(sr, pk, sc, m_new);
                         }
                         const bool grow = m_new != m_run;
                         const float alpha = grow ? ex2_approx(m_run - m_new) : 1.0f;
@@ -613,33 +591,6 @@ k_readout_tc(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk,
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
-{
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    if (!fn) {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }
-    return fn;
-}
-
-bool make_kv_map(CUtensorMap *m, const void *store, int64_t D, int64_t rows, int box_rows)
-{
-    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
-    if (!enc) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)D, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)D * 2};
-    const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
-    const cuuint32_t es[2] = {1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(store), dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 template <int DH>
 rs3_status launch(const ReadoutArgs &a, cudaStream_t st)
 {

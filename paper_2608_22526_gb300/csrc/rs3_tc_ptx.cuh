@@ -47,6 +47,25 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
+// One thread of the warp (always the same one).  A block of matrix instructions
+// is issued as `if (elect_one())` from code that the whole warp runs with
+// warp-uniform values: their descriptors then live in uniform registers.  From a
+// branch on the lane index every operand is moved there first, and an
+// instruction took about 80 clk to issue instead of the 32 to 64 it runs.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
+// Lane 0's value for the whole warp, known to be uniform.
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 __device__ __forceinline__ uint64_t gtimer()
 {
     uint64_t t;
@@ -54,22 +73,44 @@ __device__ __forceinline__ uint64_t gtimer()
     return t;
 }
 
+// The same without waiting (try_wait may suspend the thread for a while).
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // Waits for the phase with parity `parity` to complete; gives up (and raises
-// the CTA's abort flag) once more than `limit_ns` have passed, or at once if
-// the flag is up.
+// the CTA's abort flag) once more than `limit_ns` have passed (0: unless it has
+// completed already), or at once if the flag is up.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag,
                                           uint64_t limit_ns)
 {
-    if (mbar_try(bar, parity)) return true;
+    if (mbar_test(bar, parity)) return true;
+    if (limit_ns != 0 && mbar_try(bar, parity)) return true;
     const uint64_t t0 = gtimer();
     while (true) {
-        if (mbar_try(bar, parity)) return true;
         if (*abort_flag) return false;
         if (gtimer() - t0 >= limit_ns) {
             *abort_flag = 1;
             return false;
         }
+        if (mbar_try(bar, parity)) return true;
     }
+}
+
+// mbar_wait by every lane of the warp, with one answer.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag,
+                                               uint64_t limit_ns)
+{
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, limit_ns));
 }
 
 // Bounded wait that ignores the abort flag, for draining copies and matrix
@@ -340,6 +381,64 @@ __device__ __forceinline__ bool bar_and(uint32_t id, uint32_t nthreads, bool pre
         : "r"((uint32_t)pred), "r"(id), "r"(nthreads)
         : "memory");
     return res != 0;
+}
+
+// Pieces of one row's softmax over N scores (raw fp32 bits).
+
+__device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi)
+{
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+
+template <int N>
+__device__ __forceinline__ float row_max(const uint32_t (&sr)[N])
+{
+    float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+    for (int c = 0; c < N; c += 2)
+        m[c / 2 & 3] = fmaxf(m[c / 2 & 3], fmaxf(__uint_as_float(sr[c]), __uint_as_float(sr[c + 1])));
+    return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+}
+
+// Scores of keys past a range's end (columns at or past nv) become -inf: p = 0.
+template <int N>
+__device__ __forceinline__ void mask_cols(uint32_t (&sr)[N], int nv)
+{
+#pragma unroll
+    for (int c = 0; c < N; ++c)
+        if (c >= nv) sr[c] = 0xff800000u;
+}
+
+// p = 2^(s sc - ref) as bf16 pairs; returns their sum.  The scale-and-shift and
+// the sums run on packed fp32 pairs, the exps on the SFU, in batches of 16 whose
+// exps are issued back to back: one warp alone then takes 745 clk for 128
+// columns (1 064 in the order the compiler picks); two warps per scheduler take
+// 1 365 together, whatever the order.
+template <int N>
+__device__ __forceinline__ float row_exp(const uint32_t (&sr)[N], uint32_t *pk, float sc, float ref)
+{
+    static_assert(N % 16 == 0, "batches");
+    const uint64_t sc2 = f2pack(sc, sc), nref2 = f2pack(-ref, -ref);
+    uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+    for (int c0 = 0; c0 < N; c0 += 16) {
+        float x[16];
+#pragma unroll
+        for (int c = 0; c < 16; c += 2)
+            f2unpack(fma2(f2pack(__uint_as_float(sr[c0 + c]), __uint_as_float(sr[c0 + c + 1])), sc2, nref2), x[c], x[c + 1]);
+#pragma unroll
+        for (int c = 0; c < 16; ++c) asm volatile("ex2.approx.ftz.f32 %0, %0;" : "+f"(x[c]));
+#pragma unroll
+        for (int c = 0; c < 16; c += 2) {
+            acc[c / 2 & 3] = add2(acc[c / 2 & 3], f2pack(x[c], x[c + 1]));
+            pk[(c0 + c) / 2] = cvt_bf16x2(x[c], x[c + 1]);
+        }
+    }
+    float a, b;
+    f2unpack(add2(add2(acc[0], acc[1]), add2(acc[2], acc[3])), a, b);
+    return a + b;
 }
 
 }  // namespace tc
