@@ -291,6 +291,17 @@ __global__ void __launch_bounds__(PLAN_THREADS) k_plan(ReadoutArgs a)
     int64_t P = (run + a.min_chunk - 1) / a.min_chunk;
     if (P > a.grid_ctas) P = a.grid_ctas;
     __syncthreads();
+    // One unit: its groups are equally long.  With whole slices per group, the
+    // slices of all its query tiles and heads reach a key at the same time; cut
+    // anywhere, they reach it at as many times as the remainder has parts, and a
+    // bank that L2 does not hold is read from DRAM that often.  Worth leaving
+    // CTAs idle for large banks on the tensor cores (300 000 keys of 256, ten
+    // query tiles on 150 of 152 CTAs: 408 -> 281 us); where it leaves 1 in 64,
+    // always.
+    if (a.U == 1 && a.tensor && grun > 0 && P > grun) {
+        const int64_t idle = P % grun, bytes = (int64_t)s_nt[0] * a.BN * a.D * 4;
+        if (64 * idle <= P || (bytes > ((int64_t)48 << 20) && 8 * idle <= P)) P -= idle;
+    }
     PlanView v;
     v.tb = s_tb; v.wg = s_wg; v.nt = s_nt; v.gb = s_gb; v.cnt = s_cnt; v.U = a.U; v.H = a.H; v.W = run;
     v.ov = a.plan_ov;
@@ -606,6 +617,7 @@ rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, in
     // sweep of 4..32 over the 1- and 8-object sequences was best at 8..16; the
     // CUDA-core path is flat over 1..4.  A slice of at least two slots: four
     // left a 32 x 32 fp32 frame on half the CTAs (68 us against 61)
+    a->tensor = p.kind != 0;
     a->plan_ov = p.kind == 1 ? 12 : 1;
     a->max_slots = L.max_slots;
     a->max_items = L.max_items;
