@@ -533,15 +533,29 @@ std::atomic<uint64_t> g_wait_ns{1000000000ull};
 extern "C" void rs3_set_wait_limit_ns(uint64_t ns) { g_wait_ns.store(ns); }
 extern "C" uint64_t rs3_get_wait_limit_ns(void) { return g_wait_ns.load(); }
 
-ReadoutPath choose_readout_path(rs3_dtype dtype, int d)
+// The kernel and its tiles for a call.  bf16 heads of 64 and 128 have two
+// tensor-core kernels: the one with two query tiles per CTA is faster once there
+// are query tiles for half of the CTAs or so (us per call, both measured:
+// 40 tiles of 4 heads of 64: 32.7 against 35.1; 80 tiles 39 against 43; 160
+// tiles of heads of 128 75 against 86; 2 000 tiles 1 080 against 1 704), the
+// other below that (10 tiles 22.6 against 25.6; 20 tiles of heads of 128 31.8
+// against 37.2), and where a pair of tiles would often be half empty (3 tiles
+// per head, 72 in all: 25.5 against 27.0).
+ReadoutPath choose_readout_path(rs3_dtype dtype, int d, int U, int H, int k_max)
 {
     ReadoutPath p;
     const int n_sm = rs3_sm_count();
     if (dtype == RS3_BF16 && rs3_tc_supported(d)) {
+        const int64_t single = (k_max + 127) / 128, pairs = (k_max + 255) / 256;
         p.kind = 1;
         p.BM = 128;
         p.BN = rs3_tc_block_n(d);
         p.grid = n_sm;                 // one persistent CTA per SM
+        if (d <= 128 && (int64_t)U * H * single >= 40 && 8 * pairs <= 5 * single) {
+            p.kind = 2;
+            p.BM = 256;                // two query tiles per item
+            p.BN = 128;
+        }
     } else {
         int ctas;
         p.kind = 0;
@@ -554,7 +568,7 @@ ReadoutPath choose_readout_path(rs3_dtype dtype, int d)
 extern "C" size_t rs3_readout_workspace_bytes(int U, int H, int d, int k_max, rs3_dtype dtype)
 {
     if (U < 1 || H < 1 || d < 1 || k_max < 0) return 0;
-    const ReadoutPath p = choose_readout_path(dtype, d);
+    const ReadoutPath p = choose_readout_path(dtype, d, U, H, k_max);
     return readout_layout(U, H, d, k_max, p.BM, p.grid).total;
 }
 
@@ -577,11 +591,12 @@ rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, in
     if (!rs3_aligned16(q) || !rs3_aligned16(out) || !rs3_aligned16(workspace) ||
         (residual && !rs3_aligned16(residual)) || (rope && !rs3_aligned16(rope)))
         return RS3_EINVAL;
-    const ReadoutPath p = choose_readout_path(dtype, d);
+    const ReadoutPath p = choose_readout_path(dtype, d, bank->U, H, k_max);
     const ReadoutLayout L = readout_layout(bank->U, H, d, k_max, p.BM, p.grid);
     // work-item indices (group + slice) and item ranges are 32-bit.  The limit
-    // counts 32-row query tiles on the CUDA-core path, more than its kernel has.
-    const int limit_rows = p.kind == 1 ? p.BM : 32;
+    // counts 32-row query tiles on the CUDA-core path and 128-row ones on the
+    // tensor cores, at least as many as the kernels have.
+    const int limit_rows = p.kind == 0 ? 32 : 128;
     const int64_t limit_groups = (int64_t)bank->U * H * (k_max > 0 ? (k_max + limit_rows - 1) / limit_rows : 1);
     if (limit_groups + p.grid >= ((int64_t)1 << 30)) return RS3_EUNSUPPORTED;
     if (workspace_bytes < L.total) return RS3_ECAPACITY;
@@ -619,6 +634,10 @@ rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, in
     // left a 32 x 32 fp32 frame on half the CTAs (68 us against 61)
     a->tensor = p.kind != 0;
     a->plan_ov = p.kind == 1 ? 12 : 1;
+    if (p.kind == 2) {             // 128-key tiles: 3 and 12 slots, and slices of 2 and 6, are slower
+        a->plan_ov = 6;
+        a->min_chunk = 4;
+    }
     a->max_slots = L.max_slots;
     a->max_items = L.max_items;
     a->grid_ctas = p.grid;
@@ -662,6 +681,7 @@ rs3_status launch_plan(const ReadoutArgs &a, cudaStream_t st, rs3_dtype dtype)
 // the attention kernel over the plan in the workspace
 rs3_status launch_run(const ReadoutArgs &a, const ReadoutPath &p, rs3_dtype dtype, cudaStream_t st)
 {
+    if (p.kind == 2) return rs3_launch_pair_readout(a, st);
     if (p.kind == 1) return rs3_launch_tc_readout(a, st);
     return rs3_launch_simt_readout(a, dtype, st);
 }

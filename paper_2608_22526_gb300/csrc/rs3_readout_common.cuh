@@ -40,15 +40,16 @@ struct ReadoutArgs {
 };
 
 struct ReadoutPath {
-    int kind;   // 0 = CUDA-core, 1 = tensor-core (tcgen05)
+    int kind;   // 0 = CUDA-core, 1 = tensor-core (tcgen05), 2 = tensor-core, two query tiles
     int BM, BN;
     int grid;   // CTAs of the readout launch
 };
 
-ReadoutPath choose_readout_path(rs3_dtype dtype, int d);
+ReadoutPath choose_readout_path(rs3_dtype dtype, int d, int U, int H, int k_max);
 bool rs3_tc_supported(int d);
 int rs3_tc_block_n(int d);
 rs3_status rs3_launch_tc_readout(const ReadoutArgs &a, cudaStream_t st);
+rs3_status rs3_launch_pair_readout(const ReadoutArgs &a, cudaStream_t st);   // d = 64, 128
 // CUDA-core path: rows and keys of a tile and resident CTAs per SM, for a head width
 void rs3_simt_tile(int d, int &bm, int &bn, int &ctas_per_sm);
 rs3_status rs3_launch_simt_readout(const ReadoutArgs &a, rs3_dtype dtype, cudaStream_t st);

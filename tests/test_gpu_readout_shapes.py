@@ -110,6 +110,13 @@ def test_tile_edges(dtype, H, d, rope, n_ptr):
     _case(dtype, H, d, COUNTS, ROWS, n_ptr=n_ptr, rope=rope)
 
 
+@pytest.mark.parametrize("dtype,H,d", [("bf16", 2, 64), ("bf16", 1, 128), ("f32", 1, 64)])
+@pytest.mark.parametrize("part", range(4))
+def test_tile_edges_of_few_units(dtype, H, d, part):
+    """Too few query tiles for two per CTA."""
+    _case(dtype, H, d, COUNTS[part::4], ROWS[part::4], n_ptr=3, rope=part % 2 == 1)
+
+
 @pytest.mark.parametrize("dtype,H,d", [("f32", 2, 64), ("f32", 1, 256), ("bf16", 2, 64), ("bf16", 1, 128), ("bf16", 1, 256)])
 def test_one_group_cut_over_every_slice(dtype, H, d):
     """One unit with few queries: its keys are spread over all CTAs and merged."""
@@ -121,3 +128,4 @@ def test_rising_scores_move_the_reference(dtype, H, d):
     """Scores that grow along the bank by far more than 2^8 between tiles: the
     running reference moves and what is accumulated is rescaled."""
     _case(dtype, H, d, [200, 3, 129, 64], [1200, 900, 700, 1000], ramp=3.0)
+    _case(dtype, H, d, [256, 3, 129, 64, 250, 255, 1, 128, 500, 512] * 2, [1200, 900, 700, 1000, 130, 1100, 600, 257, 384, 128] * 2, ramp=3.0)
