@@ -37,29 +37,6 @@ namespace {
 
 enum { PMODE_EMPTY = 0, PMODE_MASK = 1, PMODE_BOX = 2 };
 
-// Chebyshev dilation of sIn by r into out(i) (called per cell after the row
-// pass).  Row pass: sTmp[y][x] = OR sIn[y][x-r .. x+r].
-__device__ void row_pass(const uint8_t *sIn, uint8_t *sTmp, int m, int n, int r)
-{
-    const int mn = m * n;
-    for (int i = threadIdx.x; i < mn; i += blockDim.x) {
-        const int y = i / n, x = i - y * n;
-        const int xa = max(0, x - r), xb = min(n - 1, x + r);
-        uint8_t v = 0;
-        for (int xx = xa; xx <= xb && !v; ++xx) v |= sIn[y * n + xx];
-        sTmp[i] = v;
-    }
-}
-
-__device__ __forceinline__ uint8_t col_value(const uint8_t *sTmp, int m, int n, int r, int i)
-{
-    const int y = i / n, x = i - y * n;
-    const int ya = max(0, y - r), yb = min(m - 1, y + r);
-    uint8_t v = 0;
-    for (int yy = ya; yy <= yb && !v; ++yy) v |= sTmp[yy * n + x];
-    return v;
-}
-
 // ---------------------------------------------------------------------------
 // canonical fp32 ||z||^2 (Eq. 5): eight channels of one lane's partial sum
 // ---------------------------------------------------------------------------
@@ -209,20 +186,12 @@ __device__ __forceinline__ uint32_t dsmem_ld(uint32_t a)
     return v;
 }
 
-// The prior of one unit ORed into P (words of WW per row), with `a` and `b` as
-// scratch; thread 0 gets the unit's new tracker state in t.  Every thread of
-// the CTA calls it.
-__device__ void unit_prior(const uint8_t *__restrict__ M, int m, int n, const WordWalk &walk,
-                           const rs3_track *__restrict__ track, int r_s, int c, int bbox_mode, uint32_t *P,
-                           uint32_t *a, uint32_t *b, rs3_track &t)
+// A mask's cells as bit words: f(y, k, words k and k + 1 of row y), by every
+// lane of the warp that loaded them (four rows of two words at a time).
+template <typename F>
+__device__ __forceinline__ void mask_words(const uint8_t *__restrict__ M, int m, int n, int WW, F f)
 {
-    __shared__ int s_box[4][SEL_WARPS];
-    __shared__ int s_mode, s_r, s_b[4];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int WW = walk.WW, words = m * WW;
-    if (threadIdx.x == 0) t = *track;
-    // the mask's bits and its box: a warp takes four rows of two words at a time
-    int y0 = INT_MAX, x0 = INT_MAX, y1 = -1, x1 = -1;
     for (int yb = warp; yb < m; yb += 4 * SEL_WARPS)
         for (int k = 0; k < WW; k += 2) {
             const uint8_t *row = M + yb * n + 32 * k + lane;
@@ -239,18 +208,71 @@ __device__ void unit_prior(const uint8_t *__restrict__ M, int m, int n, const Wo
                 const int y = yb + q * SEL_WARPS;
                 if (y >= m) break;
                 const uint32_t b0 = __ballot_sync(0xffffffffu, v0[q] != 0), b1 = __ballot_sync(0xffffffffu, v1[q] != 0);
-                if (lane == 0) {
-                    a[y * WW + k] = b0;
-                    if (k + 1 < WW) a[y * WW + k + 1] = b1;
-                }
-                if (b0 | b1) {
-                    y0 = min(y0, y);
-                    y1 = max(y1, y);
-                    x0 = min(x0, 32 * k + (b0 ? __ffs(b0) - 1 : __ffs(b1) + 31));
-                    x1 = max(x1, 32 * k + (b1 ? 63 - __clz(b1) : 31 - __clz(b0)));
-                }
+                f(y, k, b0, b1);
             }
         }
+}
+
+// Chebyshev dilation of bit words by r: along the rows, by at most 31 cells (a
+// neighbouring word) at a time, between the buffers a and b; returns the one
+// that holds the result ...
+__device__ __forceinline__ uint32_t *dilate_rows(uint32_t *a, uint32_t *b, int words, int n, int r, const WordWalk &walk)
+{
+    const int WW = walk.WW;
+    const uint32_t last = n & 31 ? (1u << (n & 31)) - 1u : 0xffffffffu;   // cells of a row's last word
+    uint32_t *from = a, *to = b;
+    // (beyond the row's length every cell of a row with a set one is set)
+    for (int left = min(r, n); left > 0; left -= 31) {
+        const int step = min(left, 31);
+        walk.each(words, [&](int w, int, int k) {
+            const uint32_t x = from[w], pv = k > 0 ? from[w - 1] : 0u, nx = k < WW - 1 ? from[w + 1] : 0u;
+            uint32_t o = x;
+            for (int d = 1; d <= step; ++d) o |= __funnelshift_r(x, nx, d) | __funnelshift_l(pv, x, d);
+            to[w] = k == WW - 1 ? o & last : o;
+        });
+        __syncthreads();
+        uint32_t *tmp = from;
+        from = to;
+        to = tmp;
+    }
+    return from;
+}
+
+// ... and over the rows: word w of row y.
+__device__ __forceinline__ uint32_t column_or(const uint32_t *from, int w, int y, int m, int r, int WW)
+{
+    const int up = min(r, y), down = min(r, m - 1 - y);
+    uint32_t o = 0u;
+#pragma unroll 4
+    for (int d = -up; d <= down; ++d) o |= from[w + d * WW];
+    return o;
+}
+
+// The prior of one unit ORed into P (words of WW per row), with `a` and `b` as
+// scratch; thread 0 gets the unit's new tracker state in t.  Every thread of
+// the CTA calls it.
+__device__ void unit_prior(const uint8_t *__restrict__ M, int m, int n, const WordWalk &walk,
+                           const rs3_track *__restrict__ track, int r_s, int c, int bbox_mode, uint32_t *P,
+                           uint32_t *a, uint32_t *b, rs3_track &t)
+{
+    __shared__ int s_box[4][SEL_WARPS];
+    __shared__ int s_mode, s_r, s_b[4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int WW = walk.WW, words = m * WW;
+    if (threadIdx.x == 0) t = *track;
+    int y0 = INT_MAX, x0 = INT_MAX, y1 = -1, x1 = -1;
+    mask_words(M, m, n, WW, [&](int y, int k, uint32_t b0, uint32_t b1) {
+        if (lane == 0) {
+            a[y * WW + k] = b0;
+            if (k + 1 < WW) a[y * WW + k + 1] = b1;
+        }
+        if (b0 | b1) {
+            y0 = min(y0, y);
+            y1 = max(y1, y);
+            x0 = min(x0, 32 * k + (b0 ? __ffs(b0) - 1 : __ffs(b1) + 31));
+            x1 = max(x1, 32 * k + (b1 ? 63 - __clz(b1) : 31 - __clz(b0)));
+        }
+    });
     if (lane == 0) { s_box[0][warp] = y0; s_box[1][warp] = x0; s_box[2][warp] = y1; s_box[3][warp] = x1; }
     __syncthreads();
     if (warp == 0) {
@@ -280,28 +302,8 @@ __device__ void unit_prior(const uint8_t *__restrict__ M, int m, int n, const Wo
     __syncthreads();
     const int mode = s_mode, r = s_r;
     if (mode == PMODE_MASK) {
-        // along the rows, by at most 31 cells (a neighbouring word) at a time
-        const uint32_t last = n & 31 ? (1u << (n & 31)) - 1u : 0xffffffffu;   // cells of a row's last word
-        uint32_t *from = a, *to = b;
-        for (int left = r; left > 0; left -= 31) {
-            const int step = min(left, 31);
-            walk.each(words, [&](int w, int, int k) {
-                const uint32_t x = from[w], pv = k > 0 ? from[w - 1] : 0u, nx = k < WW - 1 ? from[w + 1] : 0u;
-                uint32_t o = x;
-                for (int d = 1; d <= step; ++d) o |= __funnelshift_r(x, nx, d) | __funnelshift_l(pv, x, d);
-                to[w] = k == WW - 1 ? o & last : o;
-            });
-            __syncthreads();
-            uint32_t *tmp = from; from = to; to = tmp;
-        }
-        // and over the rows
-        walk.each(words, [&](int w, int y, int) {
-            const int up = min(r, y), down = min(r, m - 1 - y);
-            uint32_t o = 0u;
-#pragma unroll 4
-            for (int d = -up; d <= down; ++d) o |= from[w + d * WW];
-            P[w] |= o;
-        });
+        const uint32_t *from = dilate_rows(a, b, words, n, r, walk);
+        walk.each(words, [&](int w, int y, int) { P[w] |= column_or(from, w, y, m, r, WW); });
     } else if (mode == PMODE_BOX) {
         const int by0 = s_b[0] - r, bx0 = max(s_b[1] - r, 0), by1 = s_b[2] + r, bx1 = min(s_b[3] + r, n - 1);
         walk.each(words, [&](int w, int y, int k) {
@@ -624,42 +626,54 @@ k_select(const T *__restrict__ z, const uint8_t *__restrict__ masks, int m, int 
 }
 
 // ---------------------------------------------------------------------------
-// k_write_keepset: Eq. 8 with the 5% / 95% fall-through of Sec. 3.2
+// k_write_keepset: Eq. 8 with the 5% / 95% fall-through of Sec. 3.2, a CTA per
+// unit on bit words: 64 x 64 cells, radius 12, took 16.5 us (cold) cell by cell.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024)
-k_write_keepset(const uint8_t *__restrict__ seeds, const int32_t *__restrict__ unit_group, int U,
-                int G_unused, int m, int n, int D_w, double fall_lo, double fall_hi,
-                int fall_through, int union_mode, uint8_t *__restrict__ kw, int32_t *status)
+__global__ void __launch_bounds__(SEL_THREADS)
+k_write_keepset(const uint8_t *__restrict__ seeds, const int32_t *__restrict__ unit_group, int U, int m, int n,
+                int D_w, double fall_lo, double fall_hi, int fall_through, int union_mode, uint8_t *__restrict__ kw)
 {
     pdl_wait();
-    extern __shared__ __align__(16) uint8_t smem[];
-    const int mn = m * n;
-    const int u = blockIdx.x;
-    uint8_t *sS = smem;
-    uint8_t *sT = smem + ((mn + 15) & ~15);
-    const int g = unit_group[u];
-    for (int i = threadIdx.x; i < mn; i += blockDim.x) sS[i] = seeds[(size_t)u * mn + i] != 0;
-    __syncthreads();
-    if (union_mode) {
-        for (int v = 0; v < U; ++v) {
-            if (v == u || unit_group[v] != g) continue;
-            for (int i = threadIdx.x; i < mn; i += blockDim.x) sS[i] |= seeds[(size_t)v * mn + i] != 0;
+    extern __shared__ __align__(16) uint8_t sel_raw[];
+    const int mn = m * n, WW = (n + 31) >> 5, words = m * WW, u = blockIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *a = reinterpret_cast<uint32_t *>(sel_raw), *b = a + words;
+    const WordWalk walk(WW);
+    mask_words(seeds + (size_t)u * mn, m, n, WW, [&](int y, int k, uint32_t b0, uint32_t b1) {
+        if (lane == 0) {
+            a[y * WW + k] = b0;
+            if (k + 1 < WW) a[y * WW + k + 1] = b1;
         }
-        __syncthreads();
+    });
+    if (union_mode) {
+        const int g = unit_group[u];
+        for (int v0 = 0; v0 < U; v0 += 32) {
+            uint32_t in = __ballot_sync(0xffffffffu, v0 + lane < U && v0 + lane != u && unit_group[min(v0 + lane, U - 1)] == g);
+            for (; in; in &= in - 1)                       // (a word is always the same warp's)
+                mask_words(seeds + (size_t)(v0 + __ffs(in) - 1) * mn, m, n, WW, [&](int y, int k, uint32_t b0, uint32_t b1) {
+                    if (lane == 0) {
+                        a[y * WW + k] |= b0;
+                        if (k + 1 < WW) a[y * WW + k + 1] |= b1;
+                    }
+                });
+        }
     }
-    uint32_t area_local = 0;
-    for (int i = threadIdx.x; i < mn; i += blockDim.x) area_local += sS[i];
-    uint32_t area;
-    block_excl_scan(area_local, area);
+    __syncthreads();
+    uint32_t own = 0, area;
+    for (int w = threadIdx.x; w < words; w += SEL_THREADS) own += __popc(a[w]);
+    block_excl_scan(own, area);
     const double frac = (double)area / (double)mn;
     uint8_t *out = kw + (size_t)u * mn;
     if (fall_through && (frac > fall_hi || frac < fall_lo)) {
-        for (int i = threadIdx.x; i < mn; i += blockDim.x) out[i] = 1;
+        for (int i = threadIdx.x; i < mn; i += SEL_THREADS) out[i] = 1;
         return;
     }
-    row_pass(sS, sT, m, n, D_w);
+    uint32_t *from = dilate_rows(a, b, words, n, D_w, walk), *to = from == a ? b : a;
+    walk.each(words, [&](int w, int y, int) { to[w] = column_or(from, w, y, m, D_w, WW); });
     __syncthreads();
-    for (int i = threadIdx.x; i < mn; i += blockDim.x) out[i] = col_value(sT, m, n, D_w, i);
+    for (int y = warp; y < m; y += SEL_WARPS)
+        for (int k = 0; k < WW; ++k)
+            if (32 * k + lane < n) out[y * n + 32 * k + lane] = (uint8_t)(to[y * WW + k] >> lane & 1u);
 }
 
 inline int next_pow2(int x)
@@ -781,12 +795,11 @@ extern "C" rs3_status rs3_write_keepset(const uint8_t *seed_masks, const int32_t
     if (!seed_masks || !unit_group || !p || !kw_out || !status) return RS3_EINVAL;
     if (U < 1 || m < 1 || n < 1 || p->D_w < 0) return RS3_EINVAL;
     if ((long)m * n > RS3_MAX_MN) return RS3_EUNSUPPORTED;
-    const int mn = m * n;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const size_t smem = 2 * (size_t)((mn + 15) & ~15);
-    launch_pdl(k_write_keepset, dim3(U), dim3(1024), smem, st, seed_masks, unit_group, U, 0, m, n, p->D_w, p->fall_lo,
-                                           p->fall_hi, p->fall_through, p->union_mode, kw_out,
-                                           status);
+    const size_t smem = 2 * (size_t)m * ((n + 31) / 32) * 4;
+    if (rs3_kernel_smem((const void *)k_write_keepset, smem + 1024) != RS3_OK) return RS3_ECUDA;   // + its static arrays
+    launch_pdl(k_write_keepset, dim3(U), dim3(SEL_THREADS), smem, st, seed_masks, unit_group, U, m, n, p->D_w,
+               p->fall_lo, p->fall_hi, p->fall_through, p->union_mode, kw_out);
     if (cudaGetLastError() != cudaSuccess) return RS3_ECUDA;
     return RS3_OK;
 }
