@@ -50,13 +50,11 @@ __device__ __forceinline__ void copy_row(uint4 *__restrict__ dk, uint4 *__restri
 
 // Eq. 7 on the key side: one 16-byte piece of a key row (bf16: four pairs,
 // fp32: two pairs; element 2i and 2i + 1 of a head form pair i) rotated by
-// the (cos, sin) of those pairs at the row's own cell, in fp32, then rounded
-// once to the stored type.  f points at the first pair's (cos, sin).
-__device__ __forceinline__ uint4 rotate_piece(uint4 v, const float *__restrict__ f, int esz)
+// the (cos, sin) of those pairs at the row's own cell (a: the first two pairs',
+// b: the next two), in fp32, then rounded once to the stored type.
+__device__ __forceinline__ uint4 rotate_piece(uint4 v, float4 a, float4 b, int esz)
 {
     if (esz == 2) {
-        const float4 a = __ldg(reinterpret_cast<const float4 *>(f));
-        const float4 b = __ldg(reinterpret_cast<const float4 *>(f) + 1);
         const float cs[4] = {a.x, a.z, b.x, b.z}, sn[4] = {a.y, a.w, b.y, b.w};
         uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -69,7 +67,6 @@ __device__ __forceinline__ uint4 rotate_piece(uint4 v, const float *__restrict__
         }
         return make_uint4(w[0], w[1], w[2], w[3]);
     }
-    const float4 a = __ldg(reinterpret_cast<const float4 *>(f));
     const float x0 = __uint_as_float(v.x), x1 = __uint_as_float(v.y);
     const float x2 = __uint_as_float(v.z), x3 = __uint_as_float(v.w);
     return make_uint4(__float_as_uint(x0 * a.x - x1 * a.y), __float_as_uint(x0 * a.y + x1 * a.x),
@@ -84,75 +81,118 @@ __device__ __forceinline__ int nonzero_bytes(uint4 w)
 }
 
 // The commit of one frame, in one launch: CTA (c, u) owns cells
-// [c * CHUNK, (c+1) * CHUNK) of unit u, one cell per thread (CHUNK = 128, or
-// 64 where 128-cell chunks would give fewer than two CTAs per SM).
-// Its latency chain is two memory round trips: (1) the chunk's own mask bytes
-// and the unit's whole mask row (the kept rows before the chunk and in the
-// unit) are loaded together; (2) as soon as the chunk's kept cells are ranked
-// (ballot / popc) their first K and V pieces are loaded into registers, and
-// the unit's counts and the eviction / capacity decision (thread 0, from the
-// old counters) are made while those loads are in flight; then the pieces
-// are stored at their ring rows.  Every CTA arrives on the unit's counter
-// once thread 0 has read the old counters, and the last to arrive publishes
-// the new ones after its own stores, so no CTA can read counters of the frame
-// it copies (the readers of the bank are later launches).
-constexpr int COMMIT_PF = 8;        // kept rows per warp and batch (one piece per lane and row)
+// [c * CHUNK, (c+1) * CHUNK) of unit u (CHUNK = 128, or 64 where 128-cell
+// chunks would give fewer than two CTAs per SM); its warps copy PF rows each at
+// a time.
+// Its latency chain is two memory round trips: (1) the chunk's own mask bytes;
+// (2) once its kept cells are ranked (ballot / popc), the first rows' K and V
+// pieces (and the RoPE angles of the keys), together with the unit's mask row,
+// whose count before the chunk and in the unit give the rows' places and the
+// eviction / capacity decision (thread 0, from the old counters); then the
+// pieces are stored.  Objects are compact, so most chunks keep no cell: those
+// read nothing more.  Every CTA arrives on the unit's counter, with its kept
+// cells, once it has read what it needs of the old counters, and the last to
+// arrive publishes the new ones, so no CTA can read counters of the frame it
+// copies (the readers of the bank are later launches).
+// 48 units of 96 x 96 cells (130 MB, 19 us at the copy rate): 42.4 us with keys
+// rotated, 32.4 as given; 46.5 and 35 when every chunk counted its unit's mask,
+// a batch was 32 rows of 4 warps, and the angles were loaded after the keys.
+
+// A batch of pieces in registers.
+template <bool ROPE, int PF>
+struct CommitBatch {
+    uint4 k[PF], v[PF];
+    float4 f[ROPE ? PF : 1][2];
+};
 
 // Loads piece v of rows j0, j0 + NW, ... of the chunk's kept list (NW warps).
-template <int NW>
-__device__ __forceinline__ void commit_load(uint4 (&kk)[COMMIT_PF], uint4 (&vv)[COMMIT_PF],
-                                            const int32_t *s_list, int nk, int j0, int v, int nvec,
-                                            const uint8_t *ksrc, const uint8_t *vsrc, int64_t row_bytes)
+template <int NW, bool ROPE, int PF>
+__device__ __forceinline__ void commit_load(CommitBatch<ROPE, PF> &b, const int32_t *s_list, int nk, int j0, int v,
+                                            int nvec, const uint8_t *ksrc, const uint8_t *vsrc, int64_t row_bytes,
+                                            const float *rope, int d, int esz)
 {
 #pragma unroll
-    for (int r = 0; r < COMMIT_PF; ++r) {
+    for (int r = 0; r < PF; ++r) {
         const int j = j0 + NW * r;
         if (j < nk && v < nvec) {
             const int64_t so = (int64_t)s_list[j] * row_bytes + 16 * v;
-            kk[r] = __ldcs(reinterpret_cast<const uint4 *>(ksrc + so));
-            vv[r] = __ldcs(reinterpret_cast<const uint4 *>(vsrc + so));
+            b.k[r] = __ldcs(reinterpret_cast<const uint4 *>(ksrc + so));
+            b.v[r] = __ldcs(reinterpret_cast<const uint4 *>(vsrc + so));
+            if (ROPE) {                                    // the pairs of the piece, at the row's own cell
+                const int e = (16 * v) / esz;              // first element of the piece
+                const float4 *f = reinterpret_cast<const float4 *>(rope + ((int64_t)s_list[j] * (d / 2) + (e % d) / 2) * 2);
+                b.f[r][0] = __ldg(f);
+                if (esz == 2) b.f[r][1] = __ldg(f + 1);
+            }
         }
     }
 }
 
 // Stores those pieces at bank row row0 + j (a ring position, wrapped once,
 // past the pinned region; or a pinned row for a conditioning frame).
-template <int NW, bool ROPE>
-__device__ __forceinline__ void commit_store(const uint4 (&kk)[COMMIT_PF], const uint4 (&vv)[COMMIT_PF],
-                                             const int32_t *s_list, int nk, int j0, int v, int nvec,
-                                             int64_t row0, int is_cond, const BankDev &bk,
-                                             uint8_t *kdst, uint8_t *vdst, int64_t row_bytes,
-                                             const float *rope, int d, int esz)
+template <int NW, bool ROPE, int PF>
+__device__ __forceinline__ void commit_store(const CommitBatch<ROPE, PF> &b, int nk, int j0, int v, int nvec,
+                                             int64_t row0, int is_cond, const BankDev &bk, uint8_t *kdst,
+                                             uint8_t *vdst, int64_t row_bytes, int esz)
 {
 #pragma unroll
-    for (int r = 0; r < COMMIT_PF; ++r) {
+    for (int r = 0; r < PF; ++r) {
         const int j = j0 + NW * r;
         if (j < nk && v < nvec) {
             int64_t row = row0 + j;
             if (!is_cond) row = bk.pinned_cap + (row >= bk.ring_cap ? row - bk.ring_cap : row);
             const int64_t dst = row * row_bytes + 16 * v;
-            uint4 k = kk[r];
-            if (ROPE) {                                    // keys stored rotated by their own cell
-                const int e = (16 * v) / esz;              // first element of the piece
-                k = rotate_piece(k, rope + ((int64_t)s_list[j] * (d / 2) + (e % d) / 2) * 2, esz);
-            }
-            *reinterpret_cast<uint4 *>(kdst + dst) = k;
-            *reinterpret_cast<uint4 *>(vdst + dst) = vv[r];
+            *reinterpret_cast<uint4 *>(kdst + dst) = ROPE ? rotate_piece(b.k[r], b.f[r][0], b.f[r][1], esz) : b.k[r];
+            *reinterpret_cast<uint4 *>(vdst + dst) = b.v[r];
         }
     }
 }
 
-template <int CHUNK, bool ROPE>
-__global__ void __launch_bounds__(CHUNK)
+// A unit's counters before the commit, and what becomes of them.
+struct CommitState {
+    int64_t head, tail, nf, oldest, cond_len, ncond;
+    bool ok;
+    __device__ __forceinline__ void load(const int64_t *mu)
+    {
+        head = mu[BM_HEAD]; tail = mu[BM_TAIL];
+        nf = mu[BM_NFRAMES]; oldest = mu[BM_OLDEST];
+        cond_len = mu[BM_COND_LEN]; ncond = mu[BM_NCOND];
+        ok = false;
+    }
+    __device__ __forceinline__ bool sane(const BankDev &bk) const
+    {
+        return head >= 0 && tail >= head && nf >= 0 && nf <= bk.max_frames && oldest >= 0 && oldest < bk.max_frames;
+    }
+    // Eviction and capacity for a frame of L rows; returns the place of its row
+    // `pre` (a pinned row, or a ring position).
+    __device__ __forceinline__ int64_t decide(const int64_t *mu, const BankDev &bk, int is_cond, int64_t L, int64_t pre)
+    {
+        if (is_cond) {
+            ok = ncond < bk.n_cond && cond_len + L <= bk.pinned_cap;
+            return cond_len + pre;
+        }
+        if (!sane(bk)) return 0;
+        if (bk.window > 0 && nf == bk.window) {              // evict the oldest ring frame
+            head += mu[BM_HEADER_WORDS + bk.max_frames + oldest];
+            oldest = oldest + 1 == bk.max_frames ? 0 : oldest + 1;
+            nf -= 1;
+        }
+        ok = nf < bk.max_frames && (tail - head) + L <= bk.ring_cap;
+        return ok && L > 0 ? (tail + pre) % bk.ring_cap : 0; // it fits: rows wrap at most once
+    }
+};
+
+template <int CHUNK, bool ROPE, int THREADS, int PF, int MB>
+__global__ void __launch_bounds__(THREADS, MB)
 k_commit(const uint8_t *__restrict__ k_new, const uint8_t *__restrict__ v_new,
          const uint8_t *__restrict__ mask, int mn, int is_cond, int64_t row_bytes, BankDev bk,
          uint8_t *__restrict__ k_store, uint8_t *__restrict__ v_store, int32_t *status,
          const float *__restrict__ rope, int d, int esz)
 {
-    constexpr int NW = CHUNK / 32;
+    constexpr int NW = THREADS / 32, CW = CHUNK / 32;     // warps; warps with cells
     pdl_wait();
     __shared__ int32_t s_list[CHUNK];
-    __shared__ int32_t s_wc[NW];
+    __shared__ int32_t s_wc[CW];
     __shared__ int32_t s_red[2][NW];
     __shared__ int64_t s_row0;
     __shared__ int s_ok;
@@ -162,145 +202,115 @@ k_commit(const uint8_t *__restrict__ k_new, const uint8_t *__restrict__ v_new,
     int64_t *mu = bk.meta + (int64_t)u * bk.stride_words;
     const uint8_t *Mu = mask ? mask + (size_t)u * mn : nullptr;
 
-    // the unit's old counters (thread 0 decides for the CTA)
-    int64_t head0 = 0, tail0 = 0, nf0 = 0, oldest0 = 0, cond_len0 = 0, ncond0 = 0;
-    if (threadIdx.x == 0) {
-        head0 = mu[BM_HEAD]; tail0 = mu[BM_TAIL];
-        nf0 = mu[BM_NFRAMES]; oldest0 = mu[BM_OLDEST];
-        cond_len0 = mu[BM_COND_LEN]; ncond0 = mu[BM_NCOND];
-    }
-
-    // round trip 1: this thread's cell, and the kept rows of the unit and of
-    // the chunks before this one (16-byte loads when the unit's mask row is
-    // aligned, bytes for the rest)
+    // the unit's old counters (thread 0 decides for the CTA), and round trip 1:
+    // this thread's cell
+    CommitState st;
+    if (threadIdx.x == 0) st.load(mu);
     const int cell = c0 + threadIdx.x;
-    const bool keep = cell < mn && (Mu ? Mu[cell] != 0 : true);
-    int total = 0, before = 0;
-    if (Mu) {
-        const int nvec16 = (reinterpret_cast<uintptr_t>(Mu) & 15u) == 0 ? (mn >> 4) : 0;
-#pragma unroll 4
-        for (int i = threadIdx.x; i < nvec16; i += CHUNK) {
-            const int c = nonzero_bytes(__ldg(reinterpret_cast<const uint4 *>(Mu) + i));
-            total += c;
-            before += i * 16 < c0 ? c : 0;
-        }
-        for (int i = nvec16 * 16 + threadIdx.x; i < mn; i += CHUNK) {
-            const int c = Mu[i] != 0;
-            total += c;
-            before += i < c0 ? c : 0;
-        }
-    }
-
+    const bool keep = threadIdx.x < CHUNK && cell < mn && (Mu ? Mu[cell] != 0 : true);
     // ranks of the chunk's kept cells, in cell order
     const uint32_t bal = __ballot_sync(0xffffffffu, keep);
-    if (lane == 0) s_wc[warp] = __popc(bal);
+    if (lane == 0 && warp < CW) s_wc[warp] = __popc(bal);
     __syncthreads();
     int off = 0, nk = 0;
 #pragma unroll
-    for (int w = 0; w < NW; ++w) {
+    for (int w = 0; w < CW; ++w) {
         off += w < warp ? s_wc[w] : 0;
         nk += s_wc[w];
     }
-    if (keep) {
-        uint32_t lm;
-        asm("mov.u32 %0, %%lanemask_lt;" : "=r"(lm));
-        s_list[off + __popc(bal & lm)] = cell;
-    }
-    __syncthreads();
+    if (nk > 0) {                                            // uniform over the CTA
+        if (keep) {
+            uint32_t lm;
+            asm("mov.u32 %0, %%lanemask_lt;" : "=r"(lm));
+            s_list[off + __popc(bal & lm)] = cell;
+        }
+        __syncthreads();
 
-    // round trip 2: the first batch of the chunk's rows in flight ...
-    const int nvec = (int)(row_bytes / 16);
-    const uint8_t *ksrc = k_new + (size_t)u * mn * row_bytes;
-    const uint8_t *vsrc = v_new + (size_t)u * mn * row_bytes;
-    uint4 kk[COMMIT_PF], vv[COMMIT_PF];
-    commit_load<NW>(kk, vv, s_list, nk, warp, lane, nvec, ksrc, vsrc, row_bytes);
+        // round trip 2: the first batch of the chunk's rows ...
+        const int nvec = (int)(row_bytes / 16);
+        const uint8_t *ksrc = k_new + (size_t)u * mn * row_bytes;
+        const uint8_t *vsrc = v_new + (size_t)u * mn * row_bytes;
+        CommitBatch<ROPE, PF> b;
+        commit_load<NW, ROPE, PF>(b, s_list, nk, warp, lane, nvec, ksrc, vsrc, row_bytes, rope, d, esz);
 
-    // ... while the unit's counts are summed and thread 0 decides
-    if (Mu) {
-        total = warp_sum(total);
-        before = warp_sum(before);
-        if (lane == 0) { s_red[0][warp] = total; s_red[1][warp] = before; }
-    }
-    __syncthreads();
-    bool ok = false;
-    int64_t L = 0, head = head0, oldest = oldest0, nf = nf0;
-    if (threadIdx.x == 0) {
-        int64_t pre = 0;
+        // ... and the kept rows of the unit and of the chunks before this one
+        // (16-byte loads when the unit's mask row is aligned, bytes for the rest)
         if (Mu) {
+            int total = 0, before = 0;
+            const int nvec16 = (reinterpret_cast<uintptr_t>(Mu) & 15u) == 0 ? (mn >> 4) : 0;
+#pragma unroll 4
+            for (int i = threadIdx.x; i < nvec16; i += THREADS) {
+                const int c = nonzero_bytes(__ldg(reinterpret_cast<const uint4 *>(Mu) + i));
+                total += c;
+                before += i * 16 < c0 ? c : 0;
+            }
+            for (int i = nvec16 * 16 + threadIdx.x; i < mn; i += THREADS) {
+                const int c = Mu[i] != 0;
+                total += c;
+                before += i < c0 ? c : 0;
+            }
+            total = __reduce_add_sync(0xffffffffu, total);
+            before = __reduce_add_sync(0xffffffffu, before);
+            if (lane == 0) { s_red[0][warp] = total; s_red[1][warp] = before; }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int64_t L = mn, pre = c0;
+            if (Mu) {
+                L = pre = 0;
 #pragma unroll
-            for (int w = 0; w < NW; ++w) { L += s_red[0][w]; pre += s_red[1][w]; }
-        } else {
-            L = mn;
-            pre = c0;
+                for (int w = 0; w < NW; ++w) { L += s_red[0][w]; pre += s_red[1][w]; }
+            }
+            CommitState after = st;
+            s_row0 = after.decide(mu, bk, is_cond, L, pre);
+            s_ok = after.ok;
         }
-        int64_t row0 = 0;
-        if (is_cond) {
-            ok = ncond0 < bk.n_cond && cond_len0 + L <= bk.pinned_cap;
-            row0 = cond_len0 + pre;
-        } else {
-            const bool sane = head0 >= 0 && tail0 >= head0 && nf0 >= 0 && nf0 <= bk.max_frames &&
-                              oldest0 >= 0 && oldest0 < bk.max_frames;
-            if (!sane) {
-                if (ch == 0) latch_status(status, RS3_EINTERNAL);
-            } else {
-                if (bk.window > 0 && nf == bk.window) {      // evict the oldest ring frame
-                    head += mu[BM_HEADER_WORDS + bk.max_frames + oldest];
-                    oldest = oldest + 1 == bk.max_frames ? 0 : oldest + 1;
-                    nf -= 1;
+        __syncthreads();
+        if (s_ok) {
+            const int64_t row0 = s_row0;
+            uint8_t *kdst = k_store + (size_t)u * bk.rows_per_unit * row_bytes;
+            uint8_t *vdst = v_store + (size_t)u * bk.rows_per_unit * row_bytes;
+            commit_store<NW, ROPE, PF>(b, nk, warp, lane, nvec, row0, is_cond, bk, kdst, vdst, row_bytes, esz);
+            // the rest of the chunk (rows past the first batch, pieces past 32 per row)
+            for (int vb = 0; vb < nvec; vb += 32)
+                for (int jb = vb == 0 ? NW * PF : 0; jb < nk; jb += NW * PF) {
+                    commit_load<NW, ROPE, PF>(b, s_list, nk, jb + warp, vb + lane, nvec, ksrc, vsrc, row_bytes, rope, d, esz);
+                    commit_store<NW, ROPE, PF>(b, nk, jb + warp, vb + lane, nvec, row0, is_cond, bk, kdst, vdst, row_bytes, esz);
                 }
-                ok = nf < bk.max_frames && (tail0 - head) + L <= bk.ring_cap;
-                if (ok && L > 0) row0 = (tail0 + pre) % bk.ring_cap;   // it fits: rows wrap at most once
-            }
-        }
-        s_ok = ok;
-        s_row0 = row0;
-    }
-    __syncthreads();
-
-    // every read of the old counters by this CTA is done: arrive
-    unsigned long long arrived = 0;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        arrived = atomicAdd(reinterpret_cast<unsigned long long *>(mu + BM_ARRIVE), 1ull);
-    }
-
-    if (s_ok) {
-        const int64_t row0 = s_row0;
-        uint8_t *kdst = k_store + (size_t)u * bk.rows_per_unit * row_bytes;
-        uint8_t *vdst = v_store + (size_t)u * bk.rows_per_unit * row_bytes;
-        commit_store<NW, ROPE>(kk, vv, s_list, nk, warp, lane, nvec, row0, is_cond, bk, kdst, vdst,
-                               row_bytes, rope, d, esz);
-        // the rest of the chunk (rows past the first batch, pieces past 32 per row)
-        for (int vb = 0; vb < nvec; vb += 32) {
-            for (int jb = vb == 0 ? NW * COMMIT_PF : 0; jb < nk; jb += NW * COMMIT_PF) {
-                commit_load<NW>(kk, vv, s_list, nk, jb + warp, vb + lane, nvec, ksrc, vsrc, row_bytes);
-                commit_store<NW, ROPE>(kk, vv, s_list, nk, jb + warp, vb + lane, nvec, row0, is_cond, bk, kdst,
-                                       vdst, row_bytes, rope, d, esz);
-            }
         }
     }
 
-    // the last CTA of the unit to arrive publishes the new counters
-    if (threadIdx.x != 0 || arrived != (unsigned long long)(gridDim.x - 1)) return;
+    // every read of the old counters by this CTA is done: arrive, with its kept
+    // cells (high half); the last CTA of the unit to arrive publishes
+    if (threadIdx.x != 0) return;
     __threadfence();
+    const unsigned long long arrived = atomicAdd(reinterpret_cast<unsigned long long *>(mu + BM_ARRIVE),
+                                                 ((unsigned long long)nk << 32) + 1ull);
+    if ((uint32_t)arrived != gridDim.x - 1) return;
+    __threadfence();
+    const int64_t L = (int64_t)(arrived >> 32) + nk;
+    const int64_t tail0 = st.tail;
+    if (!is_cond && !st.sane(bk)) latch_status(status, RS3_EINTERNAL);
+    const bool latch = is_cond || (st.head >= 0 && st.tail >= st.head);
+    st.decide(mu, bk, is_cond, L, 0);
     mu[BM_ARRIVE] = 0;
-    if (!ok) {
-        if (is_cond || (head0 >= 0 && tail0 >= head0)) latch_status(status, RS3_ECAPACITY);
+    if (!st.ok) {
+        if (latch) latch_status(status, RS3_ECAPACITY);
         return;
     }
     if (is_cond) {
-        mu[BM_COND_LEN] = cond_len0 + L;
-        mu[BM_NCOND] = ncond0 + 1;
+        mu[BM_COND_LEN] = st.cond_len + L;
+        mu[BM_NCOND] = st.ncond + 1;
     } else {
         int64_t *fo = mu + BM_HEADER_WORDS;
         int64_t *fl = fo + bk.max_frames;
-        const int64_t slot = (oldest + nf) % bk.max_frames;
+        const int64_t slot = (st.oldest + st.nf) % bk.max_frames;
         fo[slot] = tail0;
         fl[slot] = L;
-        mu[BM_HEAD] = head;
+        mu[BM_HEAD] = st.head;
         mu[BM_TAIL] = tail0 + L;
-        mu[BM_NFRAMES] = nf + 1;
-        mu[BM_OLDEST] = oldest;
+        mu[BM_NFRAMES] = st.nf + 1;
+        mu[BM_OLDEST] = st.oldest;
     }
 }
 
@@ -414,11 +424,23 @@ rs3_status commit_launch(const rs3_bank *bank, const void *k_new, const void *v_
     const bool small = (int64_t)((mn + 127) / 128) * bank->U < 2ll * rs3_sm_count();
     const int chunk = small ? 64 : 128;
     const dim3 grid((unsigned)((mn + chunk - 1) / chunk), (unsigned)bank->U);
+    // Warps copying a chunk and rows in flight per warp (us per call, the others
+    // measured for the same shapes): rotated keys, 3 CTAs of 8 warps x 4 rows,
+    // 16 x 3 objects 42.4 (2 rows 39.4, but 26.6 against 22.4 on 12 objects;
+    // 4 CTAs 50.7, spilled); keys as given, small launches 8 warps x 4 rows 8.4
+    // (4 x 8: 10.1), large ones 4 x 8 32.4 (8 x 4: 36.7).
+    int threads = 256;
     void (*kern)(const uint8_t *, const uint8_t *, const uint8_t *, int, int, int64_t, BankDev, uint8_t *,
-                 uint8_t *, int32_t *, const float *, int, int) =
-        small ? (rope ? k_commit<64, true> : k_commit<64, false>)
-              : (rope ? k_commit<128, true> : k_commit<128, false>);
-    launch_pdl(kern, grid, dim3(chunk), 0, st,
+                 uint8_t *, int32_t *, const float *, int, int);
+    if (rope) {
+        kern = small ? k_commit<64, true, 256, 4, 3> : k_commit<128, true, 256, 4, 3>;
+    } else if (small) {
+        kern = k_commit<64, false, 256, 4, 4>;
+    } else {
+        kern = k_commit<128, false, 128, 8, 4>;
+        threads = 128;
+    }
+    launch_pdl(kern, grid, dim3(threads), 0, st,
         static_cast<const uint8_t *>(k_new), static_cast<const uint8_t *>(v_new), keep_mask, mn, is_cond,
         row_bytes, bk, static_cast<uint8_t *>(bank->k_store), static_cast<uint8_t *>(bank->v_store), status,
         rope, bank->d, elem_bytes(bank->dtype));
