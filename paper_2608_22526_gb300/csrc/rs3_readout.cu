@@ -3,11 +3,11 @@
 // pieces of both kernel paths.
 //
 // Launch sequence (no host synchronisation).  Attend phase:
-//   k_passthrough  out-of-place only: out = residual (or zeros) on every cell
 //   k_plan         one CTA: per unit, the bank's row ranges (pinned, ring
 //                  pieces, pointers) and a balanced work list of
 //                  (unit, head, query tile, KV tile range) items; long banks
-//                  are split along the keys so every SM gets work
+//                  are split along the keys so every SM gets work; out of place
+//                  the launch's other CTAs write out = residual (or zeros)
 //   k_readout_*    flash attention per item: gather the kept query rows (and
 //                  rotate them), stream the bank tiles, online softmax in the
 //                  log2 domain, fp32 accumulation; an unsplit item writes
@@ -25,17 +25,6 @@
 #include "rs3_readout_common.cuh"
 
 namespace {
-
-// ---------------------------------------------------------------------------
-// k_passthrough: unselected cells equal the residual bit for bit (Eq. 6 S_K)
-// ---------------------------------------------------------------------------
-__global__ void k_passthrough(const uint4 *__restrict__ res, uint4 *__restrict__ out, int64_t nvec)
-{
-    pdl_wait();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvec;
-         i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = res ? __ldcs(res + i) : make_uint4(0, 0, 0, 0);
-}
 
 // ---------------------------------------------------------------------------
 // k_plan: ranges and the work list
@@ -181,10 +170,17 @@ __device__ void plan_slice(const ReadoutArgs &a, const PlanView &v, int b, int &
     c.pad[0] = b;
     c.pad[1] = c.pad[2] = 0;                      // pad[1]: the unit's kept queries
     n_part = 0;
+    if (lo >= hi) {
+        a.cta_items[2 * b] = a.cta_items[2 * b + 1] = 0;
+        return;
+    }
+    // one search and its divisions for the slice's first group; the walk from
+    // there counts (16 x 3 objects, 12 groups a slice: 32 us for a search each)
+    int u, gl;
+    int64_t off;
+    locate(v, lo, u, gl, off);
+    int qt = gl / v.H, h = gl - qt * v.H;
     for (int64_t x = lo; x < hi;) {
-        int u, gl;
-        int64_t off;
-        locate(v, x, u, gl, off);
         const int64_t wg = v.wg[u];
         const int64_t len = min(hi - x, wg - off);
         const int64_t nt = v.nt[u];
@@ -196,7 +192,7 @@ __device__ void plan_slice(const ReadoutArgs &a, const PlanView &v, int b, int &
             const bool whole = t0 == 0 && t1 == nt;
             const int64_t idx = (int64_t)v.gb[u] + gl + b;
             WorkItem w;
-            w.u = u; w.qt = gl / v.H; w.h = gl % v.H; w.split = 0;
+            w.u = u; w.qt = qt; w.h = h; w.split = 0;
             w.tile_begin = (int32_t)t0;
             w.tile_end = (int32_t)t1;
             w.slot = whole ? -1 : 2 * b + (first < 0 ? 0 : 1);
@@ -218,6 +214,17 @@ __device__ void plan_slice(const ReadoutArgs &a, const PlanView &v, int b, int &
             }
         }
         x += len;
+        off += len;
+        if (off < wg) break;                        // the slice ends inside the group
+        off = 0;
+        ++gl;
+        if (++h == v.H) { h = 0; ++qt; }
+        if (gl == v.gb[u + 1] - v.gb[u]) {          // the next unit with groups
+            gl = qt = h = 0;
+            do ++u;
+            while (u < v.U && v.gb[u + 1] == v.gb[u]);
+            if (u == v.U) break;
+        }
     }
     a.cta_items[2 * b] = (int32_t)(first < 0 ? 0 : first);
     a.cta_items[2 * b + 1] = (int32_t)(first < 0 ? 0 : last + 1);
@@ -225,9 +232,20 @@ __device__ void plan_slice(const ReadoutArgs &a, const PlanView &v, int b, int &
 
 constexpr int PLAN_THREADS = 256;
 
-__global__ void __launch_bounds__(PLAN_THREADS) k_plan(ReadoutArgs a)
+// Out of place, CTAs 1.. of the launch also write out = residual (or zeros) on
+// every cell: unselected cells equal the residual bit for bit (Eq. 6 S_K), and
+// the copy hides the plan.
+__global__ void __launch_bounds__(PLAN_THREADS) k_plan(ReadoutArgs a, int64_t nvec)
 {
     pdl_wait();
+    if (blockIdx.x > 0) {
+        const uint4 *res = static_cast<const uint4 *>(a.residual);
+        uint4 *out = static_cast<uint4 *>(a.out);
+        for (int64_t i = (int64_t)(blockIdx.x - 1) * PLAN_THREADS + threadIdx.x; i < nvec;
+             i += (int64_t)(gridDim.x - 1) * PLAN_THREADS)
+            out[i] = res ? __ldcs(res + i) : make_uint4(0, 0, 0, 0);
+        return;
+    }
     ReadoutHeader *hdr = a.header;
     // [U+1] tb, [U] wg (int64); [U+1] gb, [U] nt (int32)
     extern __shared__ int64_t s_plan[];
@@ -662,19 +680,17 @@ namespace {
 // pass-through of the unselected cells (out of place only) and the plan
 rs3_status launch_plan(const ReadoutArgs &a, cudaStream_t st, rs3_dtype dtype)
 {
+    int64_t nvec = 0, blocks = 0;
     if (a.residual != a.out) {
-        const int64_t nvec = (int64_t)a.U * a.mn * a.D * (dtype == RS3_BF16 ? 2 : 4) / 16;
-        int64_t blocks = (nvec + 255) / 256;
+        nvec = (int64_t)a.U * a.mn * a.D * (dtype == RS3_BF16 ? 2 : 4) / 16;
+        blocks = (nvec + PLAN_THREADS - 1) / PLAN_THREADS;
         const int64_t cap = (int64_t)a.n_sm * 8;
         if (blocks > cap) blocks = cap;
-        launch_pdl(k_passthrough, dim3((unsigned)blocks), dim3(256), 0, st,
-                   static_cast<const uint4 *>(a.residual), static_cast<uint4 *>(a.out), nvec);
-        if (cudaGetLastError() != cudaSuccess) return RS3_ECUDA;
     }
     // plan shared memory: unit slot bases and widths (int64), group bases, tiles, kept queries (int32)
     const size_t plan_smem = (size_t)(2 * a.U + 1) * 8 + (size_t)(3 * a.U + 1) * 4;
     if (rs3_kernel_smem((const void *)k_plan, plan_smem) != RS3_OK) return RS3_EUNSUPPORTED;
-    launch_pdl(k_plan, dim3(1), dim3(PLAN_THREADS), plan_smem, st, a);
+    launch_pdl(k_plan, dim3((unsigned)(1 + blocks)), dim3(PLAN_THREADS), plan_smem, st, a, nvec);
     return cudaGetLastError() != cudaSuccess ? RS3_ECUDA : RS3_OK;
 }
 
