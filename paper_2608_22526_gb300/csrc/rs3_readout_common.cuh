@@ -116,6 +116,22 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
     return r;
 }
 
+// A 16-byte piece of a query row (four pairs) rotated by the (cos, sin) of those
+// pairs at f (Eq. 7), rounded once per element.
+__device__ __forceinline__ uint4 rotate_q_piece(uint4 v, const float *f)
+{
+    uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int p = 0; p < 4; p += 2) {
+        const float4 c = __ldg(reinterpret_cast<const float4 *>(f) + p / 2);
+        const float x0 = __uint_as_float(w[p] << 16), x1 = __uint_as_float(w[p] & 0xffff0000u);
+        const float y0 = __uint_as_float(w[p + 1] << 16), y1 = __uint_as_float(w[p + 1] & 0xffff0000u);
+        w[p] = pack_bf16x2(x0 * c.x - x1 * c.y, x0 * c.y + x1 * c.x);
+        w[p + 1] = pack_bf16x2(y0 * c.z - y1 * c.w, y0 * c.w + y1 * c.z);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // out[u][cell][c .. c+1] (store_out2) or [c .. c+3] (store_out4) =
 // residual[...] + o, rounded once to T
 template <typename T>

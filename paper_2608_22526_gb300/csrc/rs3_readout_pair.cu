@@ -89,18 +89,7 @@ __device__ __forceinline__ void store_q_row(uint32_t sq, int r, const uint16_t *
             v[c] = qrow ? __ldg(reinterpret_cast<const uint4 *>(qrow) + c0 + c) : make_uint4(0u, 0u, 0u, 0u);
         if (qrow && rope) {
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                uint32_t w[4] = {v[c].x, v[c].y, v[c].z, v[c].w};
-#pragma unroll
-                for (int p = 0; p < 4; p += 2) {
-                    const float4 f = __ldg(reinterpret_cast<const float4 *>(rope) + 2 * (c0 + c) + p / 2);
-                    const float x0 = __uint_as_float(w[p] << 16), x1 = __uint_as_float(w[p] & 0xffff0000u);
-                    const float y0 = __uint_as_float(w[p + 1] << 16), y1 = __uint_as_float(w[p + 1] & 0xffff0000u);
-                    w[p] = pack_bf16x2(x0 * f.x - x1 * f.y, x0 * f.y + x1 * f.x);
-                    w[p + 1] = pack_bf16x2(y0 * f.z - y1 * f.w, y0 * f.w + y1 * f.z);
-                }
-                v[c] = make_uint4(w[0], w[1], w[2], w[3]);
-            }
+            for (int c = 0; c < 8; ++c) v[c] = rotate_q_piece(v[c], rope + 8 * (c0 + c));
         }
 #pragma unroll
         for (int c = 0; c < 8; ++c)
