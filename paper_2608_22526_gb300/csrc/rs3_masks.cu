@@ -33,7 +33,7 @@
 // the object listed first.  close_shape() picks rows and KC.
 //
 // Each logit is read from DRAM once; halo re-reads by neighbouring tiles hit
-// L2.  16 streams x 3 objects of 384 x 384 (31 MB, 4.6 us at the copy rate): 18.5
+// L2.  16 streams x 3 objects of 384 x 384 (31 MB, 4.6 us at the copy rate): 18.1
 // us per call, half of the issue slots busy, mostly with the thresholds, the
 // argmax and its labels; 91 us with a scalar load and a ballot per 32 pixels,
 // general funnel-shift dilations and an 8-row halo per 16 rows on CTAs that
@@ -225,28 +225,13 @@ k_close_argmax(const float *__restrict__ logits, const int32_t *__restrict__ gst
     if (!sides)
         for (int p = t; p < 2 * nwin; p += CA_THREADS) sA[(p >> 1) * SW + (p & 1) * (NS + 1)] = make_uint4(0u, 0u, 0u, 0u);
     // where this lane's pixels lie in an object's image (-1: outside): the
-    // tile's rows, and the halo rows (the first 2R above the tile, the rest
-    // below); and, for s >= 4, their grid cell (4 cell + which of the four
-    // columns it takes)
+    // tile's rows, and the halo rows (the first 2R above the tile, the rest below)
     int off[NT], hoff[NH], goff[NT];
-    const int gm = h / s, gn = w / s;
-    const int gi0 = (r0 + s - 1) / s;                      // first grid row of the tile
-    uint32_t grows = 0u;                                   // which of its rows are grid rows
-    if (grid && s >= 4)
-        for (int k = gi0 * s - r0; k < brv; k += s) grows |= 1u << k;
-    constexpr int NX = NS == 3 ? 3 : 1;                    // a warp's tasks lie in one strip, unless NS = 3
-    int gx4[NX];
-#pragma unroll
-    for (int k = 0; k < NX; ++k) {
-        const int x = x0 + (NX == 1 ? warp % NS : k) * 128 + 4 * lane, gx = (x + s - 1) / s, c = gx * s - x;
-        gx4[k] = c < 4 ? 4 * gx + c : -1;
-    }
 #pragma unroll
     for (int i = 0; i < NT; ++i) {
-        const int p = warp + CA_WARPS * i, k = p / NS, x = x0 + (p % NS) * 128 + 4 * lane;
-        off[i] = p < brv * NS && x < w ? (r0 + k) * w + x : -1;
-        const int gx = NX == 1 ? gx4[0] : p % NS == 0 ? gx4[0] : p % NS == 1 ? gx4[1 % NX] : gx4[2 % NX];
-        goff[i] = off[i] >= 0 && gx >= 0 && (grows >> k & 1u) ? 4 * (gi0 + __popc(grows & ((1u << k) - 1u))) * gn + gx : -1;
+        const int p = warp + CA_WARPS * i, x = x0 + (p % NS) * 128 + 4 * lane;
+        off[i] = p < brv * NS && x < w ? (r0 + p / NS) * w + x : -1;
+        goff[i] = -1;
     }
 #pragma unroll
     for (int i = 0; i < NH; ++i) {
@@ -254,11 +239,34 @@ k_close_argmax(const float *__restrict__ logits, const int32_t *__restrict__ gst
         const int row = r0 - 2 * R + (j < 2 * R ? j : rows + j);
         hoff[i] = j < 4 * R && row >= 0 && row < h && x < w ? row * w + x : -1;
     }
+    int gm = 0, gn = 0;
+    // for s >= 4 their grid cell (4 cell + which of the four columns it takes);
+    // its divisions run while the first object's logits are on their way
+    const auto grid_cells = [&]() {
+        gm = h / s;
+        gn = w / s;
+        const int gi0 = (r0 + s - 1) / s;                  // first grid row of the tile
+        uint32_t grows = 0u;                               // which of its rows are grid rows
+        if (grid && s >= 4)
+            for (int k = gi0 * s - r0; k < brv; k += s) grows |= 1u << k;
+        constexpr int NX = NS == 3 ? 3 : 1;                // a warp's tasks lie in one strip, unless NS = 3
+        int gx4[NX];
+#pragma unroll
+        for (int k = 0; k < NX; ++k) {
+            const int x = x0 + (NX == 1 ? warp % NS : k) * 128 + 4 * lane, gx = (x + s - 1) / s, c = gx * s - x;
+            gx4[k] = c < 4 ? 4 * gx + c : -1;
+        }
+#pragma unroll
+        for (int i = 0; i < NT; ++i) {
+            const int p = warp + CA_WARPS * i, k = p / NS;
+            const int gx = NX == 1 ? gx4[0] : p % NS == 0 ? gx4[0] : p % NS == 1 ? gx4[1 % NX] : gx4[2 % NX];
+            goff[i] = off[i] >= 0 && gx >= 0 && (grows >> k & 1u) ? 4 * (gi0 + __popc(grows & ((1u << k) - 1u))) * gn + gx : -1;
+        }
+    };
     const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
     const uint32_t lane_bit = 1u << lane;
     for (int u = u0 + (int)rank; u < u1; u += KC) {
         const float *L = logits + (size_t)u * h * w;
-        uint8_t *gu = grid + (size_t)u * gm * gn;
         // 1. all of the object's loads, then its ballots: the tile, the halo
         //    and, in images wider than the tile, the 16 columns on either side
         float4 v[NT], hv[NH];
@@ -266,6 +274,8 @@ k_close_argmax(const float *__restrict__ logits, const int32_t *__restrict__ gst
         for (int i = 0; i < NT; ++i) v[i] = off[i] >= 0 ? load_logits<VEC>(L + off[i]) : none;
 #pragma unroll
         for (int i = 0; i < NH; ++i) hv[i] = hoff[i] >= 0 ? load_logits<VEC>(L + hoff[i]) : none;
+        if (u == u0 + (int)rank) grid_cells();
+        uint8_t *gu = grid + (size_t)u * gm * gn;
 #pragma unroll
         for (int i = 0; i < NT; ++i) {
             const int p = warp + CA_WARPS * i;
@@ -353,9 +363,11 @@ k_close_argmax(const float *__restrict__ logits, const int32_t *__restrict__ gst
             if (goff[i] >= 0) gu[goff[i] >> 2] = (uint8_t)(bytes >> 8 * (goff[i] & 3) & 1u);
             if (grid && s < 4 && off[i] >= 0) {            // several cells in the lane's four columns
                 const int row = r0 + p / NS, x = x0 + (p % NS) * 128 + 4 * lane;
-                if (row % s == 0)
-                    for (int gx = (x + s - 1) / s; gx * s < x + 4; ++gx)
-                        gu[row / s * gn + gx] = (uint8_t)(bytes >> 8 * (gx * s - x) & 1u);
+                const auto over_s = [s](int a) { return s == 1 ? a : s == 2 ? a >> 1 : a / 3; };
+                const int gy = over_s(row);
+                if (gy * s == row)
+                    for (int gx = over_s(x + s - 1); gx * s < x + 4; ++gx)
+                        gu[gy * gn + gx] = (uint8_t)(bytes >> 8 * (gx * s - x) & 1u);
             }
         }
     }
@@ -501,12 +513,12 @@ struct CloseShape {
 // of an object, where the cost counts the strip rows read (halo and all) and a
 // fixed part for the passes' latency, worth about 40 of them.  Two CTAs are
 // resident per SM; the rows tried are those that just fill one wave, 16 and 24.
-static CloseShape close_shape(int G, int objects, int h, int w)
+static CloseShape close_shape(int G, int objects, int h, int w, int R, int per_sm)
 {
     CloseShape best = {};
     best.ns = std::min(4, (w + 127) / 128);
     best.tiles_x = (w + 128 * best.ns - 1) / (128 * best.ns);
-    const int slots = 2 * rs3_sm_count();
+    const int slots = per_sm * rs3_sm_count();
     double least = 0.0;
     for (int KC = 1; KC <= objects; ++KC) {
         const long long columns = (long long)best.tiles_x * G * KC;     // CTAs per row of tiles
@@ -515,7 +527,7 @@ static CloseShape close_shape(int G, int objects, int h, int w)
         for (const int rows : {fit, 16, CA_ROWS}) {
             const long long ctas = columns * ((h + rows - 1) / rows);
             const double cost = (double)((ctas + slots - 1) / slots) * ((objects + KC - 1) / KC) *
-                                    (40.0 + (double)(rows + 16) * best.ns) + (KC > 1 ? 20.0 : 0.0);
+                                    (40.0 + (double)(rows + 4 * R) * best.ns) + (KC > 1 ? 20.0 : 0.0);
             if (best.KC == 0 || cost < least) {
                 least = cost;
                 best.rows = rows;
@@ -576,10 +588,12 @@ extern "C" rs3_status rs3_close_argmax(const float *logits, const int32_t *group
     // ranks past a stream's object count idle
     const int objects = std::min(8, std::max(1, (U + G - 1) / G));
     if ((long long)G * objects > 65535) return RS3_EUNSUPPORTED;
-    const CloseShape c = close_shape(G, objects, h, w);
     // 16-byte loads and 4-byte stores where the arrays allow them
     const auto low = [](const void *p) { return reinterpret_cast<uintptr_t>(p); };
     const bool vec = rs3_aligned16(logits) && ((low(palette) | low(closed)) & 3u) == 0;
+    // the kernel of a radius at run time takes twice the registers: one CTA per SM
+    // (3 objects of 480 x 480, radius 2: 14.5 us, 19.5 in two waves of smaller tiles)
+    const CloseShape c = close_shape(G, objects, h, w, radius, vec && radius == 4 ? 2 : 1);
     cudaError_t e;
     if (!vec)
         e = launch_close_strips<0, false>(c, h, G, st, logits, group_start, U, w, radius, s, palette,
