@@ -511,7 +511,7 @@ struct CloseShape {
 
 // Rows per tile and CTAs per cluster: the least waves x objects per CTA x cost
 // of an object, where the cost counts the strip rows read (halo and all) and a
-// fixed part for the passes' latency, worth about 40 of them.  Two CTAs are
+// fixed part for the passes' latency, worth about 40 of them.  `per_sm` CTAs are
 // resident per SM; the rows tried are those that just fill one wave, 16 and 24.
 static CloseShape close_shape(int G, int objects, int h, int w, int R, int per_sm)
 {

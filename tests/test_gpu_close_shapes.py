@@ -50,7 +50,7 @@ def test_radii(R):
 
 
 @pytest.mark.parametrize("objs,h,w,s", [([11, 0, 3], 52, 96, 4), ([1] * 40, 100, 256, 4), ([3] * 30, 96, 384, 6),
-                                        ([20], 23, 64, 1), ([9, 9], 384, 512, 32)])
+                                        ([20], 23, 64, 1), ([9, 9], 384, 512, 32), ([2, 2], 48, 288, 3)])
 def test_streams_and_rows(objs, h, w, s):
     _check(objs, h, w, 4, s, 500 + h)
 
