@@ -145,9 +145,11 @@ __device__ __forceinline__ uint32_t cluster_rank()
 
 // every thread of every CTA of the cluster arrives, then waits (the release /
 // acquire pair orders shared-memory writes before the barrier with reads of
-// them through DSMEM after it)
+// them through DSMEM after it).  .aligned: a warp's lanes execute it together,
+// also after a loop or a branch that some of them left early
 __device__ __forceinline__ void cluster_barrier()
 {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
                  "barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }

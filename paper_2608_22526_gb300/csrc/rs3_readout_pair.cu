@@ -447,6 +447,7 @@ k_readout_pair(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk, con
                         res[k] = a.residual ? __ldg(reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(a.residual) + ooff + c0) + k)
                                             : make_uint4(0u, 0u, 0u, 0u);
                 }
+                __syncwarp();                                          // rows without a query took no part above
                 if (n > 0) {
                     tmem_ld32(ocol + (uint32_t)c0, o);
                     tmem_wait_ld();

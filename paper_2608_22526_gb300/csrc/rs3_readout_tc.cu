@@ -564,6 +564,7 @@ k_readout_tc(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk,
                                                 : make_uint4(0u, 0u, 0u, 0u);
                     }
                     uint32_t o[16 * EG];
+                    __syncwarp();                          // rows without a query took no part above
                     if (n > 0) {
 #pragma unroll
                         for (int e = 0; e < EG; ++e) tmem_ld16(tl + (uint32_t)(col0 + 16 * e), o + 16 * e);

@@ -129,3 +129,13 @@ def test_rising_scores_move_the_reference(dtype, H, d):
     running reference moves and what is accumulated is rescaled."""
     _case(dtype, H, d, [200, 3, 129, 64], [1200, 900, 700, 1000], ramp=3.0)
     _case(dtype, H, d, [256, 3, 129, 64, 250, 255, 1, 128, 500, 512] * 2, [1200, 900, 700, 1000, 130, 1100, 600, 257, 384, 128] * 2, ramp=3.0)
+
+
+@pytest.mark.parametrize("d", [64, 128, 256])
+def test_partial_query_tiles_of_whole_items(d):
+    """More groups than CTAs, so that most items hold a whole group and write their
+    rows directly: warps in which only some rows have a query, a warp with none
+    beside them, over every chunk of columns of the epilogue."""
+    counts = [1, 31, 33, 100, 127, 129, 160, 5, 97, 140, 180, 65] * 15
+    rows = [70, 129, 64, 200, 33, 140, 65, 257, 10, 128, 130, 90] * 15
+    _case("bf16", 1, d, counts, rows, rope=True, seed=3)
