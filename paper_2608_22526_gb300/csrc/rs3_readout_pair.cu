@@ -198,36 +198,38 @@ k_readout_pair(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk, con
             // ------------------------------------------------------------------
             // TMA producer: tile t's K, then tile t's V
             // ------------------------------------------------------------------
-            uint32_t cnt = 0;
+            uint32_t ck = 0, cv = 0;                                   // K and V tiles issued
             bool ok = true;
             for (int it = it_begin; it < it_end && ok; ++it) {
                 const WorkItem w = a.items[it];
                 const RangeSet *rs = a.ranges + w.u;
-                for (int t = w.tile_begin; t < w.tile_end; ++t, ++cnt) {
+                for (int t = w.tile_begin; t < w.tile_end; ++t) {
                     int64_t row0;
                     int nvalid;
                     tile_rows(rs, t, BN, row0, nvalid);
                     const int y = (int)((int64_t)w.u * a.rows_per_unit + row0);
-                    const uint32_t ks = cnt % KSTK, vs = cnt % KSTV;
-                    if (!mbar_wait(BAR(C::B_KEMPTY + ks), ((cnt / KSTK) & 1u) ^ 1u, abort_flag, wait_ns)) { ok = false; break; }
+                    const uint32_t ks = ck % KSTK, vs = cv % KSTV;
+                    ok = mbar_wait(BAR(C::B_KEMPTY + ks), ((ck / KSTK) & 1u) ^ 1u, abort_flag, wait_ns);
+                    if (!ok) break;
                     mbar_expect_tx(BAR(C::B_KFULL + ks), (uint32_t)C::KVBYTES);
 #pragma unroll
                     for (int c = 0; c < DH / 64; ++c)
                         tma_load_2d(sK + ks * C::KVBYTES + c * (BN * 128), &tmk, BAR(C::B_KFULL + ks), w.h * DH + c * 64, y);
-                    if (!mbar_wait(BAR(C::B_VEMPTY + vs), ((cnt / KSTV) & 1u) ^ 1u, abort_flag, wait_ns)) {
-                        mbar_drain(BAR(C::B_KFULL + ks), (cnt / KSTK) & 1u);
-                        ok = false;
-                        break;
-                    }
+                    ++ck;
+                    ok = mbar_wait(BAR(C::B_VEMPTY + vs), ((cv / KSTV) & 1u) ^ 1u, abort_flag, wait_ns);
+                    if (!ok) break;
                     mbar_expect_tx(BAR(C::B_VFULL + vs), (uint32_t)C::KVBYTES);
 #pragma unroll
                     for (int c = 0; c < DH / 64; ++c)
                         tma_load_2d(sV + vs * C::KVBYTES + c * (BN * 128), &tmv, BAR(C::B_VFULL + vs), w.h * DH + c * 64, y);
+                    ++cv;
                 }
             }
-            // let every copy this thread issued land before the CTA can exit
-            for (uint32_t k = (cnt > KSTK ? cnt - KSTK : 0); k < cnt; ++k) mbar_drain(BAR(C::B_KFULL + k % KSTK), (k / KSTK) & 1u);
-            for (uint32_t k = (cnt > KSTV ? cnt - KSTV : 0); k < cnt; ++k) mbar_drain(BAR(C::B_VFULL + k % KSTV), (k / KSTV) & 1u);
+            // let every copy this thread issued land before the CTA can exit: the
+            // last one of each stage (a stage's earlier phases have been consumed, and
+            // a wait for one of them would run into the phase after the last)
+            for (uint32_t k = (ck > KSTK ? ck - KSTK : 0); k < ck; ++k) mbar_drain(BAR(C::B_KFULL + k % KSTK), (k / KSTK) & 1u);
+            for (uint32_t k = (cv > KSTV ? cv - KSTV : 0); k < cv; ++k) mbar_drain(BAR(C::B_VFULL + k % KSTV), (k / KSTV) & 1u);
         } else if (warp == 1 || warp == 2) {
             // ------------------------------------------------------------------
             // MMA issuer of query tile q (the whole warp walks, one thread issues).

@@ -231,3 +231,51 @@ def test_readout_wait_limit_runs_out_and_the_context_stays_usable():
         others = np.setdiff1d(np.arange(w.mn), keep)
         assert np.array_equal(out[0][others], x[0][others])
     assert pipe.status_code() == 0
+
+
+@pytest.mark.parametrize("H,d", [(4, 64), (2, 128), (1, 256)])
+def test_readout_gives_up_at_any_wait_without_delay(H, d):
+    """The waits run out at the first tile (0 ns) or in the middle of a CTA's work
+    (limits of the order of a tile's time), in each tensor-core kernel (two query
+    tiles per CTA at heads of 64 and 128).  The launch then drains its copies and
+    matrix operations, none of which takes a millisecond, so every call ends well
+    within the drain's own limit of one second; the next ordinary call finds its
+    tensor memory and is correct."""
+    import time
+    w = synth.Workload("limits", 11, 48, 48, H, d, "bf16", 1, 8, 4, 0.02, 0.4, 1, 3, 5)
+    pipe = Pipeline(w)
+    seq = synth.Sequence(w)
+    ob = orc.OracleBank(w.U, w.D, w.dtype, w.mn, w.n_cond, w.window, pipe.bank.ring_cap, pipe.bank.max_frames, w.n_ptr)
+    for s in range(3):
+        kn, vn = seq.kv_new(s)
+        pipe.commit(to_dev(kn), to_dev(vn), None, int(s == 0))
+        ob.commit(kn, vn, None, int(s == 0))
+    z = seq.z(3)
+    zd = to_dev(z)
+    pipe.select(zd, to_dev(seq.masks(2)))
+    out = torch.empty((w.U, w.mn, w.D), dtype=torch.bfloat16, device="cuda")
+    pipe.readout(zd, None, out)
+    torch.cuda.synchronize()
+    first = to_host(out).copy()
+    assert pipe.status_code() == 0
+    try:
+        for limit in (0, 300, 1000, 2000, 4000, 8000):
+            rs3.rs3_set_wait_limit_ns(limit)
+            t0 = time.perf_counter()
+            pipe.readout(zd, None, out)
+            torch.cuda.synchronize()
+            assert time.perf_counter() - t0 < 0.5, limit
+            code = pipe.status_code()
+            assert code == rs3.RS3_ETIMEOUT if limit == 0 else code in (0, rs3.RS3_ETIMEOUT), (limit, code)
+            pipe.status.zero_()
+    finally:
+        rs3.rs3_set_wait_limit_ns(10 ** 9)
+    pipe.readout(zd, None, out)
+    torch.cuda.synchronize()
+    assert pipe.status_code() == 0
+    again = to_host(out)
+    assert np.array_equal(again, first)
+    keep = to_host(pipe.idx)[0, : int(pipe.count[0].item())]
+    K, V = ob.kv(0)
+    A = orc.readout(z[0], w.dtype, w.H, w.d, keep[:64], K, V, w.dtype, threads=8)
+    check_readout(w.dtype, again[0][keep[:64]], A, Report(), "after the timeouts")
