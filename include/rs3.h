@@ -278,7 +278,12 @@ rs3_status rs3_bank_read_meta(const rs3_bank *bank, int64_t *host_out, int64_t *
 /* ------------------------------------------------------------------------ */
 
 /* Bytes of device workspace rs3_memory_readout needs for these sizes (the
- * work list, and the split-KV partial results of long banks). */
+ * work list, and the split-KV partial results of long banks).  It never falls
+ * as U, H or k_max grows, so a workspace sized for the largest of several calls
+ * serves all of them.  The size allows the fastest kernel; a workspace with room
+ * for the partial results of 256 query rows per SM is enough for a slower one
+ * (about half the size: bf16 heads of 64 and 128, fp32 heads up to 64), and
+ * RS3_ECAPACITY is returned only below that. */
 size_t rs3_readout_workspace_bytes(int U, int H, int d, int k_max, rs3_dtype dtype);
 
 /*

@@ -19,8 +19,10 @@
 // rs3_memory_readout_attend / _merge issue one each.
 #include "rs3_internal.cuh"
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <initializer_list>
 
 #include "rs3_readout_common.cuh"
 
@@ -515,8 +517,9 @@ namespace {
 // Bounds of the stream-K plan: item indices < groups + CTAs (group + slice);
 // a CTA has at most two partial items (slots 2b, 2b + 1); at most one merge
 // entry per CTA and per group.
-ReadoutLayout readout_layout(int U, int H, int d, int k_max, int BM, int grid)
+ReadoutLayout readout_layout(int U, int H, int d, int k_max, const ReadoutPath &p)
 {
+    const int BM = p.BM, grid = p.grid;
     ReadoutLayout L;
     const int64_t nq = k_max > 0 ? (k_max + BM - 1) / BM : 1;
     const int64_t groups = (int64_t)U * H * nq;
@@ -559,7 +562,12 @@ extern "C" uint64_t rs3_get_wait_limit_ns(void) { return g_wait_ns.load(); }
 // other below that (10 tiles 22.6 against 25.6; 20 tiles of heads of 128 31.8
 // against 37.2), and where a pair of tiles would often be half empty (3 tiles
 // per head, 72 in all: 25.5 against 27.0).
-ReadoutPath choose_readout_path(rs3_dtype dtype, int d, int U, int H, int k_max)
+//
+// A workspace that is too small for the kernel's partial results but holds those
+// of 256 rows per SM takes a smaller path: the one-tile kernel, or one CTA per SM
+// on the CUDA cores.  rs3_readout_workspace_bytes returns at least that for
+// every kernel, so a workspace sized for one call serves every smaller one.
+ReadoutPath choose_readout_path(rs3_dtype dtype, int d, int U, int H, int k_max, size_t workspace_bytes)
 {
     ReadoutPath p;
     const int n_sm = rs3_sm_count();
@@ -570,24 +578,39 @@ ReadoutPath choose_readout_path(rs3_dtype dtype, int d, int U, int H, int k_max)
         p.BN = rs3_tc_block_n(d);
         p.grid = n_sm;                 // one persistent CTA per SM
         if (d <= 128 && (int64_t)U * H * single >= 40 && 8 * pairs <= 5 * single) {
-            p.kind = 2;
-            p.BM = 256;                // two query tiles per item
-            p.BN = 128;
+            ReadoutPath two = p;
+            two.kind = 2;
+            two.BM = 256;              // two query tiles per item
+            two.BN = 128;
+            if (readout_layout(U, H, d, k_max, two).total <= workspace_bytes) p = two;
         }
     } else {
         int ctas;
         p.kind = 0;
         rs3_simt_tile(d, p.BM, p.BN, ctas);
         p.grid = ctas * n_sm;
+        if (ctas > 1 && readout_layout(U, H, d, k_max, p).total > workspace_bytes) p.grid = n_sm;
     }
     return p;
 }
 
+// What the preferred path of this call needs, and no less than a call of fewer
+// queries, units or heads may: a keep-set of three query tiles is left to the
+// one-tile kernel where one of two takes the other.
 extern "C" size_t rs3_readout_workspace_bytes(int U, int H, int d, int k_max, rs3_dtype dtype)
 {
     if (U < 1 || H < 1 || d < 1 || k_max < 0) return 0;
-    const ReadoutPath p = choose_readout_path(dtype, d, U, H, k_max);
-    return readout_layout(U, H, d, k_max, p.BM, p.grid).total;
+    size_t need = 0;
+    ReadoutPath floor;                 // 256 rows of partial results per SM
+    floor.kind = 1;
+    floor.BM = 128;
+    floor.BN = 0;
+    floor.grid = rs3_sm_count();
+    for (const int k : {k_max, k_max < 256 ? k_max : 256}) {
+        const ReadoutPath p = choose_readout_path(dtype, d, U, H, k, SIZE_MAX);
+        need = std::max(need, readout_layout(U, H, d, k_max, p).total);
+    }
+    return std::max(need, readout_layout(U, H, d, k_max, floor).total);
 }
 
 rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, int H, int d,
@@ -609,8 +632,8 @@ rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, in
     if (!rs3_aligned16(q) || !rs3_aligned16(out) || !rs3_aligned16(workspace) ||
         (residual && !rs3_aligned16(residual)) || (rope && !rs3_aligned16(rope)))
         return RS3_EINVAL;
-    const ReadoutPath p = choose_readout_path(dtype, d, bank->U, H, k_max);
-    const ReadoutLayout L = readout_layout(bank->U, H, d, k_max, p.BM, p.grid);
+    const ReadoutPath p = choose_readout_path(dtype, d, bank->U, H, k_max, workspace_bytes);
+    const ReadoutLayout L = readout_layout(bank->U, H, d, k_max, p);
     // work-item indices (group + slice) and item ranges are 32-bit.  The limit
     // counts 32-row query tiles on the CUDA-core path and 128-row ones on the
     // tensor cores, at least as many as the kernels have.

@@ -45,7 +45,8 @@ struct ReadoutPath {
     int grid;   // CTAs of the readout launch
 };
 
-ReadoutPath choose_readout_path(rs3_dtype dtype, int d, int U, int H, int k_max);
+// the path of a call with this workspace (SIZE_MAX: the path that any workspace is sized for)
+ReadoutPath choose_readout_path(rs3_dtype dtype, int d, int U, int H, int k_max, size_t workspace_bytes);
 bool rs3_tc_supported(int d);
 int rs3_tc_block_n(int d);
 rs3_status rs3_launch_tc_readout(const ReadoutArgs &a, cudaStream_t st);

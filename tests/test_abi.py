@@ -90,6 +90,19 @@ def test_workspace_sizes(binding):
     assert 0 < b <= c
 
 
+@pytest.mark.parametrize("dtype,d", [(t, d) for t in ("bf16", "f32") for d in (16, 32, 64, 128, 256)])
+def test_readout_workspace_never_falls_as_a_call_grows(binding, dtype, d):
+    size = binding.rs3_readout_workspace_bytes
+    ks = [0, 1, 64, 127, 128, 129, 255, 256, 257, 300, 384, 385, 512, 513, 640, 641, 768, 769, 1228, 2764, 9216, 16384]
+    for U, H in [(1, 1), (1, 4), (5, 4), (7, 2), (8, 4), (20, 2), (40, 1), (48, 4)]:
+        sizes = [size(U, H, d, k, dtype) for k in ks]
+        assert sizes == sorted(sizes), (U, H, sizes)
+        assert all(size(U, H, d, k, dtype) <= size(U + 1, H, d, k, dtype) for k in ks)
+        assert all(size(U, H, d, k, dtype) <= size(U, H + 1, d, k, dtype) for k in ks)
+        # no smaller for one type than what the other's smaller kernel takes
+        assert all(size(U, H, d, k, dtype) >= 256 * 148 * (4 * d + 8) for k in ks)
+
+
 def test_null_arguments_are_rejected_on_host(binding):
     lib = binding.lib
     p = binding.default_params()

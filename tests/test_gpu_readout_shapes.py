@@ -34,7 +34,7 @@ def _check(dtype, got, exact, vmax, rope, what):
         assert float(err.max()) <= F32_REL * max(float(np.abs(exact).max()), 1e-30), f"{what}: {err.max()}"
 
 
-def _case(dtype, H, d, counts, rows, n_ptr=0, rope=False, sharp=1.0, ramp=0.0, seed=0):
+def _case(dtype, H, d, counts, rows, n_ptr=0, rope=False, sharp=1.0, ramp=0.0, seed=0, ws_bytes=None):
     """One group, a unit per (count, rows) pair: `rows` bank rows in two ring
     frames, then n_ptr pointer rows.  ramp > 0 makes later keys score higher,
     so that a row's softmax reference has to move."""
@@ -70,7 +70,8 @@ def _case(dtype, H, d, counts, rows, n_ptr=0, rope=False, sharp=1.0, ramp=0.0, s
     res = _draw(rng, dtype, (U, mn, D))
     tab = rng.uniform(0, 6.28, (mn, d // 2)) if rope else None
     table = np.ascontiguousarray(np.stack([np.cos(tab), np.sin(tab)], -1).astype(np.float32)) if rope else None
-    ws = torch.empty(rs3.rs3_readout_workspace_bytes(U, H, d, k_max, dtype), dtype=torch.uint8, device="cuda")
+    ws_bytes = rs3.rs3_readout_workspace_bytes(U, H, d, k_max, dtype) if ws_bytes is None else ws_bytes
+    ws = torch.empty(ws_bytes, dtype=torch.uint8, device="cuda")
     ug = torch.zeros(U, dtype=torch.int32, device="cuda")
     cnt = torch.tensor(counts, dtype=torch.int32, device="cuda")
     out = to_dev(res)
@@ -139,3 +140,29 @@ def test_partial_query_tiles_of_whole_items(d):
     counts = [1, 31, 33, 100, 127, 129, 160, 5, 97, 140, 180, 65] * 15
     rows = [70, 129, 64, 200, 33, 140, 65, 257, 10, 128, 130, 90] * 15
     _case("bf16", 1, d, counts, rows, rope=True, seed=3)
+
+
+def _one_tile_bytes(U, H, d, k_max):
+    """Workspace of 256 rows of partial results per SM: header, a range set per
+    unit, item ranges, items, merge entries, (O, m, l) per row."""
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    up = lambda x: (x + 255) // 256 * 256
+    groups = U * H * max(1, -(-k_max // 128))
+    return (up(128) + up(8 * n_sm) + up(96 * U) + up(32 * (groups + n_sm)) + up(32 * min(groups, n_sm)) +
+            up(256 * n_sm * d * 4) + up(256 * n_sm * 8))
+
+
+@pytest.mark.parametrize("dtype,H,d", [("bf16", 4, 64), ("bf16", 4, 128), ("f32", 2, 64)])
+def test_smaller_calls_in_a_workspace_sized_for_the_largest(dtype, H, d):
+    """Keep-sets of two query tiles in a workspace sized for three (which the
+    one-tile kernel serves, with half the partial rows), and every path in a
+    workspace that only the smaller one fits; less than that is refused."""
+    U, counts = 8, [200, 256, 3, 129, 255, 64, 130, 250]
+    rows = [300, 150, 700, 64, 900, 129, 40, 500]
+    _case(dtype, H, d, counts, rows, ws_bytes=rs3.rs3_readout_workspace_bytes(U, H, d, 384, dtype))
+    least = _one_tile_bytes(U, H, d, 256)
+    assert least < rs3.rs3_readout_workspace_bytes(U, H, d, 256, dtype)
+    _case(dtype, H, d, counts, rows, rope=True, n_ptr=5, ws_bytes=least)
+    with pytest.raises(rs3.RS3Error) as e:
+        _case(dtype, H, d, counts, rows, ws_bytes=least - 256)
+    assert e.value.code == rs3.RS3_ECAPACITY
