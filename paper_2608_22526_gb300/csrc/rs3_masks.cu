@@ -344,23 +344,25 @@ k_close_argmax(const float *__restrict__ logits, const int32_t *__restrict__ gst
             const uint4 cw = sC[p];
             const bool bit[4] = {(cw.x & lane_bit) != 0, (cw.y & lane_bit) != 0, (cw.z & lane_bit) != 0,
                                  (cw.w & lane_bit) != 0};
-            const float vv[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
-            float bv[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-            uint32_t bl = 0u;
-            if (!first) {
-                const float4 b = sBV[p * 32 + lane];
-                bv[0] = b.x; bv[1] = b.y; bv[2] = b.z; bv[3] = b.w;
-                bl = sBL[p * 32 + lane];
-            }
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                if (bit[c] && vv[c] > bv[c]) {
-                    bv[c] = vv[c];
-                    bl = __byte_perm(bl, lab, c == 0 ? 0x3214 : c == 1 ? 0x3240 : c == 2 ? 0x3410 : 0x4210);
-                }
-            sBV[p * 32 + lane] = make_float4(bv[0], bv[1], bv[2], bv[3]);
-            sBL[p * 32 + lane] = bl;
             const uint32_t bytes = (uint32_t)bit[0] | (uint32_t)bit[1] << 8 | (uint32_t)bit[2] << 16 | (uint32_t)bit[3] << 24;
+            // a pixel without a label takes the object's whatever its logit
+            if (first) {
+                sBV[p * 32 + lane] = v[i];
+                sBL[p * 32 + lane] = bytes * lab;
+            } else if ((cw.x | cw.y | cw.z | cw.w) != 0u) {    // (the same for the warp)
+                const float vv[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+                const float4 best = sBV[p * 32 + lane];
+                float bv[4] = {best.x, best.y, best.z, best.w};
+                uint32_t bl = sBL[p * 32 + lane];
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (bit[c] && (vv[c] > bv[c] || (bl & 255u << 8 * c) == 0u)) {
+                        bv[c] = vv[c];
+                        bl = __byte_perm(bl, lab, c == 0 ? 0x3214 : c == 1 ? 0x3240 : c == 2 ? 0x3410 : 0x4210);
+                    }
+                sBV[p * 32 + lane] = make_float4(bv[0], bv[1], bv[2], bv[3]);
+                sBL[p * 32 + lane] = bl;
+            }
             if (closed && off[i] >= 0) store_bytes<VEC>(closed + (size_t)u * h * w + off[i], bytes);
             if (goff[i] >= 0) gu[goff[i] >> 2] = (uint8_t)(bytes >> 8 * (goff[i] & 3) & 1u);
             if (grid && s < 4 && off[i] >= 0) {            // several cells in the lane's four columns

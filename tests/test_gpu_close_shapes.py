@@ -20,9 +20,11 @@ def _off(t, skew):
     return buf[skew:].view(t.shape)
 
 
-def _check(objs, h, w, R, s, seed, skew=0):
+def _check(objs, h, w, R, s, seed, skew=0, punch=None):
     rng = np.random.default_rng(seed)
     L = synth.decoder_logits(rng, sum(objs), h, w)
+    if punch is not None:                # one pixel in twenty of every object
+        L[rng.random(L.shape) < 0.05] = punch
     U, G = sum(objs), len(objs)
     gs = np.concatenate([[0], np.cumsum(objs)]).astype(np.int32)
     mk = lambda *shape: _off(torch.full(shape, 77, dtype=torch.uint8, device="cuda"), skew)
@@ -59,3 +61,13 @@ def test_streams_and_rows(objs, h, w, s):
 def test_unaligned_arrays(skew):
     _check([2, 1], 40, 160, 4, 4, 600 + skew, skew=skew)
     _check([2, 1], 40, 160, 3, 4, 600 + skew, skew=skew)
+
+
+@pytest.mark.parametrize("skew", [0, 1])
+@pytest.mark.parametrize("objs,punch", [([1, 1], -np.inf), ([3, 2], -np.inf), ([8], -np.inf), ([11, 2], -np.inf), ([1] * 30, -np.inf),
+                                        ([1, 1], np.nan), ([1] * 30, np.nan)])
+def test_closed_pixels_of_any_logit_have_a_label(objs, punch, skew):
+    """Suppressed pixels (-inf, or NaN where one object is alone) that the closure
+    fills belong to the object, as every closed pixel that no other object takes
+    does."""
+    _check(objs, 64, 160, 4, 4, 700 + len(objs), skew=skew, punch=punch)
