@@ -41,7 +41,9 @@
 #include "rs3_internal.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <climits>
+#include <mutex>
 
 namespace {
 
@@ -49,6 +51,7 @@ constexpr int CA_WARPS = 16;
 constexpr int CA_THREADS = 32 * CA_WARPS;
 constexpr int CA_RMAX = 8;
 constexpr int CA_ROWS = 24;         // the most rows of a tile
+constexpr int CA_KCMAX = 8;         // CTAs of a cluster (the portable size)
 
 // word e of a strip shifted so that bit l holds column 4 (l + q) + e; pv and
 // nx are the same word of the strips to the left and right
@@ -513,24 +516,67 @@ struct CloseShape {
     int ns, rows, KC, tiles_x;
 };
 
+// Clusters of 1..8 CTAs of a kernel that are resident at once on the current
+// device (fit[KC]); asked from the runtime at the kernel's first call there, which
+// also raises its shared-memory limit.  A cluster lies within one GPC, so they are
+// fewer than the CTAs that fit divided by KC: 36 of 8 CTAs where 304 CTAs fit.
+template <int NS, int RC, bool VEC>
+static const int *close_fit()
+{
+    constexpr int smem = CloseSmem<NS, (RC > 0 ? RC : CA_RMAX)>::BYTES;
+    static std::mutex mu;
+    static std::atomic<bool> ready[64];
+    static int fit[64][CA_KCMAX + 1];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    if (ready[dev].load(std::memory_order_acquire)) return fit[dev];
+    std::lock_guard<std::mutex> lock(mu);
+    const auto kernel = k_close_argmax<NS, RC, VEC>;
+    if (rs3_kernel_smem((const void *)kernel, smem) != RS3_OK) return nullptr;
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, CA_THREADS, smem) != cudaSuccess || per_sm < 1)
+        return nullptr;
+    fit[dev][1] = per_sm * rs3_sm_count();
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = attr.val.clusterDim.y = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(CA_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    for (int KC = 2; KC <= CA_KCMAX; ++KC) {
+        attr.val.clusterDim.z = KC;
+        cfg.gridDim = dim3(1, 1, KC);
+        if (cudaOccupancyMaxActiveClusters(&fit[dev][KC], kernel, &cfg) != cudaSuccess) return nullptr;
+    }
+    ready[dev].store(true, std::memory_order_release);
+    return fit[dev];
+}
+
 // Rows per tile and CTAs per cluster: the least waves x objects per CTA x cost
 // of an object, where the cost counts the strip rows read (halo and all) and a
-// fixed part for the passes' latency, worth about 40 of them.  `per_sm` CTAs are
-// resident per SM; the rows tried are those that just fill one wave, 16 and 24.
-static CloseShape close_shape(int G, int objects, int h, int w, int R, int per_sm)
+// fixed part for the passes' latency, worth about 40 of them.  fit[KC] clusters
+// of KC CTAs are resident; the rows tried are those that just fill one wave (at
+// least 6: fewer are no faster), 16 and 24, and the KC those that leave a CTA
+// fewer objects.  8 objects of one stream at 256 x 256: 7.1 us in 8-row tiles of
+// 32 clusters, 10.1 in 37 clusters of 7-row tiles, one more than are resident; at
+// 1024 x 1024 28.8 and 42.1.
+static CloseShape close_shape(int G, int objects, int h, int w, int R, const int *fit)
 {
     CloseShape best = {};
     best.ns = std::min(4, (w + 127) / 128);
     best.tiles_x = (w + 128 * best.ns - 1) / (128 * best.ns);
-    const int slots = per_sm * rs3_sm_count();
+    const long long columns = (long long)best.tiles_x * G;              // tiles per row of tiles
     double least = 0.0;
     for (int KC = 1; KC <= objects; ++KC) {
-        const long long columns = (long long)best.tiles_x * G * KC;     // CTAs per row of tiles
-        const int tiles = (int)std::max(1ll, slots / columns);
-        const int fit = std::min(CA_ROWS, std::max(4, (h + tiles - 1) / tiles));
-        for (const int rows : {fit, 16, CA_ROWS}) {
-            const long long ctas = columns * ((h + rows - 1) / rows);
-            const double cost = (double)((ctas + slots - 1) / slots) * ((objects + KC - 1) / KC) *
+        const int per_cta = (objects + KC - 1) / KC;
+        if (fit[KC] < 1 || (KC > 1 && per_cta == (objects + KC - 2) / (KC - 1))) continue;
+        const int tiles = (int)std::max(1ll, fit[KC] / columns);
+        const int one_wave = std::min(CA_ROWS, std::max(6, (h + tiles - 1) / tiles));
+        for (const int rows : {one_wave, 16, CA_ROWS}) {
+            const long long n = columns * ((h + rows - 1) / rows);
+            const double cost = (double)((n + fit[KC] - 1) / fit[KC]) * per_cta *
                                     (40.0 + (double)(rows + 4 * R) * best.ns) + (KC > 1 ? 20.0 : 0.0);
             if (best.KC == 0 || cost < least) {
                 least = cost;
@@ -543,16 +589,17 @@ static CloseShape close_shape(int G, int objects, int h, int w, int R, int per_s
 }
 
 template <int NS, int RC, bool VEC>
-static cudaError_t launch_close(const CloseShape &c, int h, int G, cudaStream_t st, const float *logits,
-                                const int32_t *gstart, int U, int w, int R, int s, uint8_t *palette,
-                                uint8_t *closed, uint8_t *grid, int32_t *status)
+static cudaError_t launch_close(int G, int objects, int h, cudaStream_t st, const float *logits, const int32_t *gstart,
+                                int U, int w, int R, int s, uint8_t *palette, uint8_t *closed, uint8_t *grid,
+                                int32_t *status)
 {
-    constexpr int smem = CloseSmem<NS, (RC > 0 ? RC : CA_RMAX)>::BYTES;
-    if (rs3_kernel_smem((const void *)k_close_argmax<NS, RC, VEC>, smem) != RS3_OK) return cudaErrorInvalidValue;
+    const int *fit = close_fit<NS, RC, VEC>();
+    if (!fit) return cudaErrorInvalidValue;
+    const CloseShape c = close_shape(G, objects, h, w, R, fit);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(c.tiles_x, (h + c.rows - 1) / c.rows, G * c.KC);
     cfg.blockDim = dim3(CA_THREADS);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = CloseSmem<NS, (RC > 0 ? RC : CA_RMAX)>::BYTES;
+    cfg.gridDim = dim3(c.tiles_x, (h + c.rows - 1) / c.rows, G * c.KC);
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -568,13 +615,14 @@ static cudaError_t launch_close(const CloseShape &c, int h, int G, cudaStream_t 
 }
 
 template <int RC, bool VEC, typename... Args>
-static cudaError_t launch_close_strips(const CloseShape &c, Args... args)
+static cudaError_t launch_close_strips(int G, int objects, int h, cudaStream_t st, const float *logits,
+                                       const int32_t *gstart, int U, int w, Args... args)
 {
-    switch (c.ns) {
-    case 1: return launch_close<1, RC, VEC>(c, args...);
-    case 2: return launch_close<2, RC, VEC>(c, args...);
-    case 3: return launch_close<3, RC, VEC>(c, args...);
-    default: return launch_close<4, RC, VEC>(c, args...);
+    switch (std::min(4, (w + 127) / 128)) {
+    case 1: return launch_close<1, RC, VEC>(G, objects, h, st, logits, gstart, U, w, args...);
+    case 2: return launch_close<2, RC, VEC>(G, objects, h, st, logits, gstart, U, w, args...);
+    case 3: return launch_close<3, RC, VEC>(G, objects, h, st, logits, gstart, U, w, args...);
+    default: return launch_close<4, RC, VEC>(G, objects, h, st, logits, gstart, U, w, args...);
     }
 }
 
@@ -590,24 +638,18 @@ extern "C" rs3_status rs3_close_argmax(const float *logits, const int32_t *group
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     // objects of a stream on average, at most 8 (the portable cluster size);
     // ranks past a stream's object count idle
-    const int objects = std::min(8, std::max(1, (U + G - 1) / G));
+    const int objects = std::min(CA_KCMAX, std::max(1, (U + G - 1) / G));
     if ((long long)G * objects > 65535) return RS3_EUNSUPPORTED;
     // 16-byte loads and 4-byte stores where the arrays allow them
     const auto low = [](const void *p) { return reinterpret_cast<uintptr_t>(p); };
     const bool vec = rs3_aligned16(logits) && ((low(palette) | low(closed)) & 3u) == 0;
-    // the kernel of a radius at run time takes twice the registers: one CTA per SM
-    // (3 objects of 480 x 480, radius 2: 14.5 us, 19.5 in two waves of smaller tiles)
-    const CloseShape c = close_shape(G, objects, h, w, radius, vec && radius == 4 ? 2 : 1);
-    cudaError_t e;
-    if (!vec)
-        e = launch_close_strips<0, false>(c, h, G, st, logits, group_start, U, w, radius, s, palette,
-                                          closed, grid_masks, status);
-    else if (radius == 4)                    // the paper's 9 x 9 element
-        e = launch_close_strips<4, true>(c, h, G, st, logits, group_start, U, w, radius, s, palette,
-                                         closed, grid_masks, status);
-    else
-        e = launch_close_strips<0, true>(c, h, G, st, logits, group_start, U, w, radius, s, palette,
-                                         closed, grid_masks, status);
+    // the paper's 9 x 9 element has kernels of its own; those of a radius at run
+    // time take twice the registers, one CTA per SM
+    const auto launch = radius == 4 ? (vec ? launch_close_strips<4, true, int, int, uint8_t *, uint8_t *, uint8_t *, int32_t *>
+                                           : launch_close_strips<4, false, int, int, uint8_t *, uint8_t *, uint8_t *, int32_t *>)
+                                    : (vec ? launch_close_strips<0, true, int, int, uint8_t *, uint8_t *, uint8_t *, int32_t *>
+                                           : launch_close_strips<0, false, int, int, uint8_t *, uint8_t *, uint8_t *, int32_t *>);
+    const cudaError_t e = launch(G, objects, h, st, logits, group_start, U, w, radius, s, palette, closed, grid_masks, status);
     return e == cudaSuccess ? RS3_OK : RS3_ECUDA;
 }
 

@@ -71,3 +71,11 @@ def test_closed_pixels_of_any_logit_have_a_label(objs, punch, skew):
     fills belong to the object, as every closed pixel that no other object takes
     does."""
     _check(objs, 64, 160, 4, 4, 700 + len(objs), skew=skew, punch=punch)
+
+
+@pytest.mark.parametrize("objs,h,w,R,skew", [([8], 256, 256, 4, 0), ([8], 256, 256, 2, 0), ([8], 256, 256, 4, 1), ([5], 300, 640, 4, 0),
+                                             ([16], 130, 512, 7, 0), ([3], 40, 96, 4, 0)])
+def test_one_stream_of_several_objects(objs, h, w, R, skew):
+    """The sizes whose tiles are shared by clusters: as many as are resident at
+    once, with one, two or more objects for each of their CTAs."""
+    _check(objs, h, w, R, 4 if h % 4 == 0 else 2, 800 + h, skew=skew)
