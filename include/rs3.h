@@ -113,7 +113,8 @@ int rs3_version(void);
 /* ------------------------------------------------------------------------ */
 
 /* Bytes of device workspace rs3_select_queries is to be given (a group
- * "needed-cell" bitmap, per-unit priors and group energies). */
+ * "needed-cell" bitmap, per-unit priors and group energies).  Calls that take one
+ * launch leave it alone; the size does not depend on that. */
 size_t rs3_select_workspace_bytes(int G, int U, int m, int n);
 
 /*
@@ -162,7 +163,10 @@ rs3_status rs3_select_queries(const void *z, rs3_dtype dtype, int G, int m, int 
  *   - Sizes whose workspace (rs3_select_workspace_bytes(G, U, m, n)) exceeds
  *     8 MiB are rejected with RS3_ECAPACITY; nothing is launched.
  *   - The call allocates nothing (no cudaMalloc / cudaFree, no allocating
- *     library routine) and shares no memory between calls.
+ *     library routine) and shares no memory between calls.  It always takes
+ *     one launch, where rs3_select_queries takes three, several times faster, for
+ *     rows of thousands of channels, dozens of objects on one grid, and unions
+ *     of more than eight objects.
  */
 rs3_status rs3_select_queries_noalloc(const void *z, rs3_dtype dtype, int G, int m, int n, int C,
                                       const uint8_t *prev_masks, const int32_t *unit_group, int U,

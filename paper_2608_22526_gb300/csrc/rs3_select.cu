@@ -2,7 +2,9 @@
 // write keep-set K_w (Sec. 3.2: Eq. 8), integer-exact.
 //
 // k_select  the whole selection in one launch: a thread-block cluster of KC
-//           CTAs per unit (per group in union mode).
+//           CTAs per unit (per group in union mode).  Calls of wide rows, of many
+//           objects on one grid or of large unions take three launches through
+//           the workspace instead (below; three_launches() draws the line).
 //   1. Every CTA turns the unit's mask into bit words (a ballot per 32 cells of
 //      a row), updates the tracker (Eq. 4) and dilates: funnel-shifted words
 //      along the rows, ORs over rows.  The prior is a bit mask in shared memory.
@@ -18,7 +20,8 @@
 //      bins over the keys' range (energies share their leading bits, which puts
 //      a radix pass's keys into a few bins).  A bin of at most 32 keys is
 //      ranked by a warp, a fuller one is divided again.  Then it writes the
-//      kept cells in ascending order (block scan).
+//      kept cells in ascending order (block scan); in union mode every CTA of the
+//      cluster writes some of the group's units.
 // Bound by latency and, in one CTA per SM, by instruction issue: 512 threads
 // and no divisions in the loops, where 1024 threads took 30 000 cycles.
 // One object of 64 x 64 cells and 256 channels takes 7.6 us in a graph, eight
@@ -371,6 +374,196 @@ struct Energies {
     }
 };
 
+// The keys of list entries [lo, hi) by a CTA; before() runs ahead of the first
+// store.  lpr lanes share a row: 32, or fewer that hold one chunk each.
+template <typename T, typename F>
+__device__ __forceinline__ void energies(const T *zg, const uint16_t *list, uint32_t lo, uint32_t hi, int C, int lpr,
+                                         uint32_t *keys, uint32_t key0, bool remote, F before)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lpr == 32) {
+        constexpr int UN = sizeof(T) == 2 ? 8 : 4;
+        for (uint32_t j0 = lo; j0 < hi; j0 += UN * SEL_WARPS) {
+            Energies<T, UN> e;
+            e.load(zg, list, j0, hi, C);
+            before();
+            e.store(keys, key0, remote, j0, hi);
+        }
+        return;
+    }
+    const int nchunk = C >> 3, rpw = 32 / lpr, sub = lane / lpr, l = lane % lpr;
+    constexpr int UN = 4;
+    for (uint32_t j0 = lo; j0 < hi; j0 += UN * SEL_WARPS * rpw) {
+        Chunk8<T> x[UN];
+        float s[UN];
+#pragma unroll
+        for (int q = 0; q < UN; ++q) {
+            const uint32_t j = j0 + (q * SEL_WARPS + warp) * rpw + sub;
+            if (l < nchunk) x[q].load(zg + (size_t)list[min(j, hi - 1u)] * C + l * 8);
+        }
+#pragma unroll
+        for (int q = 0; q < UN; ++q) {
+            s[q] = l < nchunk ? x[q].add(0.f) : 0.f;
+            for (int w = lpr >> 1; w >= 1; w >>= 1) s[q] = s[q] + __shfl_xor_sync(0xffffffffu, s[q], w);
+        }
+        before();
+#pragma unroll
+        for (int q = 0; q < UN; ++q) {
+            const uint32_t j = j0 + (q * SEL_WARPS + warp) * rpw + sub;
+            if (j < hi && l == 0) {
+                if (remote) dsmem_st(key0 + 4 * j, __float_as_uint(s[q]));
+                else keys[j] = __float_as_uint(s[q]);
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// ranking (by a whole CTA)
+// ---------------------------------------------------------------------------
+// Which keys are kept: those >= from, and the first `want` of those == equal.
+// `all`: every one (no key was needed).
+struct Kept {
+    uint32_t from = 0u, equal = 0xffffffffu, want = 0u;
+    bool all = true;
+};
+
+// The k largest of nP keys (0 < k < nP), `hist` SEL_BINS words of scratch.
+__device__ __forceinline__ Kept top_keys(const uint32_t *keys, uint32_t nP, uint32_t k, uint32_t *hist)
+{
+    __shared__ uint32_t s_bin, s_rem, s_cnt, s_ncand, s_cand[32], s_mm[2][SEL_WARPS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    Kept r;
+    r.all = false;
+    if (threadIdx.x == 0) s_ncand = 0u;
+    for (int b = threadIdx.x; b < SEL_BINS; b += SEL_THREADS) hist[b] = 0;
+    __syncthreads();                                     // (and the keys)
+    // the range of the keys
+    uint32_t mi = 0xffffffffu, ma = 0u;
+    for (uint32_t j = threadIdx.x; j < nP; j += SEL_THREADS) {
+        mi = min(mi, keys[j]);
+        ma = max(ma, keys[j]);
+    }
+    mi = __reduce_min_sync(0xffffffffu, mi);
+    ma = __reduce_max_sync(0xffffffffu, ma);
+    if (lane == 0) { s_mm[0][warp] = mi; s_mm[1][warp] = ma; }
+    __syncthreads();
+    mi = __reduce_min_sync(0xffffffffu, s_mm[0][lane % SEL_WARPS]);
+    ma = __reduce_max_sync(0xffffffffu, s_mm[1][lane % SEL_WARPS]);
+    // keys of bin b of a pass lie in [base + (b << shift), base + ((b + 1) <<
+    // shift)); want: how many of the range's largest keys are kept
+    uint32_t base = mi, span = ma - mi;
+    r.want = k;
+    int shift = max(0, 32 - __clz(span | 1u) - 11);
+    for (;;) {
+        for (uint32_t j = threadIdx.x; j < nP; j += SEL_THREADS) {
+            const uint32_t d = keys[j] - base;           // wraps past every span for keys below base
+            if (d <= span) atomicAdd(&hist[d >> shift], 1u);
+        }
+        __syncthreads();
+        // thread t takes four bins, from the top
+        const uint4 h = reinterpret_cast<const uint4 *>(hist)[SEL_BINS / 4 - 1 - threadIdx.x];
+        uint32_t tot, above = block_excl_scan((h.x + h.y) + (h.z + h.w), tot);
+        if (above < r.want && r.want <= above + (h.x + h.y) + (h.z + h.w)) {
+            const uint32_t x[4] = {h.w, h.z, h.y, h.x};
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                if (above < r.want && r.want <= above + x[b]) {
+                    s_bin = SEL_BINS - 1 - 4 * threadIdx.x - b;
+                    s_rem = r.want - above;
+                    s_cnt = x[b];
+                }
+                above += x[b];
+            }
+        }
+        __syncthreads();
+        base += s_bin << shift;
+        r.want = s_rem;
+        span = (1u << shift) - 1u;
+        if (s_cnt == r.want) {                           // the whole bin is kept
+            r.from = base;
+            r.want = 0u;
+            return r;
+        }
+        if (shift == 0) {                                // a bin of equal keys
+            r.from = base + 1u;
+            r.equal = base;
+            return r;
+        }
+        if (s_cnt <= 32u) {                              // a warp ranks them (each for itself)
+            for (uint32_t j = threadIdx.x; j < nP; j += SEL_THREADS)
+                if (keys[j] - base <= span) s_cand[atomicAdd(&s_ncand, 1u)] = keys[j];
+            __syncthreads();
+            const int nc = (int)s_cnt;
+            const uint32_t x = s_cand[lane < nc ? lane : 0];
+            uint32_t gt = 0, ge = 0;
+            for (int i = 0; i < nc; ++i) {
+                const uint32_t y = __shfl_sync(0xffffffffu, x, i);
+                gt += y > x ? 1u : 0u;
+                ge += y >= x ? 1u : 0u;
+            }
+            const int at = __ffs(__ballot_sync(0xffffffffu, lane < nc && gt < r.want && r.want <= ge)) - 1;
+            r.equal = __shfl_sync(0xffffffffu, x, at);
+            r.from = r.equal + 1u;
+            r.want -= __shfl_sync(0xffffffffu, gt, at);
+            return r;
+        }
+        shift = max(0, shift - 11);
+        for (int b = threadIdx.x; b < SEL_BINS; b += SEL_THREADS) hist[b] = 0;
+        __syncthreads();
+    }
+}
+
+// Where the kept cells go.  Each thread a run of the list; a kept cell's place is
+// the number of kept larger keys before it and of equal ones, of which the first
+// `want` are kept.
+struct Place {
+    uint32_t j0, j1, off;
+    __device__ __forceinline__ Place(const uint32_t *keys, uint32_t nP, const Kept &r)
+    {
+        const uint32_t per = (nP + SEL_THREADS - 1) / SEL_THREADS;
+        j0 = threadIdx.x * per;
+        j1 = min(j0 + per, nP);
+        off = 0u;
+        if (r.all) return;
+        uint32_t mine = 0, tot;
+        for (uint32_t j = j0; j < j1; ++j) mine += (keys[j] >= r.from ? 0x10000u : 0u) + (keys[j] == r.equal ? 1u : 0u);
+        off = block_excl_scan(mine, tot);
+    }
+    // the kept cells of the list in order, into `out`, which may lie over the keys
+    __device__ __forceinline__ void compact(const uint32_t *keys, const uint16_t *list, const Kept &r, uint16_t *out) const
+    {
+        uint32_t at = (off >> 16) + min(off & 0xffffu, r.want), eq = off & 0xffffu, flags = 0u;
+        for (uint32_t j = j0; j < j1; ++j) {             // at most 32: a run of 16384 / SEL_THREADS cells
+            const uint32_t key = keys[j];
+            const bool is_eq = key == r.equal;
+            if (key >= r.from || (is_eq && eq < r.want)) flags |= 1u << (j - j0);
+            eq += is_eq ? 1u : 0u;
+        }
+        __syncthreads();
+        for (; flags; flags &= flags - 1) out[at++] = list[j0 + __ffs(flags) - 1];
+        __syncthreads();
+    }
+    // one unit's row of the output and its count
+    __device__ __forceinline__ void emit(const uint32_t *keys, const uint16_t *list, const Kept &r, uint32_t n_kept, int32_t *out,
+                         int32_t *count) const
+    {
+        if (r.all) {
+            for (uint32_t j = threadIdx.x; j < n_kept; j += SEL_THREADS) out[j] = list[j];
+        } else {
+            uint32_t gt = off >> 16, eq = off & 0xffffu;
+            for (uint32_t j = j0; j < j1; ++j) {
+                const uint32_t key = keys[j];
+                const bool is_eq = key == r.equal;
+                if (key >= r.from || (is_eq && eq < r.want)) out[gt + min(eq, r.want)] = list[j];
+                gt += key >= r.from ? 1u : 0u;
+                eq += is_eq ? 1u : 0u;
+            }
+        }
+        if (threadIdx.x == 0) *count = (int32_t)n_kept;
+    }
+};
+
 template <typename T>
 __global__ void __launch_bounds__(SEL_THREADS)
 k_select(const T *__restrict__ z, const uint8_t *__restrict__ masks, int m, int n, int C, int lpr,
@@ -380,16 +573,33 @@ k_select(const T *__restrict__ z, const uint8_t *__restrict__ masks, int m, int 
 {
     pdl_wait();
     extern __shared__ __align__(16) uint8_t sel_raw[];
-    __shared__ uint32_t s_bin, s_rem, s_cnt, s_ncand, s_cand[32], s_mm[2][SEL_WARPS];
     const SelSmem S = sel_smem(m, n);
     uint32_t *P = reinterpret_cast<uint32_t *>(sel_raw + S.prior), *hist = P;
     uint32_t *A = reinterpret_cast<uint32_t *>(sel_raw + S.a), *keys = A;
     uint32_t *B = reinterpret_cast<uint32_t *>(sel_raw + S.b), *pref = B;
     uint16_t *list = reinterpret_cast<uint16_t *>(sel_raw + S.list);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int u = blockIdx.x / KC;
+    int u = blockIdx.x / KC;
     const uint32_t rank = KC > 1 ? cluster_rank() : 0u;
     const int mn = m * n, WW = (n + 31) >> 5, words = m * WW;
+    if (union_mode) {
+        // a cluster per group: its first unit, if it has one
+        __shared__ int s_first;
+        const int group = u;
+        if (threadIdx.x == 0) s_first = U;
+        __syncthreads();
+        for (int v = threadIdx.x; v < U; v += SEL_THREADS) {
+            const int gv = unit_group[v];
+            if (gv == group) atomicMin(&s_first, v);
+            if ((gv < 0 || gv >= G) && group == 0 && rank == 0) {
+                latch_status(status, RS3_EINVAL);
+                count[v] = 0;
+            }
+        }
+        __syncthreads();
+        u = s_first;
+        if (u >= U) return;                              // uniform over the cluster
+    }
     const int g = unit_group[u];
     if (g < 0 || g >= G) {                               // uniform over the cluster
         if (rank == 0 && threadIdx.x == 0) {
@@ -398,14 +608,8 @@ k_select(const T *__restrict__ z, const uint8_t *__restrict__ masks, int m, int 
         }
         return;
     }
-    if (union_mode) {                                    // the group's first unit works for all of them
-        bool other = false;
-        for (int v = threadIdx.x; v < u; v += SEL_THREADS) other |= unit_group[v] == g;
-        if (__syncthreads_or(other)) return;             // uniform over the cluster
-    }
     const WordWalk walk(WW);
     for (int w = threadIdx.x; w < words; w += SEL_THREADS) P[w] = 0u;
-    if (threadIdx.x == 0) s_ncand = 0u;
     rs3_track tr = {};
     if (!union_mode) {
         // (P is read again only after this call's first barrier)
@@ -467,47 +671,10 @@ k_select(const T *__restrict__ z, const uint8_t *__restrict__ masks, int m, int 
         const uint32_t key0 = KC > 1 ? dsmem_addr(keys, 0u) : 0u;
         const T *zg = z + (size_t)g * mn * C;
         bool waited = KC == 1;
-        if (lpr == 32) {
-            constexpr int UN = sizeof(T) == 2 ? 8 : 4;
-            for (uint32_t j0 = lo; j0 < hi; j0 += UN * SEL_WARPS) {
-                Energies<T, UN> e;
-                e.load(zg, list, j0, hi, C);
-                if (!waited) {
-                    cluster_wait();
-                    waited = true;
-                }
-                e.store(keys, key0, KC > 1, j0, hi);
-            }
-        } else {
-            const int nchunk = C >> 3, rpw = 32 / lpr, sub = lane / lpr, l = lane % lpr;
-            constexpr int UN = 4;
-            for (uint32_t j0 = lo; j0 < hi; j0 += UN * SEL_WARPS * rpw) {
-                Chunk8<T> x[UN];
-                float s[UN];
-#pragma unroll
-                for (int q = 0; q < UN; ++q) {
-                    const uint32_t j = j0 + (q * SEL_WARPS + warp) * rpw + sub;
-                    if (l < nchunk) x[q].load(zg + (size_t)list[min(j, hi - 1u)] * C + l * 8);
-                }
-#pragma unroll
-                for (int q = 0; q < UN; ++q) {
-                    s[q] = l < nchunk ? x[q].add(0.f) : 0.f;
-                    for (int w = lpr >> 1; w >= 1; w >>= 1) s[q] = s[q] + __shfl_xor_sync(0xffffffffu, s[q], w);
-                }
-                if (!waited) {
-                    cluster_wait();
-                    waited = true;
-                }
-#pragma unroll
-                for (int q = 0; q < UN; ++q) {
-                    const uint32_t j = j0 + (q * SEL_WARPS + warp) * rpw + sub;
-                    if (j < hi && l == 0) {
-                        if (KC > 1) dsmem_st(key0 + 4 * j, __float_as_uint(s[q]));
-                        else keys[j] = __float_as_uint(s[q]);
-                    }
-                }
-            }
-        }
+        energies<T>(zg, list, lo, hi, C, lpr, keys, key0, KC > 1, [&]() {
+            if (!waited) cluster_wait();
+            waited = true;
+        });
         if (!waited) cluster_wait();
         if (KC > 1) {
             cluster_arrive();
@@ -516,123 +683,161 @@ k_select(const T *__restrict__ z, const uint8_t *__restrict__ masks, int m, int 
     } else if (KC > 1) {
         cluster_wait();
     }
-    if (rank != 0) return;
-    if (!union_mode && threadIdx.x == 0) track[u] = tr;
-
-    // keep key >= from, and the first `want` of key == equal
-    uint32_t from = 0u, equal = 0xffffffffu, want = 0u;
-    if (!keep_all && k > 0) {
-        for (int b = threadIdx.x; b < SEL_BINS; b += SEL_THREADS) hist[b] = 0;
-        __syncthreads();                                 // (KC = 1: the keys too)
-        // the range of the keys
-        uint32_t mi = 0xffffffffu, ma = 0u;
-        for (uint32_t j = threadIdx.x; j < nP; j += SEL_THREADS) {
-            mi = min(mi, keys[j]);
-            ma = max(ma, keys[j]);
-        }
-        mi = __reduce_min_sync(0xffffffffu, mi);
-        ma = __reduce_max_sync(0xffffffffu, ma);
-        if (lane == 0) { s_mm[0][warp] = mi; s_mm[1][warp] = ma; }
-        __syncthreads();
-        mi = __reduce_min_sync(0xffffffffu, s_mm[0][lane % SEL_WARPS]);
-        ma = __reduce_max_sync(0xffffffffu, s_mm[1][lane % SEL_WARPS]);
-        // keys of bin b of a pass lie in [base + (b << shift), base + ((b + 1) <<
-        // shift)); want: how many of the range's largest keys are kept
-        uint32_t base = mi, span = ma - mi;
-        want = (uint32_t)k;
-        int shift = max(0, 32 - __clz(span | 1u) - 11);
-        for (;;) {
-            for (uint32_t j = threadIdx.x; j < nP; j += SEL_THREADS) {
-                const uint32_t d = keys[j] - base;       // wraps past every span for keys below base
-                if (d <= span) atomicAdd(&hist[d >> shift], 1u);
-            }
-            __syncthreads();
-            // thread t takes four bins, from the top
-            const uint4 h = reinterpret_cast<const uint4 *>(hist)[SEL_BINS / 4 - 1 - threadIdx.x];
-            uint32_t tot, above = block_excl_scan((h.x + h.y) + (h.z + h.w), tot);
-            if (above < want && want <= above + (h.x + h.y) + (h.z + h.w)) {
-                const uint32_t x[4] = {h.w, h.z, h.y, h.x};
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    if (above < want && want <= above + x[b]) {
-                        s_bin = SEL_BINS - 1 - 4 * threadIdx.x - b;
-                        s_rem = want - above;
-                        s_cnt = x[b];
-                    }
-                    above += x[b];
-                }
-            }
-            __syncthreads();
-            base += s_bin << shift;
-            want = s_rem;
-            span = (1u << shift) - 1u;
-            if (s_cnt == want) {                         // the whole bin is kept
-                from = base;
-                want = 0u;
-                break;
-            }
-            if (shift == 0) {                            // a bin of equal keys
-                from = base + 1u;
-                equal = base;
-                break;
-            }
-            if (s_cnt <= 32u) {                          // a warp ranks them (each for itself)
-                for (uint32_t j = threadIdx.x; j < nP; j += SEL_THREADS)
-                    if (keys[j] - base <= span) s_cand[atomicAdd(&s_ncand, 1u)] = keys[j];
-                __syncthreads();
-                const int nc = (int)s_cnt;
-                const uint32_t x = s_cand[lane < nc ? lane : 0];
-                uint32_t gt = 0, ge = 0;
-                for (int i = 0; i < nc; ++i) {
-                    const uint32_t y = __shfl_sync(0xffffffffu, x, i);
-                    gt += y > x ? 1u : 0u;
-                    ge += y >= x ? 1u : 0u;
-                }
-                const int at = __ffs(__ballot_sync(0xffffffffu, lane < nc && gt < want && want <= ge)) - 1;
-                equal = __shfl_sync(0xffffffffu, x, at);
-                from = equal + 1u;
-                want -= __shfl_sync(0xffffffffu, gt, at);
-                break;
-            }
-            shift = max(0, shift - 11);
-            for (int b = threadIdx.x; b < SEL_BINS; b += SEL_THREADS) hist[b] = 0;
-            __syncthreads();
-        }
-    }
-    // each thread a run of the list; a kept cell's place is the number of kept
-    // larger keys before it and of equal ones, of which the first `want` are kept
-    const uint32_t per = (nP + SEL_THREADS - 1) / SEL_THREADS, j0 = threadIdx.x * per, j1 = min(j0 + per, nP);
     const bool ranked = !keep_all && k > 0;
-    uint32_t off = j0;
-    if (ranked) {
-        uint32_t mine = 0, tot;
-        for (uint32_t j = j0; j < j1; ++j) mine += (keys[j] >= from ? 0x10000u : 0u) + (keys[j] == equal ? 1u : 0u);
-        off = block_excl_scan(mine, tot);
+    if (!union_mode) {
+        if (rank != 0) return;
+        if (threadIdx.x == 0) track[u] = tr;
+        const Kept kept = ranked ? top_keys(keys, nP, (uint32_t)k, hist) : Kept{};
+        const Place place(keys, nP, kept);
+        place.emit(keys, list, kept, n_kept, idx + (size_t)u * k, count + u);
+        return;
     }
-    const auto emit = [&](int v) {
-        int32_t *out = idx + (size_t)v * k;
-        if (!ranked) {
-            for (uint32_t j = threadIdx.x; j < n_kept; j += SEL_THREADS) out[j] = list[j];
-        } else {
-            uint32_t gt = off >> 16, eq = off & 0xffffu;
-            for (uint32_t j = j0; j < j1; ++j) {
-                const uint32_t key = keys[j];
-                const bool is_eq = key == equal;
-                if (key >= from || (is_eq && eq < want)) out[gt + min(eq, want)] = list[j];
-                gt += key >= from ? 1u : 0u;
-                eq += is_eq ? 1u : 0u;
+    // union mode: the first CTA ranks, every CTA writes the group's units in turn
+    const uint16_t *kept_list = list;
+    if (ranked) {
+        if (rank == 0) {
+            const Kept kept = top_keys(keys, nP, (uint32_t)k, hist);
+            const Place place(keys, nP, kept);
+            place.compact(keys, list, kept, reinterpret_cast<uint16_t *>(keys));
+        }
+        if (KC > 1) {
+            cluster_arrive();
+            cluster_wait();
+            if (rank != 0)
+                for (uint32_t i = threadIdx.x; i < (n_kept + 1) / 2; i += SEL_THREADS)
+                    keys[i] = dsmem_ld(dsmem_addr(keys + i, 0u));
+            cluster_arrive();
+        }
+        __syncthreads();
+        kept_list = reinterpret_cast<const uint16_t *>(keys);
+    }
+    uint32_t seen = 0;
+    for (int v0 = u; v0 < U; v0 += 32) {
+        uint32_t in = __ballot_sync(0xffffffffu, v0 + lane < U && unit_group[min(v0 + lane, U - 1)] == g);
+        for (; in; in &= in - 1, ++seen) {
+            if (seen % (uint32_t)KC != rank) continue;
+            const int v = v0 + __ffs(in) - 1;
+            int32_t *out = idx + (size_t)v * k;
+            for (uint32_t j = threadIdx.x; j < n_kept; j += SEL_THREADS) out[j] = kept_list[j];
+            if (threadIdx.x == 0) count[v] = (int32_t)n_kept;
+        }
+    }
+    if (ranked && KC > 1) cluster_wait();                // every CTA has read the first one's list
+}
+
+// ---------------------------------------------------------------------------
+// The selection in three launches, through the workspace, for calls whose rows are
+// too much for the few SMs that a unit's cluster has, or whose objects share them:
+//   k_prior   a CTA per unit: tracker and prior; bit i of a unit's (or, in union
+//             mode, the group's) cells, and the cells that the group needs
+//   k_energy  the energies of the needed cells, over all SMs
+//   k_rank    a CTA per unit: lists, ranks and writes
+// ---------------------------------------------------------------------------
+struct SelWs {           // in the workspace; nf = ceil(mn / 32) words hold a bit per cell
+    uint32_t *need;      // [G][nf]
+    uint32_t *prior;     // [U][nf]
+    uint32_t *energy;    // [G][mn] bits of the fp32 energies
+};
+
+__global__ void __launch_bounds__(SEL_THREADS)
+k_prior(const uint8_t *__restrict__ masks, int m, int n, const int32_t *__restrict__ unit_group, int G,
+        rs3_track *__restrict__ track, int r_s, int c, int bbox_mode, int union_mode, SelWs ws, int32_t *status)
+{
+    pdl_wait();
+    extern __shared__ __align__(16) uint8_t sel_raw[];
+    const int mn = m * n, WW = (n + 31) >> 5, words = m * WW, nf = (mn + 31) >> 5, u = blockIdx.x, g = unit_group[u];
+    if (g < 0 || g >= G) {                               // k_rank writes its count
+        if (threadIdx.x == 0) latch_status(status, RS3_EINVAL);
+        return;
+    }
+    uint32_t *P = reinterpret_cast<uint32_t *>(sel_raw), *A = P + words, *B = A + words, *F = B + words;
+    for (int w = threadIdx.x; w < words; w += SEL_THREADS) P[w] = 0u;
+    for (int w = threadIdx.x; w < nf; w += SEL_THREADS) F[w] = 0u;
+    const WordWalk walk(WW);
+    rs3_track tr = {};
+    unit_prior(masks + (size_t)u * mn, m, n, walk, track + u, r_s, c, bbox_mode, P, A, B, tr);
+    if (threadIdx.x == 0) track[u] = tr;
+    // words of a row -> bits of consecutive cells
+    walk.each(words, [&](int w, int y, int k) {
+        const uint32_t x = P[w];
+        const int i = y * n + 32 * k, sh = i & 31;
+        if (x == 0u) return;
+        atomicOr(&F[i >> 5], x << sh);
+        if (sh && x >> (32 - sh)) atomicOr(&F[(i >> 5) + 1], x >> (32 - sh));
+    });
+    __syncthreads();
+    for (int w = threadIdx.x; w < nf; w += SEL_THREADS) {
+        if (!union_mode) ws.prior[(size_t)u * nf + w] = F[w];
+        if (F[w]) atomicOr(&ws.need[(size_t)g * nf + w], F[w]);
+    }
+}
+
+// The set cells of words [w0, w0 + nw) in ascending order; every thread of the
+// CTA calls it.  Returns their number.
+__device__ __forceinline__ uint32_t list_bits(const uint32_t *F, int w0, int nw, uint16_t *list)
+{
+    const int per = (nw + SEL_THREADS - 1) / SEL_THREADS, a = threadIdx.x * per, b = min(a + per, nw);
+    uint32_t own = 0, total;
+    for (int w = a; w < b; ++w) own += __popc(F[w0 + w]);
+    uint32_t off = block_excl_scan(own, total);
+    for (int w = a; w < b; ++w)
+        for (uint32_t x = F[w0 + w]; x; x &= x - 1) list[off++] = (uint16_t)(32 * (w0 + w) + __ffs(x) - 1);
+    __syncthreads();
+    return total;
+}
+
+// A warp per row (per 32 / lpr rows of few channels), over all of the groups' rows.
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_energy(const T *__restrict__ z, int G, int mn, int C, int lpr, SelWs ws)
+{
+    pdl_wait();
+    const int nchunk = C >> 3, rpw = 32 / lpr, lane = threadIdx.x & 31, sub = lane / lpr, l = lane % lpr;
+    const int nf = (mn + 31) >> 5;
+    const long total = (long)G * mn;
+    const long wid = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = ((long)gridDim.x * blockDim.x) >> 5;
+    for (long base = wid * rpw; base < total; base += nwarps * rpw) {
+        const long row = base + sub;
+        bool needed = false;
+        if (row < total) {
+            const int g = (int)(row / mn), i = (int)(row - (long)g * mn);
+            needed = (ws.need[(size_t)g * nf + (i >> 5)] >> (i & 31)) & 1u;
+        }
+        float s = 0.0f;
+        if (needed) {
+            const T *zr = z + row * (long)C;
+            for (int ch = l; ch < nchunk; ch += 32) {
+                Chunk8<T> x;
+                x.load(zr + ch * 8);
+                s = x.add(s);
             }
         }
-        if (threadIdx.x == 0) count[v] = (int32_t)n_kept;
-    };
-    if (!union_mode) {
-        emit(u);
-    } else {
-        for (int v0 = u; v0 < U; v0 += 32) {
-            uint32_t in = __ballot_sync(0xffffffffu, v0 + lane < U && unit_group[min(v0 + lane, U - 1)] == g);
-            for (; in; in &= in - 1) emit(v0 + __ffs(in) - 1);
-        }
+        for (int w = lpr >> 1; w >= 1; w >>= 1) s = s + __shfl_xor_sync(0xffffffffu, s, w);
+        if (needed && l == 0) ws.energy[row] = __float_as_uint(s);
     }
+}
+
+// Shared memory: histogram, keys, list.
+__global__ void __launch_bounds__(SEL_THREADS)
+k_rank(int mn, const int32_t *__restrict__ unit_group, int G, int union_mode, int k, SelWs ws, int32_t *__restrict__ idx,
+       int32_t *__restrict__ count)
+{
+    pdl_wait();
+    extern __shared__ __align__(16) uint8_t sel_raw[];
+    uint32_t *hist = reinterpret_cast<uint32_t *>(sel_raw), *keys = hist + SEL_BINS;
+    uint16_t *list = reinterpret_cast<uint16_t *>(keys + mn);
+    const int nf = (mn + 31) >> 5, u = blockIdx.x, g = unit_group[u];
+    if (g < 0 || g >= G) {
+        if (threadIdx.x == 0) count[u] = 0;
+        return;
+    }
+    const uint32_t nP = list_bits(union_mode ? ws.need + (size_t)g * nf : ws.prior + (size_t)u * nf, 0, nf, list);
+    const bool keep_all = nP <= (uint32_t)k;
+    if (!keep_all)
+        for (uint32_t j = threadIdx.x; j < nP; j += SEL_THREADS) keys[j] = ws.energy[(size_t)g * mn + list[j]];
+    const Kept kept = keep_all || k == 0 ? Kept{} : top_keys(keys, nP, (uint32_t)k, hist);
+    const Place place(keys, nP, kept);
+    place.emit(keys, list, kept, keep_all ? nP : (uint32_t)k, idx + (size_t)u * k, count + u);
 }
 
 // ---------------------------------------------------------------------------
@@ -698,16 +903,30 @@ inline int next_pow2(int x)
 // ---------------------------------------------------------------------------
 // host entry points
 // ---------------------------------------------------------------------------
-// The selection keeps everything in shared memory; the size is that of a group
-// bitmap, the priors and the energies in global memory, which callers allocate
-// and rs3_select_queries_noalloc's limit counts.
+namespace {
+
+// Byte offsets in the workspace of the three-launch selection.  The size is part
+// of the ABI; the prior's region holds a byte per cell, of which bits are used.
+struct SelectWs {
+    size_t prior, energy, total;
+};
+
+SelectWs select_ws(int G, int U, int m, int n)
+{
+    const size_t mn = (size_t)m * n;
+    SelectWs w;
+    w.prior = align_up((size_t)G * ((mn + 31) / 32) * 4, 256);
+    w.energy = align_up(w.prior + (size_t)U * mn, 256);
+    w.total = align_up(w.energy + (size_t)G * mn * 4, 256);
+    return w;
+}
+
+}  // namespace
+
 extern "C" size_t rs3_select_workspace_bytes(int G, int U, int m, int n)
 {
     if (G < 1 || U < 1 || m < 1 || n < 1) return 0;
-    const size_t mn = (size_t)m * n;
-    size_t off = align_up((size_t)G * ((mn + 31) / 32) * 4, 256);
-    off = align_up(off + (size_t)U * mn, 256);
-    return align_up(off + (size_t)G * mn * 4, 256);
+    return select_ws(G, U, m, n).total;
 }
 
 namespace {
@@ -725,26 +944,77 @@ rs3_status select_check(const void *z, rs3_dtype dtype, int G, int m, int n, int
     return RS3_OK;
 }
 
+// Whether three launches are the faster, by what both take when most of the grid
+// is in the priors (us on 152 SMs).  One launch: the share of a unit's channels that
+// each CTA of its cluster reads, at two CTAs per SM half as fast.  Three: their fixed
+// cost, the rows that all SMs walk and the bytes they read.  One object on 64 x 64
+// cells: 256 bf16 channels 11.6 us in one launch, 18.4 in three; 2048 channels 42 and
+// 20; 16 x 3 objects on 96 x 96, 256 channels 45 and 52; 255 objects of one grid 33
+// and 19.  (The memset, prior, energy and select kernels before took 22, 26, 66 and
+// 31.)  Where nothing has to be ranked one launch reads no rows, and three cost 12 us
+// instead of 5, still less than before.  Union mode: units past a CTA each are
+// worked off in turn by a cluster, but side by side in three launches.
+bool three_launches(int G, int U, int mn, int C, size_t esz, int union_mode, long clusters, int KC, int n_sm)
+{
+    if (union_mode && U > (long)G * KC) return true;
+    const double share = (double)mn * C / KC, rows = (double)G * mn;
+    const double one = 6.0 + 36e-6 * share * std::max(1.0, (double)clusters * KC / n_sm);
+    const double three = 16.0 + 0.12e-3 * rows + 0.05e-6 * rows * C * (double)esz;
+    return one > three;
+}
+
+// The selection: one launch, or three through the workspace (null: one).
 rs3_status select_launch(const void *z, rs3_dtype dtype, int G, int m, int n, int C, const uint8_t *prev_masks,
                          const int32_t *unit_group, int U, rs3_track *track, const rs3_params *p, int32_t *idx,
-                         int32_t *count, int32_t *status, rs3_stream_t stream)
+                         int32_t *count, void *workspace, int32_t *status, rs3_stream_t stream)
 {
-    const int64_t k = rs3_kmax(p->rho, (int64_t)m * n);
+    const int mn = m * n;
+    const int64_t k = rs3_kmax(p->rho, (int64_t)mn);
     if (k < 0) return RS3_EINVAL;
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     // CTAs per cluster: as many as are resident at once (two per SM), up to the
     // portable 8; 48 units of 96 x 96 cells: 20.9 us with 6 each, 22.6 with 4
     const long clusters = p->union_mode ? (G < U ? G : U) : U;
-    const int KC = (int)std::min(8l, std::max(1l, 2l * rs3_sm_count() / clusters));
+    const int n_sm = rs3_sm_count();
+    const int KC = (int)std::min(8l, std::max(1l, 2l * n_sm / clusters));
     const int nchunk = C / 8;
     const int lpr = nchunk >= 32 ? 32 : next_pow2(nchunk);
+    cudaError_t e;
+    if (workspace && mn >= 4 &&             // (a unit's bits fit its bytes of the workspace)
+        three_launches(G, U, mn, C, dtype == RS3_BF16 ? 2 : 4, p->union_mode, clusters, KC, n_sm)) {
+        const int nf = (mn + 31) / 32;
+        const SelectWs l = select_ws(G, U, m, n);
+        uint8_t *b = static_cast<uint8_t *>(workspace);
+        const SelWs ws = {reinterpret_cast<uint32_t *>(b), reinterpret_cast<uint32_t *>(b + l.prior),
+                          reinterpret_cast<uint32_t *>(b + l.energy)};
+        const size_t prior_smem = 4 * (3 * (size_t)m * ((n + 31) / 32) + nf);
+        const size_t rank_smem = 4 * SEL_BINS + 6 * (size_t)mn;
+        if (rs3_kernel_smem((const void *)k_prior, prior_smem + 1024) != RS3_OK ||      // + its static arrays
+            rs3_kernel_smem((const void *)k_rank, rank_smem + 1024) != RS3_OK)
+            return RS3_ECUDA;
+        if (cudaMemsetAsync(ws.need, 0, (size_t)G * nf * 4, st) != cudaSuccess) return RS3_ECUDA;
+        e = launch_pdl(k_prior, dim3(U), dim3(SEL_THREADS), prior_smem, st, prev_masks, m, n, unit_group, G, track, p->r_s,
+                       p->c, p->bbox_mode, p->union_mode, ws, status);
+        const long warps = ((long)G * mn + 32 / lpr - 1) / (32 / lpr);
+        const dim3 grid((unsigned)std::min((warps + 7) / 8, 8l * n_sm));
+        if (e == cudaSuccess)
+            e = dtype == RS3_BF16 ? launch_pdl(k_energy<uint16_t>, grid, dim3(256), 0, st, static_cast<const uint16_t *>(z),
+                                               G, mn, C, lpr, ws)
+                                  : launch_pdl(k_energy<float>, grid, dim3(256), 0, st, static_cast<const float *>(z), G, mn,
+                                               C, lpr, ws);
+        if (e == cudaSuccess)
+            e = launch_pdl(k_rank, dim3(U), dim3(SEL_THREADS), rank_smem, st, mn, unit_group, G, p->union_mode, (int)k, ws,
+                           idx, count);
+        return e == cudaSuccess ? RS3_OK : RS3_ECUDA;
+    }
     const size_t smem = sel_smem(m, n).total;
     const void *fn = dtype == RS3_BF16 ? (const void *)k_select<uint16_t> : (const void *)k_select<float>;
     if (rs3_kernel_smem(fn, smem + 1024) != RS3_OK) return RS3_ECUDA;       // + the kernel's static arrays
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(U * KC));
+    cfg.gridDim = dim3((unsigned)((p->union_mode ? G : U) * KC));    // a cluster per group in union mode
     cfg.blockDim = dim3(SEL_THREADS);
     cfg.dynamicSmemBytes = smem;
-    cfg.stream = reinterpret_cast<cudaStream_t>(stream);
+    cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -754,7 +1024,6 @@ rs3_status select_launch(const void *z, rs3_dtype dtype, int G, int m, int n, in
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e;
     if (dtype == RS3_BF16)
         e = cudaLaunchKernelEx(&cfg, k_select<uint16_t>, static_cast<const uint16_t *>(z), prev_masks, m, n, C, lpr,
                                unit_group, G, U, track, p->r_s, p->c, p->bbox_mode, p->union_mode, (int)k, KC, idx,
@@ -780,7 +1049,8 @@ extern "C" rs3_status rs3_select_queries(const void *z, rs3_dtype dtype, int G, 
     if (s != RS3_OK) return s;
     if (!rs3_aligned16(workspace)) return RS3_EINVAL;
     if (workspace_bytes < rs3_select_workspace_bytes(G, U, m, n)) return RS3_ECAPACITY;
-    return select_launch(z, dtype, G, m, n, C, prev_masks, unit_group, U, track, p, idx, count, status, stream);
+    return select_launch(z, dtype, G, m, n, C, prev_masks, unit_group, U, track, p, idx, count, workspace, status,
+                         stream);
 }
 
 // rs3_select_queries for callers that cannot allocate device memory: the same
@@ -795,7 +1065,7 @@ extern "C" rs3_status rs3_select_queries_noalloc(const void *z, rs3_dtype dtype,
     if (need > RS3_NOALLOC_LIMIT) return RS3_ECAPACITY;
     const rs3_status s = select_check(z, dtype, G, m, n, C, prev_masks, unit_group, U, track, p, idx, count, status);
     if (s != RS3_OK) return s;
-    return select_launch(z, dtype, G, m, n, C, prev_masks, unit_group, U, track, p, idx, count, status, stream);
+    return select_launch(z, dtype, G, m, n, C, prev_masks, unit_group, U, track, p, idx, count, nullptr, status, stream);
 }
 
 extern "C" rs3_status rs3_write_keepset(const uint8_t *seed_masks, const int32_t *unit_group, int U,

@@ -28,7 +28,7 @@ def _masks(rng, U, m, n, density):
     return M.reshape(U, m * n)                          # every fourth unit's mask is empty
 
 
-def _run(m, n, C, dtype, ug, G, union, rho=0.3, r_s=4, c=14, seed=0, outlier=False, rounds=2, density=0.02, bbox=0):
+def _run(m, n, C, dtype, ug, G, union, rho=0.3, r_s=4, c=14, seed=0, outlier=False, rounds=2, density=0.02, bbox=0, both=False):
     rng = np.random.default_rng([seed, m, n, C])
     U, mn = len(ug), m * n
     ug = np.asarray(ug, np.int32)
@@ -39,7 +39,8 @@ def _run(m, n, C, dtype, ug, G, union, rho=0.3, r_s=4, c=14, seed=0, outlier=Fal
     idx = torch.full((U, max(k, 1)), -7, dtype=torch.int32, device="cuda")
     cnt = torch.full((U,), -7, dtype=torch.int32, device="cuda")
     st = torch.zeros(1, dtype=torch.int32, device="cuda")
-    ws = torch.empty(rs3.rs3_select_workspace_bytes(G, U, m, n), dtype=torch.uint8, device="cuda")
+    ws = torch.full((rs3.rs3_select_workspace_bytes(G, U, m, n),), 255, dtype=torch.uint8, device="cuda")
+    track_n, idx_n, cnt_n = track_d.clone(), idx.clone(), cnt.clone()
     for t in range(rounds):
         M = _masks(rng, U, m, n, density)
         if t:
@@ -56,6 +57,9 @@ def _run(m, n, C, dtype, ug, G, union, rho=0.3, r_s=4, c=14, seed=0, outlier=Fal
         for u in range(U):
             assert np.array_equal(i_d[u, :c_d[u]], sel.keep(u)), (t, u)
         assert np.array_equal(to_host(track_d), track), t
+        if both:                                        # the one launch of calls without a workspace
+            rs3.rs3_select_queries_noalloc(to_dev(z), dtype, G, m, n, C, to_dev(M), to_dev(ug), U, track_n, p, idx_n, cnt_n, st)
+            assert torch.equal(cnt, cnt_n) and torch.equal(idx, idx_n) and torch.equal(track_d, track_n), t
     assert int(st.item()) == 0
 
 
@@ -92,12 +96,12 @@ def test_seed_box_prior():
 
 
 @pytest.mark.parametrize("union", [False, True])
-def test_units_without_a_grid_are_skipped(union):
+def test_units_without_a_grid_are_skipped(union, C=64, more=0):
     """A group id out of range latches RS3_EINVAL, its unit keeps its tracker and
     selects nothing, the others are selected as usual."""
-    m, n, C, G = 30, 40, 64, 2
+    m, n, G = 30, 40, 2
     rng = np.random.default_rng(3)
-    ug = np.array([0, 5, 1, -1, 0], np.int32)
+    ug = np.array([0, 5, 1, -1, 0] + [0] * more, np.int32)
     U, mn = len(ug), m * n
     M = _masks(rng, U, m, n, 0.05)
     M[:, 7:200] = 1
@@ -119,3 +123,23 @@ def test_units_without_a_grid_are_skipped(union):
     for i, u in enumerate(good):
         assert c_d[u] == sel.count[i] and np.array_equal(i_d[u, :c_d[u]], sel.keep(i))
         assert np.array_equal(t_d[u], track[i])
+
+
+@pytest.mark.parametrize("m,n,C,dtype,ug,G,union,rho", [
+    (64, 64, 2048, "bf16", [0], 1, False, 0.1), (64, 64, 1024, "f32", [0, 1], 2, False, 0.3), (50, 65, 4096, "bf16", [0, 1, 0], 2, False, 0.02),
+    (128, 128, 1024, "bf16", [0], 1, True, 0.3), (64, 64, 256, "bf16", [0] * 70, 1, False, 0.2), (37, 33, 64, "bf16", [0, 1] * 9, 2, True, 0.3),
+    (24, 28, 264, "f32", [0] * 75, 1, True, 1.0), (40, 1, 64, "bf16", [0] * 9, 1, True, 0.3), (1, 500, 8, "bf16", [0] * 12, 1, True, 0.0),
+    (300, 31, 40, "f32", [0] * 10, 1, True, 0.05), (16384, 1, 64, "bf16", [0] * 9, 1, True, 0.3), (2, 2, 64, "bf16", [0] * 9, 1, True, 0.5),
+    (1, 3, 64, "bf16", [0] * 9, 1, True, 0.5)])
+def test_three_launches(m, n, C, dtype, ug, G, union, rho):
+    """Calls of wide rows, of many objects on one grid and of large unions go
+    through the workspace in three launches; the one launch of a call without a
+    workspace selects the same."""
+    _run(m, n, C, dtype, ug, G, union, rho=rho, density=0.3, both=True, bbox=len(ug) == 18)
+    if len(ug) > 1:
+        _run(m, n, C, dtype, ug, G, not union, rho=rho, density=0.3, both=True)
+
+
+@pytest.mark.parametrize("union", [False, True])
+def test_units_without_a_grid_in_three_launches(union):
+    test_units_without_a_grid_are_skipped(union, C=4096, more=10)
