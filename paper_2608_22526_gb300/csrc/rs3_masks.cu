@@ -150,11 +150,20 @@ __device__ __forceinline__ uint32_t cluster_rank()
 // acquire pair orders shared-memory writes before the barrier with reads of
 // them through DSMEM after it).  .aligned: a warp's lanes execute it together,
 // also after a loop or a branch that some of them left early
-__device__ __forceinline__ void cluster_barrier()
+__device__ __forceinline__ void cluster_arrive()
 {
     __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
-                 "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_barrier()
+{
+    cluster_arrive();
+    cluster_wait();
 }
 
 __device__ __forceinline__ uint32_t dsmem_addr(const void *p, uint32_t rank)
@@ -423,91 +432,177 @@ k_close_argmax(const float *__restrict__ logits, const int32_t *__restrict__ gst
 // ---------------------------------------------------------------------------
 // Seed box and down_s of pixel masks
 // ---------------------------------------------------------------------------
-// One launch: the CTAs of a cluster share a unit's rows.  Each finds its band's
-// extreme rows and columns (16-byte loads, eight in flight per thread; byte j of
-// a chunk is column 16 c + j) and writes its share of the grid mask; the boxes
-// meet through DSMEM, then the first CTA writes the tracker and each its share
-// of the filled grid box.  Bound by latency: 8 masks of 1024 x 1024 (8.5 MB, 1.3
-// us at the copy rate) and their write keep-sets take 15.9 us in two calls, near
-// the cost of issuing them; 26.5 us with three launches here and cell-by-cell
-// dilations there.
-constexpr int SEED_KC = 8, SEED_THREADS = 1024;
+// Masks of up to about 1 MB take one launch (k_seed): the KC <= 8 CTAs of a cluster
+// share a unit's rows.  Each finds its band's extreme rows and columns, the boxes
+// meet through DSMEM, then the first CTA writes the tracker and each its share of
+// the grid mask and of the filled grid box.  Bound by latency (3 us of launch,
+// barriers and reductions) and by what one SM can read, about 35 GB/s when all of
+// a cluster's do: larger masks are spread over all SMs, in three launches.
+constexpr int SEED_KC = 8, SEED_BATCH = 8;
+constexpr int SCAN_THREADS = 256, SCAN_CHUNKS = SCAN_THREADS * SEED_BATCH;   // k_seed_scan: a CTA's chunks, about
 
-__global__ void __cluster_dims__(SEED_KC, 1, 1) __launch_bounds__(SEED_THREADS)
-k_seed(const uint8_t *__restrict__ masks, int h, int w, int s, rs3_track *__restrict__ track,
-       uint8_t *__restrict__ grid, uint8_t *__restrict__ box)
+// The extreme set rows and columns (y0, x0, y1, x1) of rows [r0, r0 + nr) of a mask
+// of cpr 16-byte chunks per row, by a CTA; in every lane of its first warp.  `dx` is
+// blockDim.x modulo cpr.  Eight loads in flight per thread; byte j of a chunk is
+// column 16 c + j.  A thread's chunks ascend, so its first and last set ones give
+// its rows, and only a chunk that reaches past the columns seen so far is looked into.
+__device__ __forceinline__ int4 band_box(const uint8_t *__restrict__ M, int r0, int nr, uint32_t cpr, uint32_t dx)
 {
-    pdl_wait();
-    __shared__ int4 s_warp[SEED_THREADS / 32], s_box;        // (y0, x0, y1, x1)
-    const int u = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t rank = cluster_rank();
-    const uint8_t *M = masks + (size_t)u * h * w;
-    const int rows = (h + SEED_KC - 1) / SEED_KC, r0 = min((int)rank * rows, h), nr = min(rows, h - r0);
-    const int cpr = w >> 4;                                  // chunks per row
-    const uint4 *base = reinterpret_cast<const uint4 *>(M + (size_t)r0 * w);
-    int y0 = INT_MAX, x0 = INT_MAX, y1 = -1, x1 = -1;
-    const uint32_t chunks = (uint32_t)nr * cpr;
-    for (uint32_t c0 = threadIdx.x; c0 < chunks; c0 += 8 * SEED_THREADS) {
-        uint4 v[8];
+    __shared__ int4 s_warp[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const uint4 *base = reinterpret_cast<const uint4 *>(M + (size_t)r0 * cpr * 16);
+    const uint32_t chunks = (uint32_t)nr * cpr, T = blockDim.x;
+    uint32_t first = 0xffffffffu, last = 0u;                 // set chunks
+    int x0 = INT_MAX, x1 = -1;
+    uint32_t cx = threadIdx.x % cpr;                         // the next chunk's column
+    for (uint32_t c0 = threadIdx.x; c0 < chunks; c0 += SEED_BATCH * T) {
+        uint4 v[SEED_BATCH];
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-            v[k] = c0 + k * SEED_THREADS < chunks ? __ldg(base + c0 + k * SEED_THREADS) : make_uint4(0u, 0u, 0u, 0u);
+        for (int k = 0; k < SEED_BATCH; ++k)
+            v[k] = c0 + k * T < chunks ? __ldg(base + c0 + k * T) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            if ((v[k].x | v[k].y | v[k].z | v[k].w) == 0u) continue;
-            const uint32_t c = c0 + k * SEED_THREADS, row32 = c / (uint32_t)cpr;
-            const int row = (int)row32, xb = 16 * (int)(c - row32 * cpr);
-            const uint32_t wd[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+        for (int k = 0; k < SEED_BATCH; ++k) {
+            if ((v[k].x | v[k].y | v[k].z | v[k].w) != 0u) {
+                last = c0 + k * T;
+                first = min(first, last);
+                const int xb = 16 * (int)cx;
+                if (xb < x0 || xb + 15 > x1) {
+                    const uint32_t wd[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint32_t nz = __vcmpne4(wd[j], 0u);     // 0xff in every non-zero byte
-                if (nz) {
-                    x0 = min(x0, xb + 4 * j + ((__ffs(nz) - 1) >> 3));
-                    x1 = max(x1, xb + 4 * j + ((31 - __clz(nz)) >> 3));
+                    for (int j = 0; j < 4; ++j) {
+                        const uint32_t nz = __vcmpne4(wd[j], 0u);     // 0xff in every non-zero byte
+                        if (nz) {
+                            x0 = min(x0, xb + 4 * j + ((__ffs(nz) - 1) >> 3));
+                            x1 = max(x1, xb + 4 * j + ((31 - __clz(nz)) >> 3));
+                        }
+                    }
                 }
             }
-            y0 = min(y0, r0 + row);
-            y1 = max(y1, r0 + row);
+            cx += dx;
+            if (cx >= cpr) cx -= cpr;
         }
     }
-    const int m = h / s, n = w / s;
-    const uint32_t cells = (uint32_t)m * n, share = (cells + SEED_KC - 1) / SEED_KC;
-    const uint32_t ca = min(rank * share, cells), cb = min(ca + share, cells);
-    if (grid)
-        for (uint32_t c = ca + threadIdx.x; c < cb; c += SEED_THREADS) {
-            const uint32_t i = c / (uint32_t)n, j = c - i * n;
-            grid[(size_t)u * cells + c] = M[(size_t)i * s * w + (size_t)j * s] != 0;
-        }
+    int y0 = INT_MAX, y1 = -1;
+    if (x1 >= 0) {
+        y0 = r0 + (int)(first / cpr);
+        y1 = r0 + (int)(last / cpr);
+    }
     y0 = __reduce_min_sync(0xffffffffu, y0);
     x0 = __reduce_min_sync(0xffffffffu, x0);
     y1 = __reduce_max_sync(0xffffffffu, y1);
     x1 = __reduce_max_sync(0xffffffffu, x1);
     if (lane == 0) s_warp[warp] = make_int4(y0, x0, y1, x1);
     __syncthreads();
-    if (warp == 0) {
-        const int4 b = s_warp[lane];
-        y0 = __reduce_min_sync(0xffffffffu, b.x);
-        x0 = __reduce_min_sync(0xffffffffu, b.y);
-        y1 = __reduce_max_sync(0xffffffffu, b.z);
-        x1 = __reduce_max_sync(0xffffffffu, b.w);
-        if (lane == 0) s_box = make_int4(y0, x0, y1, x1);
+    int4 b = s_warp[lane < nw ? lane : 0];
+    if (warp == 0)
+        b = make_int4(__reduce_min_sync(0xffffffffu, b.x), __reduce_min_sync(0xffffffffu, b.y),
+                      __reduce_max_sync(0xffffffffu, b.z), __reduce_max_sync(0xffffffffu, b.w));
+    return b;
+}
+
+// Sizes of a call that the kernels would divide for.
+struct SeedDims {
+    int h, w, s, m, n;
+    int rows;            // image rows per CTA
+    uint32_t cpr, dx;    // chunks per row; threads of a CTA modulo that
+    uint32_t share;      // grid cells per CTA
+};
+
+__device__ __forceinline__ uint8_t in_box(const rs3_track &t, uint32_t c, int n)
+{
+    const int i = (int)(c / (uint32_t)n), j = (int)(c - (uint32_t)i * n);
+    return t.valid && i >= t.y0 && i <= t.y1 && j >= t.x0 && j <= t.x1;
+}
+
+__global__ void __launch_bounds__(512)
+k_seed(const uint8_t *__restrict__ masks, SeedDims d, int KC, rs3_track *__restrict__ track, uint8_t *__restrict__ grid,
+       uint8_t *__restrict__ box)
+{
+    pdl_wait();
+    __shared__ int4 s_box;                                   // (y0, x0, y1, x1)
+    const int u = blockIdx.y, lane = threadIdx.x & 31;
+    const uint32_t rank = KC > 1 ? cluster_rank() : 0u, T = blockDim.x;
+    const uint8_t *M = masks + (size_t)u * d.h * d.w;
+    const int r0 = min((int)rank * d.rows, d.h), nr = min(d.rows, d.h - r0);
+    const int4 b = band_box(M, r0, nr, d.cpr, d.dx);
+    if (threadIdx.x == 0) s_box = b;
+    if (KC > 1) cluster_arrive();                            // (orders s_box within the CTA too)
+    else __syncthreads();
+    // beside the other CTAs' arrivals
+    const uint32_t cells = (uint32_t)d.m * d.n, ca = min(rank * d.share, cells), cb = min(ca + d.share, cells);
+    if (grid)
+        for (uint32_t c = ca + threadIdx.x; c < cb; c += T) {
+            const uint32_t i = c / (uint32_t)d.n, j = c - i * d.n;
+            grid[(size_t)u * cells + c] = M[(size_t)i * d.s * d.w + (size_t)j * d.s] != 0;
+        }
+    int y0, x0, y1, x1;
+    if (KC > 1) {
+        cluster_wait();
+        const uint32_t from = dsmem_addr(&s_box, lane < KC ? lane : 0u);
+        y0 = __reduce_min_sync(0xffffffffu, (int)dsmem_ld_u32(from));
+        x0 = __reduce_min_sync(0xffffffffu, (int)dsmem_ld_u32(from + 4u));
+        y1 = __reduce_max_sync(0xffffffffu, (int)dsmem_ld_u32(from + 8u));
+        x1 = __reduce_max_sync(0xffffffffu, (int)dsmem_ld_u32(from + 12u));
+        cluster_arrive();
+    } else {
+        y0 = s_box.x; x0 = s_box.y; y1 = s_box.z; x1 = s_box.w;
     }
-    cluster_barrier();                                       // (orders s_box within the CTA too)
-    const uint32_t from = dsmem_addr(&s_box, lane < SEED_KC ? lane : 0u);
-    y0 = __reduce_min_sync(0xffffffffu, (int)dsmem_ld_u32(from));
-    x0 = __reduce_min_sync(0xffffffffu, (int)dsmem_ld_u32(from + 4u));
-    y1 = __reduce_max_sync(0xffffffffu, (int)dsmem_ld_u32(from + 8u));
-    x1 = __reduce_max_sync(0xffffffffu, (int)dsmem_ld_u32(from + 12u));
     // the pixel box divided by s (rounding down); no pixels: all zeros
     rs3_track t = {0, 0, 0, 0, 0, 0};
-    if (y1 >= 0) t = rs3_track{y0 / s, x0 / s, y1 / s, x1 / s, 1, 0};
+    if (y1 >= 0) t = rs3_track{y0 / d.s, x0 / d.s, y1 / d.s, x1 / d.s, 1, 0};
     if (rank == 0 && threadIdx.x == 0) track[u] = t;
     if (box)
-        for (uint32_t c = ca + threadIdx.x; c < cb; c += SEED_THREADS) {
-            const int i = (int)(c / (uint32_t)n), j = (int)(c - (uint32_t)i * n);
-            box[(size_t)u * cells + c] = t.valid && i >= t.y0 && i <= t.y1 && j >= t.x0 && j <= t.x1;
-        }
-    cluster_barrier();                                       // no CTA leaves while another reads its box
+        for (uint32_t c = ca + threadIdx.x; c < cb; c += T) box[(size_t)u * cells + c] = in_box(t, c, d.n);
+    if (KC > 1) cluster_wait();                              // no CTA leaves while another reads its box
+}
+
+// The three launches of larger masks.  The box is divided by s before it is merged
+// (rounding down keeps the order), so the tracker is in its final state after the
+// scan, but for the units without a set pixel.
+__global__ void k_seed_init(rs3_track *track, int U)
+{
+    pdl_wait();
+    const int u = blockIdx.x * blockDim.x + threadIdx.x;
+    if (u < U) track[u] = rs3_track{INT_MAX, INT_MAX, -1, -1, 0, 0};
+}
+
+// A CTA per band of rows and unit: its box, merged into the unit's tracker with
+// atomics, and its rows of the grid mask.
+__global__ void __launch_bounds__(SCAN_THREADS)
+k_seed_scan(const uint8_t *__restrict__ masks, SeedDims d, rs3_track *track, uint8_t *__restrict__ grid)
+{
+    pdl_wait();
+    const int u = blockIdx.y, r0 = blockIdx.x * d.rows, nr = min(d.rows, d.h - r0);
+    const uint8_t *M = masks + (size_t)u * d.h * d.w;
+    const int4 b = band_box(M, r0, nr, d.cpr, d.dx);
+    if (threadIdx.x == 0 && b.z >= 0) {
+        atomicMin(&track[u].y0, b.x / d.s);
+        atomicMin(&track[u].x0, b.y / d.s);
+        atomicMax(&track[u].y1, b.z / d.s);
+        atomicMax(&track[u].x1, b.w / d.s);
+        track[u].valid = 1;
+    }
+    if (!grid) return;
+    const int i0 = (r0 + d.s - 1) / d.s, i1 = min((r0 + nr + d.s - 1) / d.s, d.m);
+    for (uint32_t c = threadIdx.x; c < (uint32_t)(i1 - i0) * d.n; c += SCAN_THREADS) {
+        const uint32_t i = c / (uint32_t)d.n, j = c - i * d.n;
+        grid[((size_t)u * d.m + i0 + i) * d.n + j] = M[(size_t)(i0 + i) * d.s * d.w + (size_t)j * d.s] != 0;
+    }
+}
+
+// The filled grid box, and zeros for the tracker of a unit without a set pixel
+// (written by one thread: the others read `valid` alone of it, which stays 0).
+__global__ void __launch_bounds__(SCAN_THREADS)
+k_seed_finish(SeedDims d, rs3_track *track, uint8_t *__restrict__ box)
+{
+    pdl_wait();
+    const int u = blockIdx.y;
+    rs3_track t = {0, 0, 0, 0, 0, 0};
+    if (track[u].valid) t = track[u];
+    else if (blockIdx.x == 0 && threadIdx.x == 0) track[u] = t;
+    const uint32_t cells = (uint32_t)d.m * d.n, c0 = blockIdx.x * d.share, c1 = min(c0 + d.share, cells);
+    if (box)
+        for (uint32_t c = c0 + threadIdx.x; c < c1; c += SCAN_THREADS) box[(size_t)u * cells + c] = in_box(t, c, d.n);
 }
 
 }  // namespace
@@ -662,7 +757,49 @@ extern "C" rs3_status rs3_seed_from_masks(const uint8_t *masks, int U, int h, in
     if (h % s != 0 || w % s != 0) return RS3_EINVAL;
     if (U > 65535) return RS3_EUNSUPPORTED;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const cudaError_t e = launch_pdl(k_seed, dim3(SEED_KC, U), dim3(SEED_THREADS), 0, st, masks, h, w, s, track,
-                                     grid_masks, box_masks);
+    SeedDims d;
+    d.h = h; d.w = w; d.s = s; d.m = h / s; d.n = w / s;
+    d.cpr = (uint32_t)w / 16;
+    const long long chunks = (long long)h * d.cpr, cells = (long long)d.m * d.n;
+    // Over all SMs, in three launches, past 1 MB a mask or 16 MB in all (us per call
+    // in a graph, cluster and bands; called eagerly the three launches take 11.5 and
+    // the one 8 or its own time): 1 x 1024 x 1024 8.2 and 5.0, 1 x 1080 x 1920 11.6 and
+    // 5.0, 1 x 4096 x 4096 72 and 8, 16 x 1024 x 1024 10.8 and 8.2, 48 x 384 x 384 5.6
+    // and 6.1, 100 x 512 x 512 9.9 and 11.3, 48 x 1024 x 1024 17.8 and 14.7.
+    if (chunks > 65536 || U * chunks >= 1 << 20) {
+        d.rows = (int)std::min((long long)h, std::max(1ll, SCAN_CHUNKS / (long long)d.cpr));
+        d.dx = SCAN_THREADS % d.cpr;
+        d.share = 4 * SCAN_THREADS;
+        cudaError_t e = launch_pdl(k_seed_init, dim3((U + 255) / 256), dim3(256), 0, st, track, U);
+        if (e == cudaSuccess)
+            e = launch_pdl(k_seed_scan, dim3((h + d.rows - 1) / d.rows, U), dim3(SCAN_THREADS), 0, st, masks, d, track,
+                           grid_masks);
+        if (e == cudaSuccess)
+            e = launch_pdl(k_seed_finish, dim3(box_masks ? (unsigned)((cells + d.share - 1) / d.share) : 1u, U),
+                           dim3(SCAN_THREADS), 0, st, d, track, box_masks);
+        return e == cudaSuccess ? RS3_OK : RS3_ECUDA;
+    }
+    // Threads per unit: as many as load it in one batch of each, but no more than
+    // are resident at once (1024 per SM by their registers).
+    const long long want = std::max(256ll, std::min((chunks + SEED_BATCH - 1) / SEED_BATCH, 1024ll * rs3_sm_count() / U));
+    const int threads = want <= 128 * SEED_KC ? 256 : 512;
+    const int KC = (int)std::min((long long)SEED_KC, (want + threads - 1) / threads);
+    d.rows = (h + KC - 1) / KC;
+    d.dx = (uint32_t)threads % d.cpr;
+    d.share = (uint32_t)((cells + KC - 1) / KC);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(KC, U);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = KC;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_seed, masks, d, KC, track, grid_masks, box_masks);
     return e == cudaSuccess ? RS3_OK : RS3_ECUDA;
 }

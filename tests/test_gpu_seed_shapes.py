@@ -38,6 +38,14 @@ def test_seeds(U, h, w, s):
         assert np.array_equal(b[u], want)
 
 
+@pytest.mark.parametrize("U,h,w,s", [(3, 1040, 1056, 16), (20, 1024, 896, 32), (1, 40000, 32, 8), (1, 8, 200000, 8), (2, 1030, 2064, 2),
+                                     (200, 256, 256, 16), (400, 128, 128, 8), (7, 96, 208, 1), (50, 144, 144, 3)])
+def test_seeds_of_large_and_of_many_masks(U, h, w, s):
+    """Masks past 1 MB, or 16 MB in all, are spread in bands over all SMs; many
+    small ones get a CTA or two each."""
+    test_seeds(U, h, w, s)
+
+
 def _dilated(S, m, n, r):
     """Cells within Chebyshev distance r of a set one, by window counts (the
     oracle visits every window's cells: too slow for large radii)."""
