@@ -199,31 +199,32 @@ __device__ __forceinline__ uint32_t dsmem_ld(uint32_t a)
     return v;
 }
 
-// A mask's cells as bit words: f(y, k, words k and k + 1 of row y), by every
-// lane of the warp that loaded them (four rows of two words at a time).
-template <typename F>
-__device__ __forceinline__ void mask_words(const uint8_t *__restrict__ M, int m, int n, int WW, F f)
+// A mask's cells as bits of consecutive words, F[i / 32]: a warp's lanes read 32
+// adjacent cells, whatever the grid's shape, eight words at a time.
+__device__ __forceinline__ void flat_bits(const uint8_t *__restrict__ M, int mn, uint32_t *F)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int yb = warp; yb < m; yb += 4 * SEL_WARPS)
-        for (int k = 0; k < WW; k += 2) {
-            const uint8_t *row = M + yb * n + 32 * k + lane;
-            const bool in0 = 32 * k + lane < n, in1 = 32 * k + 32 + lane < n;
-            uint8_t v0[4], v1[4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nf = (mn + 31) >> 5;
+    for (int w0 = warp; w0 < nf; w0 += 8 * SEL_WARPS) {
+        uint8_t v[8];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const bool in = yb + q * SEL_WARPS < m;
-                v0[q] = in && in0 ? __ldg(row + q * SEL_WARPS * n) : (uint8_t)0;
-                v1[q] = in && in1 ? __ldg(row + q * SEL_WARPS * n + 32) : (uint8_t)0;
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int y = yb + q * SEL_WARPS;
-                if (y >= m) break;
-                const uint32_t b0 = __ballot_sync(0xffffffffu, v0[q] != 0), b1 = __ballot_sync(0xffffffffu, v1[q] != 0);
-                f(y, k, b0, b1);
-            }
+        for (int q = 0; q < 8; ++q) {
+            const int i = 32 * (w0 + q * SEL_WARPS) + lane;
+            v[q] = i < mn ? __ldg(M + i) : (uint8_t)0;
         }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const uint32_t x = __ballot_sync(0xffffffffu, v[q] != 0);
+            if (lane == 0 && w0 + q * SEL_WARPS < nf) F[w0 + q * SEL_WARPS] = x;
+        }
+    }
+}
+
+// Word k of row y from them.
+__device__ __forceinline__ uint32_t row_word(const uint32_t *F, int nf, int n, int y, int k)
+{
+    const int i = y * n + 32 * k, w = i >> 5, left = n - 32 * k;
+    const uint32_t x = __funnelshift_r(F[w], w + 1 < nf ? F[w + 1] : 0u, i & 31);
+    return left < 32 ? x & ((1u << left) - 1u) : x;
 }
 
 // Chebyshev dilation of bit words by r: along the rows, by at most 31 cells (a
@@ -274,18 +275,22 @@ __device__ void unit_prior(const uint8_t *__restrict__ M, int m, int n, const Wo
     const int WW = walk.WW, words = m * WW;
     if (threadIdx.x == 0) t = *track;
     int y0 = INT_MAX, x0 = INT_MAX, y1 = -1, x1 = -1;
-    mask_words(M, m, n, WW, [&](int y, int k, uint32_t b0, uint32_t b1) {
-        if (lane == 0) {
-            a[y * WW + k] = b0;
-            if (k + 1 < WW) a[y * WW + k + 1] = b1;
-        }
-        if (b0 | b1) {
+    flat_bits(M, m * n, b);
+    __syncthreads();
+    walk.each(words, [&](int w, int y, int k) {
+        const uint32_t x = row_word(b, (m * n + 31) >> 5, n, y, k);
+        a[w] = x;
+        if (x) {
             y0 = min(y0, y);
             y1 = max(y1, y);
-            x0 = min(x0, 32 * k + (b0 ? __ffs(b0) - 1 : __ffs(b1) + 31));
-            x1 = max(x1, 32 * k + (b1 ? 63 - __clz(b1) : 31 - __clz(b0)));
+            x0 = min(x0, 32 * k + __ffs(x) - 1);
+            x1 = max(x1, 32 * k + 31 - __clz(x));
         }
     });
+    y0 = __reduce_min_sync(0xffffffffu, y0);
+    x0 = __reduce_min_sync(0xffffffffu, x0);
+    y1 = __reduce_max_sync(0xffffffffu, y1);
+    x1 = __reduce_max_sync(0xffffffffu, x1);
     if (lane == 0) { s_box[0][warp] = y0; s_box[1][warp] = x0; s_box[2][warp] = y1; s_box[3][warp] = x1; }
     __syncthreads();
     if (warp == 0) {
@@ -564,8 +569,10 @@ struct Place {
     }
 };
 
+// (bf16: eight rows' loads in flight take 64 registers; left to itself the compiler
+// stops at 54 and waits in between: 16 x 3 objects of 96 x 96 23.1 us, 21.0 so)
 template <typename T>
-__global__ void __launch_bounds__(SEL_THREADS)
+__global__ void __launch_bounds__(SEL_THREADS, sizeof(T) == 2 ? 2 : 1)
 k_select(const T *__restrict__ z, const uint8_t *__restrict__ masks, int m, int n, int C, int lpr,
          const int32_t *__restrict__ unit_group, int G, int U, rs3_track *__restrict__ track, int r_s, int c,
          int bbox_mode, int union_mode, int k, int KC, int32_t *__restrict__ idx, int32_t *__restrict__ count,
@@ -655,11 +662,18 @@ k_select(const T *__restrict__ z, const uint8_t *__restrict__ masks, int m, int 
     }
     __syncthreads();
     const uint32_t below = (1u << lane) - 1u;
-    for (int y = warp; y < m; y += SEL_WARPS)
-        for (int k = 0; k < WW; ++k) {
-            const uint32_t bits = P[y * WW + k];
-            if (bits >> lane & 1u) list[pref[y * WW + k] + __popc(bits & below)] = (uint16_t)(y * n + 32 * k + lane);
+    if (n >= 8) {                                        // a lane per bit, or, in narrow rows, a thread per row
+        for (int y = warp; y < m; y += SEL_WARPS)
+            for (int k = 0; k < WW; ++k) {
+                const uint32_t bits = P[y * WW + k];
+                if (bits >> lane & 1u) list[pref[y * WW + k] + __popc(bits & below)] = (uint16_t)(y * n + 32 * k + lane);
+            }
+    } else {
+        for (int y = threadIdx.x; y < m; y += SEL_THREADS) {
+            uint32_t at = pref[y];
+            for (uint32_t bits = P[y]; bits; bits &= bits - 1) list[at++] = (uint16_t)(y * n + __ffs(bits) - 1);
         }
+    }
     const bool keep_all = nP <= (uint32_t)k;
     const uint32_t n_kept = keep_all ? nP : (uint32_t)k;
     __syncthreads();
@@ -842,8 +856,52 @@ k_rank(int mn, const int32_t *__restrict__ unit_group, int G, int union_mode, in
 
 // ---------------------------------------------------------------------------
 // k_write_keepset: Eq. 8 with the 5% / 95% fall-through of Sec. 3.2, a CTA per
-// unit on bit words: 64 x 64 cells, radius 12, took 16.5 us (cold) cell by cell.
+// unit on bit words.  64 x 64 cells, radius 24, in a graph: 4.8 us, 12.2 cell by
+// cell; union of 48 objects 13.7 us, 46.
 // ---------------------------------------------------------------------------
+// The union of a group's masks as bits (as flat_bits): four words of eight masks
+// in flight per warp.  Every thread of the CTA calls it.
+__device__ __forceinline__ void group_bits(const uint8_t *__restrict__ masks, int mn, const int32_t *__restrict__ unit_group,
+                                           int U, int g, uint32_t *F)
+{
+    __shared__ int s_unit[SEL_THREADS], s_n;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nf = (mn + 31) >> 5;
+    for (int w = threadIdx.x; w < nf; w += SEL_THREADS) F[w] = 0u;
+    for (int v0 = 0; v0 < U; v0 += SEL_THREADS) {
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();
+        const int v = v0 + threadIdx.x;
+        if (v < U && unit_group[v] == g) s_unit[atomicAdd(&s_n, 1)] = v;     // (in any order)
+        __syncthreads();
+        const int units = s_n;
+        for (int w0 = warp; w0 < nf; w0 += 4 * SEL_WARPS) {
+            uint32_t any[4] = {0u, 0u, 0u, 0u};
+            for (int j0 = 0; j0 < units; j0 += 8) {
+                uint8_t x[8][4];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const uint8_t *M = masks + (size_t)s_unit[min(j0 + j, units - 1)] * mn;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int i = 32 * (w0 + q * SEL_WARPS) + lane;
+                        x[j][q] = i < mn ? __ldg(M + i) : (uint8_t)0;
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) any[q] |= x[j][q];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t b = __ballot_sync(0xffffffffu, any[q] != 0u);
+                if (lane == 0 && w0 + q * SEL_WARPS < nf) F[w0 + q * SEL_WARPS] |= b;   // always this warp's
+            }
+        }
+        __syncthreads();
+    }
+}
+
 __global__ void __launch_bounds__(SEL_THREADS)
 k_write_keepset(const uint8_t *__restrict__ seeds, const int32_t *__restrict__ unit_group, int U, int m, int n,
                 int D_w, double fall_lo, double fall_hi, int fall_through, int union_mode, uint8_t *__restrict__ kw)
@@ -851,28 +909,12 @@ k_write_keepset(const uint8_t *__restrict__ seeds, const int32_t *__restrict__ u
     pdl_wait();
     extern __shared__ __align__(16) uint8_t sel_raw[];
     const int mn = m * n, WW = (n + 31) >> 5, words = m * WW, u = blockIdx.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t *a = reinterpret_cast<uint32_t *>(sel_raw), *b = a + words;
     const WordWalk walk(WW);
-    mask_words(seeds + (size_t)u * mn, m, n, WW, [&](int y, int k, uint32_t b0, uint32_t b1) {
-        if (lane == 0) {
-            a[y * WW + k] = b0;
-            if (k + 1 < WW) a[y * WW + k + 1] = b1;
-        }
-    });
-    if (union_mode) {
-        const int g = unit_group[u];
-        for (int v0 = 0; v0 < U; v0 += 32) {
-            uint32_t in = __ballot_sync(0xffffffffu, v0 + lane < U && v0 + lane != u && unit_group[min(v0 + lane, U - 1)] == g);
-            for (; in; in &= in - 1)                       // (a word is always the same warp's)
-                mask_words(seeds + (size_t)(v0 + __ffs(in) - 1) * mn, m, n, WW, [&](int y, int k, uint32_t b0, uint32_t b1) {
-                    if (lane == 0) {
-                        a[y * WW + k] |= b0;
-                        if (k + 1 < WW) a[y * WW + k + 1] |= b1;
-                    }
-                });
-        }
-    }
+    if (union_mode) group_bits(seeds, mn, unit_group, U, unit_group[u], b);
+    else flat_bits(seeds + (size_t)u * mn, mn, b);
+    __syncthreads();
+    walk.each(words, [&](int w, int y, int k) { a[w] = row_word(b, (mn + 31) >> 5, n, y, k); });
     __syncthreads();
     uint32_t own = 0, area;
     for (int w = threadIdx.x; w < words; w += SEL_THREADS) own += __popc(a[w]);
@@ -886,9 +928,14 @@ k_write_keepset(const uint8_t *__restrict__ seeds, const int32_t *__restrict__ u
     uint32_t *from = dilate_rows(a, b, words, n, D_w, walk), *to = from == a ? b : a;
     walk.each(words, [&](int w, int y, int) { to[w] = column_or(from, w, y, m, D_w, WW); });
     __syncthreads();
-    for (int y = warp; y < m; y += SEL_WARPS)
-        for (int k = 0; k < WW; ++k)
-            if (32 * k + lane < n) out[y * n + 32 * k + lane] = (uint8_t)(to[y * WW + k] >> lane & 1u);
+    const int dy = SEL_THREADS / n, dx = SEL_THREADS - dy * n;
+    int y = (int)threadIdx.x / n, x = (int)threadIdx.x - y * n;
+    for (int i = threadIdx.x; i < mn; i += SEL_THREADS) {
+        out[i] = (uint8_t)(to[y * WW + (x >> 5)] >> (x & 31) & 1u);
+        y += dy;
+        x += dx;
+        if (x >= n) { x -= n; ++y; }
+    }
 }
 
 inline int next_pow2(int x)

@@ -80,3 +80,19 @@ def test_write_keepsets(m, n, D_w, union):
         assert np.array_equal(to_host(kw), ref), fall
         if D_w <= 5 and mn <= 4096:
             assert np.array_equal(ref, orc.write_keepset(S, ug, m, n, D_w, fall_through=fall, union_mode=union))
+
+
+@pytest.mark.parametrize("U,G,m,n", [(600, 3, 30, 33), (40, 1, 64, 64), (9, 2, 2100, 7), (17, 1, 5, 300)])
+def test_write_keepsets_of_large_groups(U, G, m, n):
+    """More units than the CTA lists at a time, more than eight of a group, rows
+    shorter and longer than a word."""
+    rng = np.random.default_rng([U, m, n])
+    ug = rng.integers(0, G, U).astype(np.int32)
+    S = np.zeros((U, m * n), np.uint8)
+    S[np.arange(U)[::2], rng.integers(0, m * n, size=U)[::2]] = 255
+    p = rs3.default_params(D_w=3, union_mode=1, fall_through=0)
+    kw = torch.full((U, m * n), 77, dtype=torch.uint8, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    rs3.rs3_write_keepset(to_dev(S), to_dev(ug), U, m, n, p, kw, st)
+    ref = [_dilated(np.any(S[ug == g] != 0, axis=0), m, n, 3) for g in range(G)]
+    assert np.array_equal(to_host(kw), np.stack([ref[g] for g in ug]))
