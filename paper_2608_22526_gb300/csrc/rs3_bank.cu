@@ -218,6 +218,14 @@ k_commit(const uint8_t *__restrict__ k_new, const uint8_t *__restrict__ v_new,
         off += w < warp ? s_wc[w] : 0;
         nk += s_wc[w];
     }
+    // Once every read of the old counters by this CTA is done it arrives, with its
+    // kept cells (high half), ahead of its stores: the fence would wait for those.
+    // The last CTA of the unit to arrive publishes.
+    unsigned long long arrived = 0;
+    const auto arrive = [&]() {
+        __threadfence();
+        arrived = atomicAdd(reinterpret_cast<unsigned long long *>(mu + BM_ARRIVE), ((unsigned long long)nk << 32) + 1ull);
+    };
     if (nk > 0) {                                            // uniform over the CTA
         if (keep) {
             uint32_t lm;
@@ -266,6 +274,7 @@ k_commit(const uint8_t *__restrict__ k_new, const uint8_t *__restrict__ v_new,
             s_ok = after.ok;
         }
         __syncthreads();
+        if (threadIdx.x == 0) arrive();
         if (s_ok) {
             const int64_t row0 = s_row0;
             uint8_t *kdst = k_store + (size_t)u * bk.rows_per_unit * row_bytes;
@@ -280,12 +289,8 @@ k_commit(const uint8_t *__restrict__ k_new, const uint8_t *__restrict__ v_new,
         }
     }
 
-    // every read of the old counters by this CTA is done: arrive, with its kept
-    // cells (high half); the last CTA of the unit to arrive publishes
     if (threadIdx.x != 0) return;
-    __threadfence();
-    const unsigned long long arrived = atomicAdd(reinterpret_cast<unsigned long long *>(mu + BM_ARRIVE),
-                                                 ((unsigned long long)nk << 32) + 1ull);
+    if (nk == 0) arrive();
     if ((uint32_t)arrived != gridDim.x - 1) return;
     __threadfence();
     const int64_t L = (int64_t)(arrived >> 32) + nk;
@@ -421,21 +426,26 @@ rs3_status commit_launch(const rs3_bank *bank, const void *k_new, const void *v_
     const int mn = bank->mn;
     const int64_t row_bytes = (int64_t)bank->D * (int64_t)elem_bytes(bank->dtype);
     // 128-cell chunks, or 64-cell ones where those would give under two CTAs per SM
-    const bool small = (int64_t)((mn + 127) / 128) * bank->U < 2ll * rs3_sm_count();
+    // (without a mask only where all 64-cell CTAs are resident: all of them copy)
+    const int64_t two_per_sm = 2ll * rs3_sm_count();
+    const bool few = (int64_t)((mn + 127) / 128) * bank->U < two_per_sm;
+    const bool small = few && (rope || keep_mask || (int64_t)((mn + 63) / 64) * bank->U <= two_per_sm);
     const int chunk = small ? 64 : 128;
     const dim3 grid((unsigned)((mn + chunk - 1) / chunk), (unsigned)bank->U);
     // Warps copying a chunk and rows in flight per warp (us per call, the others
-    // measured for the same shapes): rotated keys, 3 CTAs of 8 warps x 4 rows,
-    // 16 x 3 objects 42.4 (2 rows 39.4, but 26.6 against 22.4 on 12 objects;
-    // 4 CTAs 50.7, spilled); keys as given, small launches 8 warps x 4 rows 8.4
-    // (4 x 8: 10.1), large ones 4 x 8 32.4 (8 x 4: 36.7).
+    // measured for the same shapes).  Rotated keys: 3 CTAs of 8 warps x 4 rows;
+    // 16 x 3 objects 41 (2 rows 39.4, but 26.6 against 22.4 on 12 objects); the 80
+    // registers of 3 CTAs spill 184 bytes per thread, 4 CTAs more (50.7).  Keys as
+    // given: 2 CTAs of 8 warps x 8 rows for few CTAs, 8 objects of 64 x 64 7.2 and,
+    // without a mask, 13.6 in 128-cell chunks, 14.4 in 64-cell ones (2 warps x 16 7.8
+    // and 15.1, 8 x 4 7.1 and 14.8, rows of 4 KB 22 and 38); 4 x 8 for many CTAs.
     int threads = 256;
     void (*kern)(const uint8_t *, const uint8_t *, const uint8_t *, int, int, int64_t, BankDev, uint8_t *,
                  uint8_t *, int32_t *, const float *, int, int);
     if (rope) {
         kern = small ? k_commit<64, true, 256, 4, 3> : k_commit<128, true, 256, 4, 3>;
-    } else if (small) {
-        kern = k_commit<64, false, 256, 4, 4>;
+    } else if (few) {
+        kern = small ? k_commit<64, false, 256, 8, 2> : k_commit<128, false, 256, 8, 2>;
     } else {
         kern = k_commit<128, false, 128, 8, 4>;
         threads = 128;

@@ -7,6 +7,7 @@ ring wrap and eviction, with keys stored plain and rotated.  Every bank row
 and counter is checked against the oracle's bank."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import oracle as orc
 from paper_2608_22526_gb300 import rs3, synth
@@ -61,3 +62,35 @@ def test_commit_odd_grid_wide_rows_wrap(m, n, U, frames, rope):
             tol = 2.0 ** -7 * np.abs(r) + 2.0 ** -20 * max(float(np.abs(r).max()), 1e-30)
             assert (np.abs(g - r) <= tol).all(), f"K rows of unit {u}"
             assert (ks[u][rows] == ob.K[u][rows]).mean() > 0.99, f"K rows of unit {u}"
+
+
+@pytest.mark.parametrize("m,n,U,masked", [(37, 45, 2, False), (37, 45, 20, False), (37, 45, 20, True), (96, 96, 6, True), (96, 96, 6, False),
+                                          (70, 71, 12, False)])
+def test_commit_of_whole_and_sparse_frames(m, n, U, masked):
+    """Every shape of the copy for keys as given: 64-cell chunks, 128-cell ones
+    without a mask where their CTAs are few, and the large launch; units of one
+    kept cell, none and all, the ring wrapping."""
+    mn, H, d, window = m * n, 2, 64, 2
+    rng = np.random.default_rng([m, U])
+    bank = rs3.Bank(U, H, d, "bf16", mn, 0, window, window * mn, window, 0)
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ob = orc.OracleBank(U, H * d, "bf16", mn, 0, window, bank.ring_cap, bank.max_frames, 0)
+    for t in range(4):
+        k, v = (synth.random_bf16(rng, (U, mn, H * d)) for _ in range(2))
+        mask = None
+        if masked:
+            mask = (rng.random((U, mn)) < rng.random((U, 1))).astype(np.uint8) * 255
+            mask[t % U] = 1
+            mask[(t + 1) % U] = 0
+            mask[(t + 2) % U] = 0
+            mask[(t + 2) % U, rng.integers(0, mn)] = 1
+        rs3.rs3_bank_commit(bank, to_dev(k), to_dev(v), None if mask is None else to_dev(mask), 0, st)
+        assert ob.commit(k, v, mask, 0) == [0] * U
+    assert int(st.item()) == 0
+    meta, fr = rs3.rs3_bank_read_meta(bank)
+    ks, vs = to_host(bank.k_store), to_host(bank.v_store)
+    for u in range(U):
+        assert list(meta[u, :2]) == list(ob.state[u, :2]) and meta[u, 7] == ob.length(u)
+        assert [tuple(x) for x in fr[u, : meta[u, 3]]] == ob.frames(u)
+        rows = ob.logical_rows(u)
+        assert np.array_equal(ks[u][rows], ob.K[u][rows]) and np.array_equal(vs[u][rows], ob.V[u][rows])
