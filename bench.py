@@ -703,8 +703,8 @@ def gpu_arm(args):
         dist.destroy_process_group()
 
 
-ATTEND_KERNELS = "k_plan + k_readout_tc or k_readout_pair (in place: no pass-through)"
-RUN_KERNEL = "k_readout_tc, or k_readout_pair for heads of 64 and 128 (tcgen05 attention kernels; bf16 workloads)"
+ATTEND_KERNELS = "k_plan + k_readout_tc or k_readout_either (in place: no pass-through)"
+RUN_KERNEL = "k_readout_tc, or k_readout_either for heads of 64 and 128 (tcgen05 attention kernels; bf16 workloads)"
 
 
 def launches_per_pass(w):
@@ -884,7 +884,7 @@ def readout_source_hash():
     import re
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2608_22526_gb300", "csrc")
-    for f in ("rs3_readout.cu", "rs3_readout_tc.cu", "rs3_readout_pair.cu", "rs3_readout_common.cuh",
+    for f in ("rs3_readout.cu", "rs3_readout_tc.cu", "rs3_readout_tc.cuh", "rs3_readout_pair.cu", "rs3_readout_common.cuh",
               "rs3_tc_host.cuh", "rs3_tc_ptx.cuh"):
         p = os.path.join(csrc, f)
         if os.path.exists(p):

@@ -62,9 +62,12 @@ struct CombineItem {
 };
 
 struct ReadoutHeader {
-    int32_t n_items;
+    int32_t n_items;        // bound on the item indices
     int32_t n_combine;
-    int32_t pad[30];
+    int32_t slices;
+    int32_t n_part;         // partial pieces of all split groups
+    int32_t bm;             // query rows of an item: which kernel the items are for
+    int32_t pad[27];
 };
 
 struct ReadoutLayout {      // byte offsets inside the workspace

@@ -4,7 +4,8 @@
 //
 // Launch sequence (no host synchronisation).  Attend phase:
 //   k_plan         one CTA: per unit, the bank's row ranges (pinned, ring
-//                  pieces, pointers) and a balanced work list of
+//                  pieces, pointers), for bf16 heads of 64 and 128 the number of
+//                  query tiles per item, and a balanced work list of
 //                  (unit, head, query tile, KV tile range) items; long banks
 //                  are split along the keys so every SM gets work; out of place
 //                  the launch's other CTAs write out = residual (or zeros)
@@ -31,14 +32,35 @@ namespace {
 // ---------------------------------------------------------------------------
 // k_plan: ranges and the work list
 // ---------------------------------------------------------------------------
-__device__ RangeSet unit_ranges(const ReadoutArgs &a, int u, int cnt)
+// A unit's part of the plan: kept queries and the bank's row ranges, without tiles.
+// What is wrong with its inputs is latched by the calls with `latch`; a unit without a
+// valid grid or bank has no work.
+__device__ RangeSet unit_ranges(const ReadoutArgs &a, int u, bool latch)
 {
-    RangeSet rs;
+    // every load first (none depends on another), then the checks
     const int64_t *mu = a.meta + (int64_t)u * a.meta_stride_words;
-    const int64_t cond = mu[BM_COND_LEN];
-    const int64_t head = mu[BM_HEAD], tail = mu[BM_TAIL], ptr = mu[BM_PTRLEN];
+    int cnt = a.count[u];
+    const int g = a.unit_group[u];
+    const int64_t head = mu[BM_HEAD], tail = mu[BM_TAIL], cond = mu[BM_COND_LEN], ptr = mu[BM_PTRLEN];
+    RangeSet rs;
     for (int r = 0; r < 4; ++r) { rs.start[r] = 0; rs.len[r] = 0; rs.tiles[r] = 0; }
-    rs.start[0] = 0;
+    rs.n_tiles = rs.nq = rs.cnt = 0;
+    rs.splits = 1;
+    rs.slot_base = -1;
+    if (cnt < 0 || cnt > a.k_max) {
+        if (latch) latch_status(a.status, RS3_EINVAL);
+        cnt = cnt < 0 ? 0 : a.k_max;
+    }
+    if (g < 0 || g >= a.G) {
+        if (latch) latch_status(a.status, RS3_EINVAL);
+        cnt = 0;
+    }
+    if (!(head >= 0 && tail >= head && tail - head <= a.ring_cap && cond >= 0 && cond <= a.pinned_cap && ptr >= 0 &&
+          ptr <= a.n_ptr)) {
+        if (latch) latch_status(a.status, RS3_EINTERNAL);
+        return rs;
+    }
+    rs.cnt = cnt;
     rs.len[0] = (int32_t)cond;
     const int64_t live = tail - head;
     if (live > 0 && a.ring_cap > 0) {
@@ -51,17 +73,20 @@ __device__ RangeSet unit_ranges(const ReadoutArgs &a, int u, int cnt)
     }
     rs.start[3] = a.pinned_cap + a.ring_cap;
     rs.len[3] = (int32_t)ptr;
-    int nt = 0;
-    for (int r = 0; r < 4; ++r) {
-        rs.tiles[r] = (rs.len[r] + a.BN - 1) / a.BN;
-        nt += rs.tiles[r];
-    }
-    rs.n_tiles = nt;
-    rs.cnt = cnt;
-    rs.nq = (cnt + a.BM - 1) / a.BM;
-    rs.splits = 1;
-    rs.slot_base = -1;
     return rs;
+}
+
+// Its key tiles of BN rows (a power of two) and query tiles of BM.
+__device__ __forceinline__ void cut_tiles(RangeSet &rs, int BM, int BN)
+{
+    const int sh = 31 - __clz(BN);
+    rs.n_tiles = 0;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        rs.tiles[r] = (rs.len[r] + BN - 1) >> sh;
+        rs.n_tiles += rs.tiles[r];
+    }
+    rs.nq = (rs.cnt + BM - 1) >> (31 - __clz(BM));
 }
 
 // Exclusive block scan of an (int64, int32) pair per thread; returns the
@@ -135,6 +160,7 @@ struct PlanView {
     int64_t W;
     int P;
     int ov;              // leading slots of a group (the start-up cost)
+    int mark;            // of every item range: RS3_PAIR_ITEMS or 0
 };
 
 // b W / P; in 32 bits when b W cannot reach 2^32 (W < 2^22, b < 1024)
@@ -173,7 +199,8 @@ __device__ void plan_slice(const ReadoutArgs &a, const PlanView &v, int b, int &
     c.pad[1] = c.pad[2] = 0;                      // pad[1]: the unit's kept queries
     n_part = 0;
     if (lo >= hi) {
-        a.cta_items[2 * b] = a.cta_items[2 * b + 1] = 0;
+        a.cta_items[2 * b] = v.mark;
+        a.cta_items[2 * b + 1] = 0;
         return;
     }
     // one search and its divisions for the slice's first group; the walk from
@@ -228,11 +255,42 @@ __device__ void plan_slice(const ReadoutArgs &a, const PlanView &v, int b, int &
             if (u == v.U) break;
         }
     }
-    a.cta_items[2 * b] = (int32_t)(first < 0 ? 0 : first);
+    a.cta_items[2 * b] = (int32_t)(first < 0 ? 0 : first) | v.mark;
     a.cta_items[2 * b + 1] = (int32_t)(first < 0 ? 0 : last + 1);
 }
 
 constexpr int PLAN_THREADS = 256;
+
+// Whether two query tiles per CTA are the faster for a call (bf16 heads of 64 and
+// 128): by the score tiles (128 queries x 128 keys) that both kernels go through,
+// S1 of single tiles and S2 of pairs.  A pair costs 1.7 (d = 128: 1.65) times
+// a tile, and as much again as 1 (3.75) tiles per CTA more to start.  Over 263 shapes,
+// 1 to 16 objects of 1 to 8 heads, 300 to 4 096 kept queries and banks of 2 to 7 frames,
+// the choice is within 9% of the better one, and right beyond that: one object's 3
+// to 7 tiles per head 15.6 us against 25.2 with pairs, 16 objects 260 against 165.
+// `mine` is this thread's unit of the first round.  Every thread of the CTA calls it.
+__device__ __forceinline__ bool two_tiles(const ReadoutArgs &a, const RangeSet &mine)
+{
+    __shared__ float s_sum[2][PLAN_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float s1 = 0.f, s2 = 0.f;
+    for (int u = threadIdx.x; u < a.U; u += PLAN_THREADS) {
+        RangeSet rs = u < PLAN_THREADS ? mine : unit_ranges(a, u, false);
+        cut_tiles(rs, 128, 128);
+        s1 += (float)rs.nq * (float)rs.n_tiles;
+        s2 += (float)((rs.nq + 1) >> 1) * (float)rs.n_tiles;
+    }
+    s1 = warp_sum(s1);
+    s2 = warp_sum(s2);
+    if (lane == 0) { s_sum[0][warp] = s1; s_sum[1][warp] = s2; }
+    __syncthreads();
+    s1 = s2 = 0.f;
+#pragma unroll
+    for (int w = 0; w < PLAN_THREADS / 32; ++w) { s1 += s_sum[0][w]; s2 += s_sum[1][w]; }
+    s1 *= a.H;
+    s2 *= a.H;
+    return a.d == 64 ? s1 > 1.7f * s2 + (float)a.n_sm : s1 > 1.65f * s2 + 3.75f * (float)a.n_sm;
+}
 
 // Out of place, CTAs 1.. of the launch also write out = residual (or zeros) on
 // every cell: unselected cells equal the residual bit for bit (Eq. 6 S_K), and
@@ -255,6 +313,12 @@ __global__ void __launch_bounds__(PLAN_THREADS) k_plan(ReadoutArgs a, int64_t nv
     int32_t *s_gb = reinterpret_cast<int32_t *>(s_wg + a.U), *s_nt = s_gb + (a.U + 1), *s_cnt = s_nt + a.U;
     __shared__ int s_np, s_nc;
     if (threadIdx.x == 0) { s_np = 0; s_nc = 0; }
+    RangeSet mine = {};                             // this thread's unit of the first round
+    if (threadIdx.x < a.U) mine = unit_ranges(a, threadIdx.x, true);
+    struct { int BM, BN, ov, min_chunk; } cfg = {a.BM, a.BN, a.plan_ov, a.min_chunk};
+    // pairs of query tiles: 3 and 12 leading slots, and slices of 2 and 6, are slower
+    const bool pairs = a.either && two_tiles(a, mine);
+    if (pairs) cfg = {2 * a.BM, 128, 6, 4};
     // per unit: the bank's ranges, its groups and their width, scanned into
     // slot and group bases (rounds of blockDim units)
     int64_t run = 0;
@@ -264,31 +328,10 @@ __global__ void __launch_bounds__(PLAN_THREADS) k_plan(ReadoutArgs a, int64_t nv
         int64_t slots = 0;
         int32_t groups = 0;
         if (u < a.U) {
-            // every load first (none depends on another), then the checks
-            const int64_t *mu = a.meta + (int64_t)u * a.meta_stride_words;
-            int cnt = a.count[u];
-            const int g = a.unit_group[u];
-            const int64_t head = mu[BM_HEAD], tail = mu[BM_TAIL], cond = mu[BM_COND_LEN], ptr = mu[BM_PTRLEN];
-            if (cnt < 0 || cnt > a.k_max) {
-                latch_status(a.status, RS3_EINVAL);
-                cnt = cnt < 0 ? 0 : a.k_max;
-            }
-            if (g < 0 || g >= a.G) {                // no work for a unit without a valid grid
-                latch_status(a.status, RS3_EINVAL);
-                cnt = 0;
-            }
-            const bool sane = head >= 0 && tail >= head && tail - head <= a.ring_cap && cond >= 0 &&
-                              cond <= a.pinned_cap && ptr >= 0 && ptr <= a.n_ptr;
-            RangeSet rs;
-            if (!sane) {
-                latch_status(a.status, RS3_EINTERNAL);
-                for (int r = 0; r < 4; ++r) { rs.start[r] = 0; rs.len[r] = 0; rs.tiles[r] = 0; }
-                rs.n_tiles = 0; rs.cnt = 0; rs.nq = 0; rs.splits = 1; rs.slot_base = -1;
-            } else {
-                rs = unit_ranges(a, u, cnt);
-            }
+            RangeSet rs = u0 > 0 ? unit_ranges(a, u, true) : mine;
+            cut_tiles(rs, cfg.BM, cfg.BN);
             a.ranges[u] = rs;
-            s_wg[u] = (int64_t)a.plan_ov + rs.n_tiles;
+            s_wg[u] = (int64_t)cfg.ov + rs.n_tiles;
             s_nt[u] = rs.n_tiles;
             s_cnt[u] = rs.cnt;
             groups = rs.nq * a.H;
@@ -308,7 +351,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) k_plan(ReadoutArgs a, int64_t nv
         s_tb[a.U] = run;
         s_gb[a.U] = grun;
     }
-    int64_t P = (run + a.min_chunk - 1) / a.min_chunk;
+    int64_t P = (run + cfg.min_chunk - 1) / cfg.min_chunk;
     if (P > a.grid_ctas) P = a.grid_ctas;
     __syncthreads();
     // One unit: its groups are equally long.  With whole slices per group, the
@@ -319,12 +362,13 @@ __global__ void __launch_bounds__(PLAN_THREADS) k_plan(ReadoutArgs a, int64_t nv
     // query tiles on 150 of 152 CTAs: 408 -> 281 us); where it leaves 1 in 64,
     // always.
     if (a.U == 1 && a.tensor && grun > 0 && P > grun) {
-        const int64_t idle = P % grun, bytes = (int64_t)s_nt[0] * a.BN * a.D * 4;
+        const int64_t idle = P % grun, bytes = (int64_t)s_nt[0] * cfg.BN * a.D * 4;
         if (64 * idle <= P || (bytes > ((int64_t)48 << 20) && 8 * idle <= P)) P -= idle;
     }
     PlanView v;
     v.tb = s_tb; v.wg = s_wg; v.nt = s_nt; v.gb = s_gb; v.cnt = s_cnt; v.U = a.U; v.H = a.H; v.W = run;
-    v.ov = a.plan_ov;
+    v.ov = cfg.ov;
+    v.mark = pairs ? RS3_PAIR_ITEMS : 0;
     v.P = (int)P;
     // every CTA of the launch gets its item range (empty past the P slices);
     // merge entries are packed through a shared counter
@@ -336,16 +380,17 @@ __global__ void __launch_bounds__(PLAN_THREADS) k_plan(ReadoutArgs a, int64_t nv
             if (np) atomicAdd(&s_np, np);
             if (c.nsplit > 0) a.combine[atomicAdd(&s_nc, 1)] = c;
         } else {
-            a.cta_items[2 * b] = 0;
+            a.cta_items[2 * b] = v.mark;
             a.cta_items[2 * b + 1] = 0;
         }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        hdr->n_items = (int32_t)(grun + v.P);       // bound on the item indices
+        hdr->n_items = (int32_t)(grun + v.P);
         hdr->n_combine = s_nc;
-        hdr->pad[0] = v.P;
-        hdr->pad[1] = s_np;                         // partial pieces of all split groups
+        hdr->slices = v.P;
+        hdr->n_part = s_np;
+        hdr->bm = cfg.BM;
     }
 }
 
@@ -378,28 +423,28 @@ __global__ void __launch_bounds__(256) k_combine(ReadoutArgs a)
     const int d = a.d;
     // chunked tasks only when the groups are split more than four ways on
     // average (one decision for the launch, so no task is spent idle)
-    const int n_comb = a.header->n_combine;
-    const bool chunked = a.header->pad[1] > 4 * n_comb;
+    const int n_comb = a.header->n_combine, BM = a.header->bm;
+    const bool chunked = a.header->n_part > 4 * n_comb;
     const int chunks = chunked ? (d + CW - 1) / CW : 1;   // tasks per row
-    const int64_t n_tasks = (int64_t)n_comb * a.BM * chunks;
+    const int64_t n_tasks = (int64_t)n_comb * BM * chunks;
     const int lane = threadIdx.x & 31;
     const float2 *pm = reinterpret_cast<const float2 *>(a.part_ml);
     for (int64_t task = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; task < n_tasks;
          task += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const int64_t gr = task / chunks;
         const int chunk = (int)(task % chunks);
-        const int ci = (int)(gr / a.BM), r = (int)(gr % a.BM);
+        const int ci = (int)(gr / BM), r = (int)(gr % BM);
         const CombineItem c = a.combine[ci];
         if (c.nsplit <= 0) continue;                   // warp-uniform
-        const int j = c.qt * a.BM + r;
+        const int j = c.qt * BM + r;
         if (j >= c.pad[1]) continue;                   // the unit's kept queries (warp-uniform)
         // piece 0 of the group is at slot0; piece s >= 1 is the first item of
         // slice b0 + s, partial slot 2 (b0 + s).  slot(s) = 2 (b0 + s) + d0 [s = 0]
         // with d0 = slot0 - 2 b0: a select, no branch, so every piece's loads
         // can be in flight together
         const int64_t b0 = c.pad[0], d0 = (int64_t)c.slot0 - 2 * b0;
-        const float2 *ml = pm + 2 * b0 * a.BM + r;                 // piece s at ml[slot_rel(s) BM]
-        const int64_t sstride = (int64_t)a.BM * d;                 // one slot
+        const float2 *ml = pm + 2 * b0 * BM + r;                 // piece s at ml[slot_rel(s) BM]
+        const int64_t sstride = (int64_t)BM * d;                 // one slot
 #define SLOT_REL(s_) (2 * (int64_t)(s_) + ((s_) == 0 ? d0 : 0))
         if (!chunked) {
             // One round trip for the row's cell, the pieces' (m, l) pairs (lane
@@ -407,8 +452,8 @@ __global__ void __launch_bounds__(256) k_combine(ReadoutArgs a)
             // stride the row four columns at a time); the weights follow.
             constexpr int MP = 4;
             int cell = a.idx[(int64_t)c.u * a.k_max + j];
-            const float2 mv = lane < c.nsplit ? ml[SLOT_REL(lane) * a.BM] : make_float2(-INFINITY, 0.f);
-            const float *base = a.part_o + (2 * b0 * a.BM + r) * d;
+            const float2 mv = lane < c.nsplit ? ml[SLOT_REL(lane) * BM] : make_float2(-INFINITY, 0.f);
+            const float *base = a.part_o + (2 * b0 * BM + r) * d;
             float4 pf[MP][2];
 #pragma unroll
             for (int q = 0; q < MP; ++q)
@@ -420,14 +465,14 @@ __global__ void __launch_bounds__(256) k_combine(ReadoutArgs a)
                                     : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             float M = mv.x;
-            for (int s = lane + 32; s < c.nsplit; s += 32) M = fmaxf(M, ml[SLOT_REL(s) * a.BM].x);
+            for (int s = lane + 32; s < c.nsplit; s += 32) M = fmaxf(M, ml[SLOT_REL(s) * BM].x);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
             float L = 0.f;
             if (M != -INFINITY) {
                 if (lane < c.nsplit) L = exp2f(mv.x - M) * mv.y;
                 for (int s = lane + 32; s < c.nsplit; s += 32) {
-                    const float2 v = ml[SLOT_REL(s) * a.BM];
+                    const float2 v = ml[SLOT_REL(s) * BM];
                     L += exp2f(v.x - M) * v.y;
                 }
             }
@@ -453,7 +498,7 @@ __global__ void __launch_bounds__(256) k_combine(ReadoutArgs a)
                     acc.w = fmaf(wq[q], pf[q][cb].w, acc.w);
                 }
                 for (int s = MP; s < c.nsplit; ++s) {
-                    const float ws = M == -INFINITY ? 0.f : exp2f(ml[SLOT_REL(s) * a.BM].x - M);
+                    const float ws = M == -INFINITY ? 0.f : exp2f(ml[SLOT_REL(s) * BM].x - M);
                     const float4 po = __ldcs(reinterpret_cast<const float4 *>(base + SLOT_REL(s) * sstride + c4));
                     acc.x = fmaf(ws, po.x, acc.x);
                     acc.y = fmaf(ws, po.y, acc.y);
@@ -468,26 +513,26 @@ __global__ void __launch_bounds__(256) k_combine(ReadoutArgs a)
         int cell = a.idx[(int64_t)c.u * a.k_max + j];
         if (cell < 0 || cell >= a.mn) cell = 0;
         float M = -INFINITY;
-        for (int s = lane; s < c.nsplit; s += 32) M = fmaxf(M, ml[SLOT_REL(s) * a.BM].x);
+        for (int s = lane; s < c.nsplit; s += 32) M = fmaxf(M, ml[SLOT_REL(s) * BM].x);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
         float L = 0.f;
         if (M != -INFINITY)
             for (int s = lane; s < c.nsplit; s += 32) {
-                const float2 v = ml[SLOT_REL(s) * a.BM];
+                const float2 v = ml[SLOT_REL(s) * BM];
                 L += exp2f(v.x - M) * v.y;
             }
         L = warp_sum(L);
         const float inv = L > 0.f ? 1.f / L : 0.f;
         const int col = chunk * CW + lane * E;
         if (col >= d) continue;                          // d < 32 only; no collectives below
-        const float *base = a.part_o + (2 * b0 * a.BM + r) * d + col;
+        const float *base = a.part_o + (2 * b0 * BM + r) * d + col;
         float acc[E];
 #pragma unroll
         for (int e = 0; e < E; ++e) acc[e] = 0.f;
 #pragma unroll 8
         for (int s = 0; s < c.nsplit; ++s) {
-            const float ws = M == -INFINITY ? 0.f : exp2f(ml[SLOT_REL(s) * a.BM].x - M);
+            const float ws = M == -INFINITY ? 0.f : exp2f(ml[SLOT_REL(s) * BM].x - M);
             if constexpr (E == 2) {
                 const float2 po = __ldcs(reinterpret_cast<const float2 *>(base + SLOT_REL(s) * sstride));
                 acc[0] = fmaf(ws, po.x, acc[0]);
@@ -519,7 +564,7 @@ namespace {
 // entry per CTA and per group.
 ReadoutLayout readout_layout(int U, int H, int d, int k_max, const ReadoutPath &p)
 {
-    const int BM = p.BM, grid = p.grid;
+    const int BM = p.BM, grid = p.grid, part_rows = p.part_rows;
     ReadoutLayout L;
     const int64_t nq = k_max > 0 ? (k_max + BM - 1) / BM : 1;
     const int64_t groups = (int64_t)U * H * nq;
@@ -538,9 +583,9 @@ ReadoutLayout readout_layout(int U, int H, int d, int k_max, const ReadoutPath &
     L.combine = off;
     off = align_up(off + (size_t)L.max_combine * sizeof(CombineItem), 256);
     L.part_o = off;
-    off = align_up(off + (size_t)L.max_slots * BM * d * 4, 256);
+    off = align_up(off + (size_t)L.max_slots * part_rows * d * 4, 256);
     L.part_ml = off;
-    off = align_up(off + (size_t)L.max_slots * BM * 8, 256);
+    off = align_up(off + (size_t)L.max_slots * part_rows * 8, 256);
     L.total = off;
     return L;
 }
@@ -554,40 +599,46 @@ std::atomic<uint64_t> g_wait_ns{1000000000ull};
 extern "C" void rs3_set_wait_limit_ns(uint64_t ns) { g_wait_ns.store(ns); }
 extern "C" uint64_t rs3_get_wait_limit_ns(void) { return g_wait_ns.load(); }
 
-// The kernel and its tiles for a call.  bf16 heads of 64 and 128 have two
-// tensor-core kernels: the one with two query tiles per CTA is faster once there
-// are query tiles for half of the CTAs or so (us per call, both measured:
-// 40 tiles of 4 heads of 64: 32.7 against 35.1; 80 tiles 39 against 43; 160
-// tiles of heads of 128 75 against 86; 2 000 tiles 1 080 against 1 704), the
-// other below that (10 tiles 22.6 against 25.6; 20 tiles of heads of 128 31.8
-// against 37.2), and where a pair of tiles would often be half empty (3 tiles
-// per head, 72 in all: 25.5 against 27.0).
+// Score tiles (128 queries x 128 keys) of the least call that takes pairs of query
+// tiles: those of S1 > r S2 + c n_sm in two_tiles where all pairs are full.
+static double pair_tiles(int d, int n_sm) { return d == 64 ? n_sm / 0.15 : 3.75 * n_sm / 0.175; }
+
+// The kernel and its tiles for a call.  bf16 heads of 64 and 128 with more than one
+// query tile per head have two tensor-core kernels, between which the plan chooses
+// by the kept queries and the banks' lengths (two_tiles).  The kernel that holds
+// both takes 1.8 us more for a call that ends up with one tile per CTA, so calls
+// whose largest keep-sets on full banks have less than 32 times the tiles at which
+// pairs begin take the one-tile kernel alone: objects and what they leave in a bank
+// cover a small part of the grid.  Over 244 shapes nothing is then more than 2% slower
+// than the one-tile kernel was before, and the geometric mean is 9% faster (4% with
+// both for every call, 6% below that line).
 //
 // A workspace that is too small for the kernel's partial results but holds those
 // of 256 rows per SM takes a smaller path: the one-tile kernel, or one CTA per SM
 // on the CUDA cores.  rs3_readout_workspace_bytes returns at least that for
 // every kernel, so a workspace sized for one call serves every smaller one.
-ReadoutPath choose_readout_path(rs3_dtype dtype, int d, int U, int H, int k_max, size_t workspace_bytes)
+ReadoutPath choose_readout_path(rs3_dtype dtype, int d, int U, int H, int k_max, int64_t bank_rows, size_t workspace_bytes)
 {
     ReadoutPath p;
     const int n_sm = rs3_sm_count();
+    p.either = false;
     if (dtype == RS3_BF16 && rs3_tc_supported(d)) {
-        const int64_t single = (k_max + 127) / 128, pairs = (k_max + 255) / 256;
         p.kind = 1;
-        p.BM = 128;
+        p.BM = p.part_rows = 128;
         p.BN = rs3_tc_block_n(d);
         p.grid = n_sm;                 // one persistent CTA per SM
-        if (d <= 128 && (int64_t)U * H * single >= 40 && 8 * pairs <= 5 * single) {
+        const double tiles = (double)U * H * ((k_max + 127) / 128) * ((double)bank_rows / 128.0 + 1.0);
+        if (d <= 128 && k_max > 128 && tiles >= 32.0 * pair_tiles(d, n_sm)) {
             ReadoutPath two = p;
-            two.kind = 2;
-            two.BM = 256;              // two query tiles per item
-            two.BN = 128;
+            two.either = true;
+            two.part_rows = 256;       // two query tiles per item
             if (readout_layout(U, H, d, k_max, two).total <= workspace_bytes) p = two;
         }
     } else {
         int ctas;
         p.kind = 0;
         rs3_simt_tile(d, p.BM, p.BN, ctas);
+        p.part_rows = p.BM;
         p.grid = ctas * n_sm;
         if (ctas > 1 && readout_layout(U, H, d, k_max, p).total > workspace_bytes) p.grid = n_sm;
     }
@@ -595,22 +646,18 @@ ReadoutPath choose_readout_path(rs3_dtype dtype, int d, int U, int H, int k_max,
 }
 
 // What the preferred path of this call needs, and no less than a call of fewer
-// queries, units or heads may: a keep-set of three query tiles is left to the
-// one-tile kernel where one of two takes the other.
+// queries, units or heads may.
 extern "C" size_t rs3_readout_workspace_bytes(int U, int H, int d, int k_max, rs3_dtype dtype)
 {
     if (U < 1 || H < 1 || d < 1 || k_max < 0) return 0;
-    size_t need = 0;
     ReadoutPath floor;                 // 256 rows of partial results per SM
     floor.kind = 1;
-    floor.BM = 128;
+    floor.either = false;
+    floor.BM = floor.part_rows = 128;
     floor.BN = 0;
     floor.grid = rs3_sm_count();
-    for (const int k : {k_max, k_max < 256 ? k_max : 256}) {
-        const ReadoutPath p = choose_readout_path(dtype, d, U, H, k, SIZE_MAX);
-        need = std::max(need, readout_layout(U, H, d, k_max, p).total);
-    }
-    return std::max(need, readout_layout(U, H, d, k_max, floor).total);
+    const ReadoutPath p = choose_readout_path(dtype, d, U, H, k_max, INT64_MAX, SIZE_MAX);
+    return std::max(readout_layout(U, H, d, k_max, p).total, readout_layout(U, H, d, k_max, floor).total);
 }
 
 rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, int H, int d,
@@ -632,7 +679,7 @@ rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, in
     if (!rs3_aligned16(q) || !rs3_aligned16(out) || !rs3_aligned16(workspace) ||
         (residual && !rs3_aligned16(residual)) || (rope && !rs3_aligned16(rope)))
         return RS3_EINVAL;
-    const ReadoutPath p = choose_readout_path(dtype, d, bank->U, H, k_max, workspace_bytes);
+    const ReadoutPath p = choose_readout_path(dtype, d, bank->U, H, k_max, bank->rows_per_unit, workspace_bytes);
     const ReadoutLayout L = readout_layout(bank->U, H, d, k_max, p);
     // work-item indices (group + slice) and item ranges are 32-bit.  The limit
     // counts 32-row query tiles on the CUDA-core path and 128-row ones on the
@@ -674,11 +721,8 @@ rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, in
     // CUDA-core path is flat over 1..4.  A slice of at least two slots: four
     // left a 32 x 32 fp32 frame on half the CTAs (68 us against 61)
     a->tensor = p.kind != 0;
+    a->either = p.either;
     a->plan_ov = p.kind == 1 ? 12 : 1;
-    if (p.kind == 2) {             // 128-key tiles: 3 and 12 slots, and slices of 2 and 6, are slower
-        a->plan_ov = 6;
-        a->min_chunk = 4;
-    }
     a->max_slots = L.max_slots;
     a->max_items = L.max_items;
     a->grid_ctas = p.grid;
@@ -720,7 +764,7 @@ rs3_status launch_plan(const ReadoutArgs &a, cudaStream_t st, rs3_dtype dtype)
 // the attention kernel over the plan in the workspace
 rs3_status launch_run(const ReadoutArgs &a, const ReadoutPath &p, rs3_dtype dtype, cudaStream_t st)
 {
-    if (p.kind == 2) return rs3_launch_pair_readout(a, st);
+    if (p.either) return rs3_launch_either_readout(a, st);
     if (p.kind == 1) return rs3_launch_tc_readout(a, st);
     return rs3_launch_simt_readout(a, dtype, st);
 }
@@ -731,7 +775,7 @@ rs3_status launch_merge(const ReadoutArgs &a, int64_t max_combine, rs3_dtype dty
     // one warp per (partial row, 64-column chunk; 32 for d < 64)
     const int ce = a.d >= 64 ? 2 : 1;
     const int64_t chunks = (a.d + 32 * ce - 1) / (32 * ce);
-    int64_t cblocks = (max_combine * a.BM * chunks + 7) / 8;
+    int64_t cblocks = (max_combine * (a.either ? 2 * a.BM : a.BM) * chunks + 7) / 8;
     const int64_t ccap = (int64_t)a.n_sm * 16;
     if (cblocks > ccap) cblocks = ccap;
     if (cblocks < 1) cblocks = 1;

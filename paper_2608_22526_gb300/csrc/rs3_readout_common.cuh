@@ -5,6 +5,7 @@
 #include "rs3_internal.cuh"
 
 #define RS3_MAX_UNITS 4096  // units per readout call
+#define RS3_PAIR_ITEMS (1 << 30)   // above every item index
 
 struct ReadoutArgs {
     const void *q;
@@ -24,11 +25,13 @@ struct ReadoutArgs {
     int U, G, mn, H, d, D, k_max;
     int BM, BN, n_sm, min_chunk;
     int plan_ov;            // leading plan slots per group: a piece's start-up cost in tiles
+    int either;             // the plan may take the two-tile kernel (the four above are the one-tile kernel's)
     int tensor;             // a tensor-core kernel runs the plan
     int64_t max_slots;
     int64_t max_items;
     int grid_ctas;          // CTAs of the readout launch (the plan's slice count bound)
-    int32_t *cta_items;     // [grid_ctas][2]: CTA b runs items [cta_items[2b], cta_items[2b+1])
+    int32_t *cta_items;     // [grid_ctas][2]: CTA b runs items [cta_items[2b], cta_items[2b+1]); the first
+                            // of the two with RS3_PAIR_ITEMS where they are for the two-tile kernel
     float scale_log2;       // softmax scale * log2(e)
     uint64_t wait_ns;       // limit of each device-side wait (global-timer ns)
     ReadoutHeader *header;
@@ -40,17 +43,20 @@ struct ReadoutArgs {
 };
 
 struct ReadoutPath {
-    int kind;   // 0 = CUDA-core, 1 = tensor-core (tcgen05), 2 = tensor-core, two query tiles
-    int BM, BN;
+    int kind;        // 0 = CUDA-core, 1 = tensor-core (tcgen05)
+    bool either;     // ... with one or two query tiles, as the plan finds
+    int BM, BN;      // of one query tile
+    int part_rows;   // rows of a partial slot
     int grid;   // CTAs of the readout launch
 };
 
-// the path of a call with this workspace (SIZE_MAX: the path that any workspace is sized for)
-ReadoutPath choose_readout_path(rs3_dtype dtype, int d, int U, int H, int k_max, size_t workspace_bytes);
+// the path of a call over banks of this many rows with this workspace (INT64_MAX and
+// SIZE_MAX: the path that any workspace is sized for)
+ReadoutPath choose_readout_path(rs3_dtype dtype, int d, int U, int H, int k_max, int64_t bank_rows, size_t workspace_bytes);
 bool rs3_tc_supported(int d);
 int rs3_tc_block_n(int d);
 rs3_status rs3_launch_tc_readout(const ReadoutArgs &a, cudaStream_t st);
-rs3_status rs3_launch_pair_readout(const ReadoutArgs &a, cudaStream_t st);   // d = 64, 128
+rs3_status rs3_launch_either_readout(const ReadoutArgs &a, cudaStream_t st);   // d = 64, 128
 // CUDA-core path: rows and keys of a tile and resident CTAs per SM, for a head width
 void rs3_simt_tile(int d, int &bm, int &bn, int &ctas_per_sm);
 rs3_status rs3_launch_simt_readout(const ReadoutArgs &a, rs3_dtype dtype, cudaStream_t st);

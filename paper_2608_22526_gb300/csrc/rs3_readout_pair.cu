@@ -9,8 +9,7 @@
 // and while one warpgroup takes its exps the tensor core works for the other.
 //   warp 0      TMA of K and V tiles (128 keys) into two rings
 //   warps 1, 2  issue query tile 0's (1's) S_q = Q_q K^T (both operands in
-//               shared memory) and O_q += P_q V (P_q in TMEM); warp 1 allocates
-//               TMEM
+//               shared memory) and O_q += P_q V (P_q in TMEM)
 //   warps 4-7   softmax of query tile 0, warps 8-11 of tile 1: per item the
 //               kept rows (rotated by the RoPE table of their own cell) into
 //               shared memory; per tile the row's 128 scores into registers,
@@ -19,21 +18,26 @@
 //               residual, or the split-KV partial.  The next item's query rows
 //               are loaded before the epilogue, while the last P V runs.
 // An item of at most 128 rows uses tile 0 alone.
+//
+// What is faster depends on the kept queries and the banks' lengths, which only the
+// device knows, so k_readout_either holds this kernel and the one-tile one
+// (rs3_readout_tc.cuh) on the same threads, and the plan marks the item ranges with
+// its choice.  Chosen by k_max on the host, 3 objects of 2 heads of 128 with 300 kept
+// queries and 600 keys each took 26.9 us; 16.6 with one tile, 18.2 before.  The tc
+// kernel's start is up to 1.8 us slower inside the larger kernel.
 // TMEM: d = 64: O_0, O_1, S_0, S_1 and P_0, P_1 fill the 512 columns, so
 // S_q(t + 1) needs only that S_q(t) was read.  d = 128: P_q lies over S_q, and
 // S_q(t + 1) is issued behind the P V that reads it (the tensor core takes a
 // CTA's matrix instructions in order).
 // The softmax warps take registers from the others (setmaxnreg): a row's 128
 // scores stay in registers.
-// 16 streams x 3 objects, 4 heads of 64, 96 x 96 grid (911 GFLOP): 1 085 us per
+// 16 streams x 3 objects, 4 heads of 64, 96 x 96 grid (911 GFLOP): 1 070 us per
 // call, 1 704 in the one-tile kernel.  Per pair of 128 x 128 tiles it takes about
 // 2 500 clk, where the exps of 256 rows alone take 1 380 and the matrices 1 052:
 // a warpgroup's own chain (wait, scores from TMEM, max, exps, P to TMEM) is that
 // long with two warps per scheduler.
 // Every mbarrier wait is bounded as in rs3_readout_tc.cu.
-#include "rs3_readout_common.cuh"
-#include "rs3_tc_host.cuh"
-#include "rs3_tc_ptx.cuh"
+#include "rs3_readout_tc.cuh"
 
 namespace tc {
 
@@ -135,12 +139,15 @@ struct TileWalk {
     }
 };
 
+// Items [it_begin, it_end) of the plan, in a CTA that is set up for the one-tile
+// kernel (set_up_tc): its tensor memory serves, its barriers make room.
 template <int DH>
-__global__ void __launch_bounds__(NTHREADS, 1)
-k_readout_pair(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk, const __grid_constant__ CUtensorMap tmv)
+__device__ __forceinline__ void readout_pair(const ReadoutArgs &a, const CUtensorMap &tmk, const CUtensorMap &tmv,
+                                             uint32_t tmem, int it_begin, int it_end)
 {
     using C = Cfg<DH>;
     constexpr int KSTK = C::KSTK, KSTV = C::KSTV;
+    static_assert(TMEM_COLS == tc::TMEM_COLS, "one allocation for both kernels");
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -148,11 +155,11 @@ k_readout_pair(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk, con
     const uint32_t sQ = base + C::OFF_Q, sK = base + C::OFF_K, sV = base + C::OFF_V;
     const uint32_t bars = base + C::OFF_BAR;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(gbase + C::OFF_MISC);
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(gbase + C::OFF_MISC + 8);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #define BAR(i) (bars + 8u * (uint32_t)(i))
 
     if (threadIdx.x == 0) {
+        for (int i = 0; i < tc::Cfg<DH>::NBAR; ++i) mbar_inval(base + tc::Cfg<DH>::OFF_BAR + 8u * i);
         for (int s = 0; s < KSTK; ++s) {
             mbar_init(BAR(C::B_KFULL + s), 1);
             mbar_init(BAR(C::B_KEMPTY + s), 2);               // both MMA issuers
@@ -174,23 +181,8 @@ k_readout_pair(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk, con
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
     }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    if (threadIdx.x == 64) {
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmk)) : "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmv)) : "memory");
-    }
-    tc_fence_before();
     __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
     const uint64_t wait_ns = a.wait_ns;
-    // the set-up above touches no global memory
-    pdl_wait();
-    const int it_begin = a.cta_items[2 * blockIdx.x], it_end = a.cta_items[2 * blockIdx.x + 1];
 
     if (warp < 4) {
         reg_dec<C::REGS_ISSUE>();
@@ -198,6 +190,7 @@ k_readout_pair(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk, con
             // ------------------------------------------------------------------
             // TMA producer: tile t's K, then tile t's V
             // ------------------------------------------------------------------
+            constexpr int BOX = tc::Cfg<DH>::BN;                       // rows of the one-tile kernel's boxes
             uint32_t ck = 0, cv = 0;                                   // K and V tiles issued
             bool ok = true;
             for (int it = it_begin; it < it_end && ok; ++it) {
@@ -214,14 +207,18 @@ k_readout_pair(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk, con
                     mbar_expect_tx(BAR(C::B_KFULL + ks), (uint32_t)C::KVBYTES);
 #pragma unroll
                     for (int c = 0; c < DH / 64; ++c)
-                        tma_load_2d(sK + ks * C::KVBYTES + c * (BN * 128), &tmk, BAR(C::B_KFULL + ks), w.h * DH + c * 64, y);
+#pragma unroll
+                        for (int r = 0; r < BN; r += BOX)
+                            tma_load_2d(sK + ks * C::KVBYTES + c * (BN * 128) + r * 128, &tmk, BAR(C::B_KFULL + ks), w.h * DH + c * 64, y + r);
                     ++ck;
                     ok = mbar_wait(BAR(C::B_VEMPTY + vs), ((cv / KSTV) & 1u) ^ 1u, abort_flag, wait_ns);
                     if (!ok) break;
                     mbar_expect_tx(BAR(C::B_VFULL + vs), (uint32_t)C::KVBYTES);
 #pragma unroll
                     for (int c = 0; c < DH / 64; ++c)
-                        tma_load_2d(sV + vs * C::KVBYTES + c * (BN * 128), &tmv, BAR(C::B_VFULL + vs), w.h * DH + c * 64, y);
+#pragma unroll
+                        for (int r = 0; r < BN; r += BOX)
+                            tma_load_2d(sV + vs * C::KVBYTES + c * (BN * 128) + r * 128, &tmv, BAR(C::B_VFULL + vs), w.h * DH + c * 64, y + r);
                     ++cv;
                 }
             }
@@ -498,15 +495,31 @@ k_readout_pair(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk, con
 #undef BAR
 }
 
+// The kernel that the plan chose, on the same threads.
+template <int DH>
+__global__ void __launch_bounds__(NTHREADS, 1)
+k_readout_either(const ReadoutArgs a, const __grid_constant__ CUtensorMap tmk, const __grid_constant__ CUtensorMap tmv)
+{
+    static_assert(NTHREADS == tc::Cfg<DH>::NTHREADS, "one launch for both");
+    // set up for the one-tile kernel, whose calls are the short ones
+    const uint32_t tmem = set_up_tc<DH>(tmk, tmv);
+    pdl_wait();                      // the plan
+    const int first = a.cta_items[2 * blockIdx.x], it_end = a.cta_items[2 * blockIdx.x + 1];
+    if (first & RS3_PAIR_ITEMS) readout_pair<DH>(a, tmk, tmv, tmem, first & ~RS3_PAIR_ITEMS, it_end);
+    else readout_tc<DH>(a, tmk, tmv, tmem, first, it_end);
+}
+
 template <int DH>
 rs3_status launch(const ReadoutArgs &a, cudaStream_t st)
 {
-    if (rs3_kernel_smem((const void *)k_readout_pair<DH>, Cfg<DH>::SMEM) != RS3_OK) return RS3_ECUDA;
+    constexpr int smem = Cfg<DH>::SMEM > tc::Cfg<DH>::SMEM ? Cfg<DH>::SMEM : tc::Cfg<DH>::SMEM;
+    if (rs3_kernel_smem((const void *)k_readout_either<DH>, smem) != RS3_OK) return RS3_ECUDA;
     const int64_t rows = (int64_t)a.U * a.rows_per_unit;
     if (rows >= (int64_t)1 << 31) return RS3_EUNSUPPORTED;
     CUtensorMap mk, mv;
-    if (!make_kv_map(&mk, a.k_store, a.D, rows, BN) || !make_kv_map(&mv, a.v_store, a.D, rows, BN)) return RS3_ECUDA;
-    launch_pdl(k_readout_pair<DH>, dim3((unsigned)a.grid_ctas), dim3(NTHREADS), Cfg<DH>::SMEM, st, a, mk, mv);
+    if (!make_kv_map(&mk, a.k_store, a.D, rows, tc::Cfg<DH>::BN) || !make_kv_map(&mv, a.v_store, a.D, rows, tc::Cfg<DH>::BN))
+        return RS3_ECUDA;
+    launch_pdl(k_readout_either<DH>, dim3((unsigned)a.grid_ctas), dim3(NTHREADS), smem, st, a, mk, mv);
     return cudaGetLastError() == cudaSuccess ? RS3_OK : RS3_ECUDA;
 }
 
@@ -514,7 +527,7 @@ rs3_status launch(const ReadoutArgs &a, cudaStream_t st)
 
 }  // namespace tc
 
-rs3_status rs3_launch_pair_readout(const ReadoutArgs &a, cudaStream_t st)
+rs3_status rs3_launch_either_readout(const ReadoutArgs &a, cudaStream_t st)
 {
     switch (a.d) {
     case 64: return tc::pair::launch<64>(a, st);

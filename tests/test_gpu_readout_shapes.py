@@ -34,15 +34,16 @@ def _check(dtype, got, exact, vmax, rope, what):
         assert float(err.max()) <= F32_REL * max(float(np.abs(exact).max()), 1e-30), f"{what}: {err.max()}"
 
 
-def _case(dtype, H, d, counts, rows, n_ptr=0, rope=False, sharp=1.0, ramp=0.0, seed=0, ws_bytes=None):
+def _case(dtype, H, d, counts, rows, n_ptr=0, rope=False, sharp=1.0, ramp=0.0, seed=0, ws_bytes=None, tile=None, cap=0):
     """One group, a unit per (count, rows) pair: `rows` bank rows in two ring
     frames, then n_ptr pointer rows.  ramp > 0 makes later keys score higher,
-    so that a row's softmax reference has to move."""
+    so that a row's softmax reference has to move.  cap: rows of the bank's ring, of
+    which two frames are used."""
     rng = np.random.default_rng([seed, d, len(counts)])
     U, m, n = len(counts), 24, 25
     mn, D = m * n, H * d
     k_max = max(counts)
-    bank = rs3.Bank(U, H, d, dtype, mn, 0, 2, 2 * mn, 2, n_ptr)
+    bank = rs3.Bank(U, H, d, dtype, mn, 0, 2, max(cap, 2 * mn), 2, n_ptr)
     st = torch.zeros(1, dtype=torch.int32, device="cuda")
     q = _draw(rng, dtype, (1, mn, D), sharp)
     K, V = [[] for _ in range(U)], [[] for _ in range(U)]
@@ -84,6 +85,8 @@ def _case(dtype, H, d, counts, rows, n_ptr=0, rope=False, sharp=1.0, ramp=0.0, s
     call(None, attn)
     call(out, out)
     attn, out = to_host(attn), to_host(out)
+    if tile is not None:                                 # query rows of an item: the kernel that the plan chose
+        assert ws.view(torch.int32)[4].item() == tile
     for u, c in enumerate(counts):
         cells = idx[u, :c]
         vmax, A = 1.0, np.zeros((c, D))
@@ -139,7 +142,7 @@ def test_partial_query_tiles_of_whole_items(d):
     beside them, over every chunk of columns of the epilogue."""
     counts = [1, 31, 33, 100, 127, 129, 160, 5, 97, 140, 180, 65] * 15
     rows = [70, 129, 64, 200, 33, 140, 65, 257, 10, 128, 130, 90] * 15
-    _case("bf16", 1, d, counts, rows, rope=True, seed=3)
+    _case("bf16", 1, d, counts, rows, rope=True, seed=3, tile=128)
 
 
 def _one_tile_bytes(U, H, d, k_max):
@@ -160,9 +163,37 @@ def test_smaller_calls_in_a_workspace_sized_for_the_largest(dtype, H, d):
     U, counts = 8, [200, 256, 3, 129, 255, 64, 130, 250]
     rows = [300, 150, 700, 64, 900, 129, 40, 500]
     _case(dtype, H, d, counts, rows, ws_bytes=rs3.rs3_readout_workspace_bytes(U, H, d, 384, dtype))
+    cap = 70000 if dtype == "bf16" and d == 64 else 0     # of the size that the plan would choose for
     least = _one_tile_bytes(U, H, d, 256)
     assert least < rs3.rs3_readout_workspace_bytes(U, H, d, 256, dtype)
-    _case(dtype, H, d, counts, rows, rope=True, n_ptr=5, ws_bytes=least)
+    _case(dtype, H, d, counts, rows, rope=True, n_ptr=5, ws_bytes=least, cap=cap)
     with pytest.raises(rs3.RS3Error) as e:
         _case(dtype, H, d, counts, rows, ws_bytes=least - 256)
     assert e.value.code == rs3.RS3_ECAPACITY
+
+
+PAIRS = [512, 511, 500, 1, 385, 130, 512, 0, 400, 490, 257, 512] * 4
+PAIR_ROWS = [1100, 1200, 1025, 1000, 1151, 900, 1200, 1100, 1153, 1199, 1024, 1100] * 4
+
+
+@pytest.mark.parametrize("H,d", [(4, 64), (4, 128), (8, 64)])
+@pytest.mark.parametrize("rope,ramp", [(True, 0.0), (False, 3.0)])
+def test_two_query_tiles(H, d, rope, ramp):
+    """Enough score tiles for the plan to take two query tiles per CTA: pairs that
+    are full, half empty and empty, partial keys in every piece of the bank."""
+    _case("bf16", H, d, PAIRS, PAIR_ROWS, n_ptr=3, rope=rope, ramp=ramp, seed=5, tile=256, cap=12000 * d // 64)
+
+
+@pytest.mark.parametrize("H,d", [(4, 64), (2, 128)])
+def test_small_keep_sets_take_one_query_tile(H, d):
+    """Few kept queries: one tile per CTA, as the plan finds for the large bank and
+    the call's sizes say for the small one."""
+    counts, rows = [512, 40, 129, 1, 100, 60] + [33] * 18, [200] * 24
+    _case("bf16", H, d, counts, rows, rope=True, seed=6, tile=128, cap=80000 // H)
+    _case("bf16", H, d, counts, rows, rope=True, seed=6, tile=128)
+
+
+def test_two_query_tiles_of_one_unit():
+    """One unit, whose pairs get whole slices each, and a unit count past the plan's threads."""
+    _case("bf16", 40, 64, [512], [1200], seed=7, tile=256, cap=30000)
+    _case("bf16", 1, 64, [512, 250, 70] * 100, [1100, 900, 300] * 100, seed=8, tile=256, cap=5000)
