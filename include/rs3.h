@@ -311,11 +311,11 @@ size_t rs3_readout_workspace_bytes(int U, int H, int d, int k_max, rs3_dtype dty
  *   out       device [U][mn][H*d]
  *   scale     softmax scale; 0 selects 1/sqrt(d) (Eq. 6's 1/sqrt(C_k) per head)
  *   workspace device, >= rs3_readout_workspace_bytes(...), 16-byte aligned
- * bf16: tensor-core path for d in {64, 128, 256}, fp32 accumulation.  fp32:
- * CUDA-core FFMA path for d % 16 == 0, d <= 256.
- * Limits: U <= 4096, mn <= 16384; the work list holds fewer than 2^21
- * entries (U * H * ceil(k_max / BM) plus one per SM, BM = 128 on the bf16
- * path and 32 on the fp32 path), else RS3_EUNSUPPORTED.
+ * bf16: tensor-core path for d in {64, 128, 256}, fp32 accumulation; fp32, and
+ * bf16 with d in {16, 32}: CUDA-core FFMA path, d a power of two in [16, 256].
+ * Limits: U <= 4096, mn <= 16384; the work list holds fewer than 2^30
+ * entries (U * H * ceil(k_max / BM) plus one per CTA, counted with BM = 128 on the
+ * tensor cores and 32 on the CUDA cores), else RS3_EUNSUPPORTED.
  */
 rs3_status rs3_memory_readout(const void *q, rs3_dtype dtype, int G, int mn, int H, int d,
                               const int32_t *unit_group, const int32_t *idx,

@@ -38,6 +38,7 @@
 // argmax and its labels; 91 us with a scalar load and a ballot per 32 pixels,
 // general funnel-shift dilations and an 8-row halo per 16 rows on CTAs that
 // filled 1.3 waves.  8 objects of 1024 x 1024: 79 -> 44 us.
+#include "rs3_cluster.cuh"
 #include "rs3_internal.cuh"
 
 #include <algorithm>
@@ -137,56 +138,6 @@ __device__ __forceinline__ void store_bits(uint4 *dst, float4 v, int lane)
     const uint32_t b0 = __ballot_sync(0xffffffffu, v.x > 0.f), b1 = __ballot_sync(0xffffffffu, v.y > 0.f);
     const uint32_t b2 = __ballot_sync(0xffffffffu, v.z > 0.f), b3 = __ballot_sync(0xffffffffu, v.w > 0.f);
     if (lane == 0) *dst = make_uint4(b0, b1, b2, b3);
-}
-
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-// every thread of every CTA of the cluster arrives, then waits (the release /
-// acquire pair orders shared-memory writes before the barrier with reads of
-// them through DSMEM after it).  .aligned: a warp's lanes execute it together,
-// also after a loop or a branch that some of them left early
-__device__ __forceinline__ void cluster_arrive()
-{
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait()
-{
-    __syncwarp();
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_barrier()
-{
-    cluster_arrive();
-    cluster_wait();
-}
-
-__device__ __forceinline__ uint32_t dsmem_addr(const void *p, uint32_t rank)
-{
-    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    return r;
-}
-
-__device__ __forceinline__ float4 dsmem_ld_f32x4(uint32_t a)
-{
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ uint32_t dsmem_ld_u32(uint32_t a)
-{
-    uint32_t v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
-    return v;
 }
 
 // Shared memory of a CTA, in 16-byte words: bits of window rows x (NS + 2)

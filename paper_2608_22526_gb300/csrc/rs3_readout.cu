@@ -357,10 +357,11 @@ __global__ void __launch_bounds__(PLAN_THREADS) k_plan(ReadoutArgs a, int64_t nv
     // One unit: its groups are equally long.  With whole slices per group, the
     // slices of all its query tiles and heads reach a key at the same time; cut
     // anywhere, they reach it at as many times as the remainder has parts, and a
-    // bank that L2 does not hold is read from DRAM that often.  Worth leaving
-    // CTAs idle for large banks on the tensor cores (300 000 keys of 256, ten
-    // query tiles on 150 of 152 CTAs: 408 -> 281 us); where it leaves 1 in 64,
-    // always.
+    // bank that L2 does not hold is read from DRAM that often.  Worth leaving one
+    // CTA in eight idle for large banks on the tensor cores (300 000 keys of 256, ten
+    // query tiles on 150 of 152 CTAs: 392 -> 285 us); where it leaves 1 in 64,
+    // always.  The line at 48 MB of K and V is a constant fitted on this part, whose L2
+    // holds 126 MB; nothing derives it.
     if (a.U == 1 && a.tensor && grun > 0 && P > grun) {
         const int64_t idle = P % grun, bytes = (int64_t)s_nt[0] * cfg.BN * a.D * 4;
         if (64 * idle <= P || (bytes > ((int64_t)48 << 20) && 8 * idle <= P)) P -= idle;
@@ -665,7 +666,7 @@ rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, in
                                int k_max, const rs3_bank *bank, const float *rope,
                                const void *residual, void *out, float scale, void *workspace,
                                size_t workspace_bytes, int32_t *status, ReadoutArgs *a,
-                               ReadoutPath *path, int64_t *grid_items, int64_t *grid_combine)
+                               ReadoutPath *path, int64_t *grid_combine)
 {
     if (!q || !unit_group || !idx || !count || !bank || !out || !workspace || !status)
         return RS3_EINVAL;
@@ -724,7 +725,6 @@ rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, in
     a->either = p.either;
     a->plan_ov = p.kind == 1 ? 12 : 1;
     a->max_slots = L.max_slots;
-    a->max_items = L.max_items;
     a->grid_ctas = p.grid;
     a->cta_items = reinterpret_cast<int32_t *>(ws + L.cta_items);
     const float sc = scale > 0.f ? scale : 1.0f / sqrtf((float)d);
@@ -737,7 +737,6 @@ rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, in
     a->part_o = reinterpret_cast<float *>(ws + L.part_o);
     a->part_ml = reinterpret_cast<float *>(ws + L.part_ml);
     *path = p;
-    *grid_items = L.max_items;
     *grid_combine = L.max_combine;
     return RS3_OK;
 }
@@ -791,10 +790,9 @@ rs3_status launch_merge(const ReadoutArgs &a, int64_t max_combine, rs3_dtype dty
 
 }  // namespace
 
-rs3_status rs3_readout_launch(const ReadoutArgs &a, const ReadoutPath &p, int64_t max_items,
+rs3_status rs3_readout_launch(const ReadoutArgs &a, const ReadoutPath &p,
                               int64_t max_combine, rs3_dtype dtype, cudaStream_t st, int phases)
 {
-    (void)max_items;
     if (phases & RS3_PHASE_PLAN) {
         const rs3_status s = launch_plan(a, st, dtype);
         if (s != RS3_OK) return s;
@@ -816,12 +814,12 @@ rs3_status readout_call(const void *q, rs3_dtype dtype, int G, int mn, int H, in
 {
     ReadoutArgs a;
     ReadoutPath p;
-    int64_t gi, gc;
+    int64_t gc;
     const rs3_status s = rs3_readout_prepare(q, dtype, G, mn, H, d, unit_group, idx, count, k_max,
                                              bank, rope, residual, out, scale, workspace,
-                                             workspace_bytes, status, &a, &p, &gi, &gc);
+                                             workspace_bytes, status, &a, &p, &gc);
     if (s != RS3_OK) return s;
-    return rs3_readout_launch(a, p, gi, gc, dtype, reinterpret_cast<cudaStream_t>(stream), phases);
+    return rs3_readout_launch(a, p, gc, dtype, reinterpret_cast<cudaStream_t>(stream), phases);
 }
 
 }  // namespace

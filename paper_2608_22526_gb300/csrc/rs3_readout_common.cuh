@@ -28,7 +28,6 @@ struct ReadoutArgs {
     int either;             // the plan may take the two-tile kernel (the four above are the one-tile kernel's)
     int tensor;             // a tensor-core kernel runs the plan
     int64_t max_slots;
-    int64_t max_items;
     int grid_ctas;          // CTAs of the readout launch (the plan's slice count bound)
     int32_t *cta_items;     // [grid_ctas][2]: CTA b runs items [cta_items[2b], cta_items[2b+1]); the first
                             // of the two with RS3_PAIR_ITEMS where they are for the two-tile kernel
@@ -65,11 +64,11 @@ rs3_status rs3_readout_prepare(const void *q, rs3_dtype dtype, int G, int mn, in
                                int k_max, const rs3_bank *bank, const float *rope,
                                const void *residual, void *out, float scale, void *workspace,
                                size_t workspace_bytes, int32_t *status, ReadoutArgs *a,
-                               ReadoutPath *path, int64_t *grid_items, int64_t *grid_combine);
+                               ReadoutPath *path, int64_t *grid_combine);
 // phases of a readout: the attention over the bank (pass-through, plan,
 // readout kernel) and the merge of split-KV partials
 enum { RS3_PHASE_PLAN = 1, RS3_PHASE_RUN = 4, RS3_PHASE_ATTEND = 1 | 4, RS3_PHASE_MERGE = 2 };
-rs3_status rs3_readout_launch(const ReadoutArgs &a, const ReadoutPath &p, int64_t max_items,
+rs3_status rs3_readout_launch(const ReadoutArgs &a, const ReadoutPath &p,
                               int64_t max_combine, rs3_dtype dtype, cudaStream_t st, int phases);
 
 // Tile t of a unit's bank (tiles of BN rows, never crossing a range end) ->

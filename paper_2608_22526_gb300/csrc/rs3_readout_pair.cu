@@ -36,7 +36,7 @@
 // 2 500 clk, where the exps of 256 rows alone take 1 380 and the matrices 1 052:
 // a warpgroup's own chain (wait, scores from TMEM, max, exps, P to TMEM) is that
 // long with two warps per scheduler.
-// Every mbarrier wait is bounded as in rs3_readout_tc.cu.
+// Every mbarrier wait is bounded as in rs3_readout_tc.cuh.
 #include "rs3_readout_tc.cuh"
 
 namespace tc {

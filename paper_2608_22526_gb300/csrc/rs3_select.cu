@@ -28,6 +28,7 @@
 // 14.0 us, and 16 streams x 3 objects of 96 x 96 20.9 us per call (7.3 us at the
 // copy rate); 20.3, 25.9 and 59 us as three launches that passed the priors and
 // the energies through global memory.
+#include "rs3_cluster.cuh"
 #include "rs3_internal.cuh"
 
 #include <algorithm>
@@ -162,42 +163,6 @@ struct WordWalk {
         }
     }
 };
-
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// (.aligned: a warp's lanes execute it together, also after a loop or a branch
-// that some of them left early)
-__device__ __forceinline__ void cluster_arrive()
-{
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait()
-{
-    __syncwarp();
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t dsmem_addr(const void *p, uint32_t rank)
-{
-    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void dsmem_st(uint32_t a, uint32_t v)
-{
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ uint32_t dsmem_ld(uint32_t a)
-{
-    uint32_t v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
-    return v;
-}
 
 // A mask's cells as bits of consecutive words, F[i / 32]: a warp's lanes read 32
 // adjacent cells, whatever the grid's shape, eight words at a time.
@@ -372,7 +337,7 @@ struct Energies {
             r = r + __shfl_xor_sync(0xffffffffu, r, 1);
             const uint32_t j = j0 + (q + (h16 ? 1 : 0) + (h8 ? 2 : 0)) * SEL_WARPS + warp;
             if ((lane & 7) == 0 && j < hi) {
-                if (remote) dsmem_st(key0 + 4 * j, __float_as_uint(r));
+                if (remote) dsmem_st_u32(key0 + 4 * j, __float_as_uint(r));
                 else keys[j] = __float_as_uint(r);
             }
         }
@@ -416,7 +381,7 @@ __device__ __forceinline__ void energies(const T *zg, const uint16_t *list, uint
         for (int q = 0; q < UN; ++q) {
             const uint32_t j = j0 + (q * SEL_WARPS + warp) * rpw + sub;
             if (j < hi && l == 0) {
-                if (remote) dsmem_st(key0 + 4 * j, __float_as_uint(s[q]));
+                if (remote) dsmem_st_u32(key0 + 4 * j, __float_as_uint(s[q]));
                 else keys[j] = __float_as_uint(s[q]);
             }
         }
@@ -638,7 +603,7 @@ k_select(const T *__restrict__ z, const uint8_t *__restrict__ masks, int m, int 
             cluster_wait();
             for (int w = threadIdx.x; w < words; w += SEL_THREADS) {
                 uint32_t o = P[w];
-                for (int q = 0; q < KC; ++q) o |= dsmem_ld(dsmem_addr(P + w, (uint32_t)q));
+                for (int q = 0; q < KC; ++q) o |= dsmem_ld_u32(dsmem_addr(P + w, (uint32_t)q));
                 A[w] = o;
             }
             cluster_arrive();
@@ -719,7 +684,7 @@ k_select(const T *__restrict__ z, const uint8_t *__restrict__ masks, int m, int 
             cluster_wait();
             if (rank != 0)
                 for (uint32_t i = threadIdx.x; i < (n_kept + 1) / 2; i += SEL_THREADS)
-                    keys[i] = dsmem_ld(dsmem_addr(keys + i, 0u));
+                    keys[i] = dsmem_ld_u32(dsmem_addr(keys + i, 0u));
             cluster_arrive();
         }
         __syncthreads();

@@ -6,6 +6,8 @@
 #include <cuda.h>
 #include <stdint.h>
 
+#include "rs3_readout_common.cuh"
+
 namespace tc {
 
 constexpr uint64_t DRAIN_LIMIT_NS = 1000000000ull;  // a drain of work in flight gives up after 1 s
@@ -391,13 +393,6 @@ __device__ __forceinline__ bool bar_and(uint32_t id, uint32_t nthreads, bool pre
 
 // Pieces of one row's softmax over N scores (raw fp32 bits).
 
-__device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi)
-{
-    uint32_t r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-    return r;
-}
-
 template <int N>
 __device__ __forceinline__ float row_max(const uint32_t (&sr)[N])
 {
@@ -439,7 +434,7 @@ __device__ __forceinline__ float row_exp(const uint32_t (&sr)[N], uint32_t *pk, 
 #pragma unroll
         for (int c = 0; c < 16; c += 2) {
             acc[c / 2 & 3] = add2(acc[c / 2 & 3], f2pack(x[c], x[c + 1]));
-            pk[(c0 + c) / 2] = cvt_bf16x2(x[c], x[c + 1]);
+            pk[(c0 + c) / 2] = pack_bf16x2(x[c], x[c + 1]);
         }
     }
     float a, b;
