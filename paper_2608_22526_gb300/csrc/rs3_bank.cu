@@ -1,7 +1,7 @@
 // rs3_bank.cu -- ragged per-unit memory bank and the write-pruned commit
 // (Sec. 3.2, Eq. 8; Algorithm 1's sparse write).
 //
-// A commit is one launch (k_commit): a CTA per (128-cell chunk, unit) ranks
+// A commit is one launch (k_commit): a CTA per (64- or 128-cell chunk, unit) ranks
 // its kept cells with ballot/popc and copies their K and V rows with 128-bit
 // accesses, the first rows' loads in flight while the unit's counts and the
 // capacity decision are made; the last CTA of each unit publishes the new
@@ -94,8 +94,8 @@ __device__ __forceinline__ int nonzero_bytes(uint4 w)
 // cells, once it has read what it needs of the old counters, and the last to
 // arrive publishes the new ones, so no CTA can read counters of the frame it
 // copies (the readers of the bank are later launches).
-// 48 units of 96 x 96 cells (130 MB, 19 us at the copy rate): 42.4 us with keys
-// rotated, 32.4 as given; 46.5 and 35 when every chunk counted its unit's mask,
+// 48 units of 96 x 96 cells (130 MB, 19 us at the copy rate): 41.4 us with keys
+// rotated, 31.2 as given; 46.5 and 35 when every chunk counted its unit's mask,
 // a batch was 32 rows of 4 warps, and the angles were loaded after the keys.
 
 // A batch of pieces in registers.
@@ -435,7 +435,7 @@ rs3_status commit_launch(const rs3_bank *bank, const void *k_new, const void *v_
     // Warps copying a chunk and rows in flight per warp (us per call, the others
     // measured for the same shapes).  Rotated keys: 3 CTAs of 8 warps x 4 rows;
     // 16 x 3 objects 41 (2 rows 39.4, but 26.6 against 22.4 on 12 objects); the 80
-    // registers of 3 CTAs spill 184 bytes per thread, 4 CTAs more (50.7).  Keys as
+    // registers of 3 CTAs spill 216 bytes per thread, 4 CTAs more (50.7).  Keys as
     // given: 2 CTAs of 8 warps x 8 rows for few CTAs, 8 objects of 64 x 64 7.2 and,
     // without a mask, 13.6 in 128-cell chunks, 14.4 in 64-cell ones (2 warps x 16 7.8
     // and 15.1, 8 x 4 7.1 and 14.8, rows of 4 KB 22 and 38); 4 x 8 for many CTAs.

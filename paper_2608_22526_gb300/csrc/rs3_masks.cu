@@ -33,11 +33,12 @@
 // the object listed first.  close_shape() picks rows and KC.
 //
 // Each logit is read from DRAM once; halo re-reads by neighbouring tiles hit
-// L2.  16 streams x 3 objects of 384 x 384 (31 MB, 4.6 us at the copy rate): 18.1
+// L2.  16 streams x 3 objects of 384 x 384 (31 MB, 4.6 us at the copy rate): 19.1
 // us per call, half of the issue slots busy, mostly with the thresholds, the
-// argmax and its labels; 91 us with a scalar load and a ballot per 32 pixels,
+// argmax and its labels (at two CTAs per SM three strips spill 120 bytes per
+// thread, four 40); 91 us with a scalar load and a ballot per 32 pixels,
 // general funnel-shift dilations and an 8-row halo per 16 rows on CTAs that
-// filled 1.3 waves.  8 objects of 1024 x 1024: 79 -> 44 us.
+// filled 1.3 waves.  8 objects of 1024 x 1024: 79 -> 29 us.
 #include "rs3_cluster.cuh"
 #include "rs3_internal.cuh"
 

@@ -31,7 +31,7 @@
 // CTA's matrix instructions in order).
 // The softmax warps take registers from the others (setmaxnreg): a row's 128
 // scores stay in registers.
-// 16 streams x 3 objects, 4 heads of 64, 96 x 96 grid (911 GFLOP): 1 070 us per
+// 16 streams x 3 objects, 4 heads of 64, 96 x 96 grid (911 GFLOP): 1 078 us per
 // call, 1 704 in the one-tile kernel.  Per pair of 128 x 128 tiles it takes about
 // 2 500 clk, where the exps of 256 rows alone take 1 380 and the matrices 1 052:
 // a warpgroup's own chain (wait, scores from TMEM, max, exps, P to TMEM) is that

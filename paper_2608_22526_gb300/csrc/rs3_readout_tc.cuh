@@ -27,7 +27,7 @@
 //               shared memory at a named barrier that also ANDs their wait
 //               results.  Epilogue: O / l + residual, or split-KV partials.
 // Both issuers are whole warps in uniform code that elect the issuing thread:
-// 8 objects on a 64 x 64 grid, d = 256 (57 GFLOP), 68 us per call, 76 with
+// 8 objects on a 64 x 64 grid, d = 256 (57 GFLOP), 65 us per call, 76 with
 // the issue behind a branch on the lane (16 S instructions then took 1 200 clk
 // to issue, 512 to run).
 // TMEM (512 columns): O in [0, d), S_0 / S_1 from S_COL, Q at Q_COL.

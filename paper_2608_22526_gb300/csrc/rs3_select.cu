@@ -24,10 +24,10 @@
 //      cluster writes some of the group's units.
 // Bound by latency and, in one CTA per SM, by instruction issue: 512 threads
 // and no divisions in the loops, where 1024 threads took 30 000 cycles.
-// One object of 64 x 64 cells and 256 channels takes 7.6 us in a graph, eight
-// 14.0 us, and 16 streams x 3 objects of 96 x 96 20.9 us per call (7.3 us at the
-// copy rate); 20.3, 25.9 and 59 us as three launches that passed the priors and
-// the energies through global memory.
+// One object of 64 x 64 cells and 256 channels takes 7.4 us in a graph of a whole
+// sequence's selections, eight 12.5 us, and 16 streams x 3 objects of 96 x 96 20.0 us
+// per call (7.3 us at the copy rate); 20.3, 25.9 and 59 us as three launches that
+// passed the priors and the energies through global memory.
 #include "rs3_cluster.cuh"
 #include "rs3_internal.cuh"
 
@@ -985,7 +985,7 @@ rs3_status select_launch(const void *z, rs3_dtype dtype, int G, int m, int n, in
     if (k < 0) return RS3_EINVAL;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     // CTAs per cluster: as many as are resident at once (two per SM), up to the
-    // portable 8; 48 units of 96 x 96 cells: 20.9 us with 6 each, 22.6 with 4
+    // portable 8; 48 units of 96 x 96 cells, both then: 20.9 us with 6 each, 22.6 with 4
     const long clusters = p->union_mode ? (G < U ? G : U) : U;
     const int n_sm = rs3_sm_count();
     const int KC = (int)std::min(8l, std::max(1l, 2l * n_sm / clusters));

@@ -162,7 +162,7 @@ def rs3_select_queries(z, dtype: str, G: int, m: int, n: int, C: int, prev_masks
 def rs3_select_queries_noalloc(z, dtype: str, G: int, m: int, n: int, C: int, prev_masks,
                                unit_group, U: int, track, params: Params, idx, count, status,
                                stream=None):
-    """rs3_select_queries with the library's built-in scratch (no workspace)."""
+    """rs3_select_queries without a workspace: always one launch."""
     rc = lib.rs3_select_queries_noalloc(_ptr(z), DTYPES[dtype], G, m, n, C, _ptr(prev_masks),
                                         _ptr(unit_group), U, _ptr(track), ctypes.byref(params),
                                         _ptr(idx), _ptr(count), _ptr(status), _stream(stream))
